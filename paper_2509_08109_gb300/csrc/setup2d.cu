@@ -37,50 +37,101 @@ struct Tensor2 {
     }
 };
 
-// Q1 element matrix of cell (ci,cj): K[a][b] = sum_q 1/4 grad(phi_a)^T G grad(phi_b),
-// G from the cell's coefficient (above), J = dx/dxi on the reference cell
-// (isoparametric map of the four nodal coordinates).  Corner a = ax + 2 ay
-// sits at node (ci+ax, cj+ay).  Returns false if det J <= 0.
+// Reference-cell derivatives of a bilinear field given at a cell's corners:
+// d/dxi is linear in eta and d/deta linear in xi, so each takes two values at
+// the Gauss points (10 FP64 operations, against 32 for a sum over the four
+// corners at every point).
+struct EdgeMap2 {
+    double u[2];   // d/dxi at eta_q
+    double v[2];   // d/deta at xi_q
+    __device__ __forceinline__ void set(const double x[4]) {
+        const double e0 = x[1] - x[0], e1 = x[3] - x[2], f0 = x[2] - x[0], f1 = x[3] - x[1];
+        const double de = e1 - e0, df = f1 - f0;
+        u[0] = e0 + kG0 * de;
+        u[1] = e0 + kG1 * de;
+        v[0] = f0 + kG0 * df;
+        v[1] = f0 + kG1 * df;
+    }
+};
+
+struct CellMap2 {
+    EdgeMap2 x, y;
+    __device__ __forceinline__ void load(const double* __restrict__ X, const double* __restrict__ Y, int n, int ci,
+                                         int cj) {
+        const long long id = (long long)cj * n + ci;
+        const double xa[4] = {X[id], X[id + 1], X[id + n], X[id + n + 1]};
+        const double ya[4] = {Y[id], Y[id + 1], Y[id + n], Y[id + n + 1]};
+        x.set(xa);
+        y.set(ya);
+    }
+};
+
+// Q1 element matrix of a cell: K_ab = sum_q 1/4 grad(phi_a)^T G grad(phi_b), G
+// from the cell's coefficient (above), J = dx/dxi (isoparametric map).  Corner
+// a = ax + 2 ay; the symmetric half a <= b in the order of sym4.  Sum
+// factorisation over the 2x2 Gauss points: the shape functions are products of
+// 1 - t, t per direction, so with s = -1, +1 for corner bit 0, 1
+//   K_ab = sx sx' M11[ay+by] + sy sy' M22[ax+bx] + sx sy' N[ay][bx] + sx' sy N[by][ax],
+// about 160 FP64 operations in all (the direct sum takes about 600).
+// Returns false if det J <= 0.
+__host__ __device__ constexpr int sym4(int a, int b) {   // a <= b
+    return a * 4 - a * (a - 1) / 2 + (b - a);
+}
+
+// Contractions of two Gauss-point values with (1-t)^2, t(1-t), t^2 as sum and
+// difference: (1-t)^2 and t^2 at the two points are 1/3 +- 1/(2 sqrt 3).  Where
+// the metric is constant the difference vanishes and the entries keep the
+// exact ratios 2 : 1 : 2, so an element's row sums, which every coarser level
+// amplifies, come out as exact zeros.
+constexpr double kThird = 1.0 / 3.0, kSixth = 1.0 / 6.0, kHalfGap = 0.5 * (kG1 - kG0);
+__device__ __forceinline__ void pair3(double s0, double s1, double out[3]) {
+    const double S = s0 + s1, D = s0 - s1, t = kThird * S;
+    out[0] = t + kHalfGap * D;
+    out[1] = kSixth * S;
+    out[2] = t - kHalfGap * D;
+}
+
 template <class C>
-__device__ bool element2d(const double* __restrict__ X, const double* __restrict__ Y, int n, int ci, int cj,
-                          const C& coef, double K[4][4]) {
-    double xa[4], ya[4];
+__device__ __forceinline__ bool element2d(const CellMap2& M, const C& coef, double K[10]) {
+    bool ok = true;
+    double s11[2], g11[2][2], s22[2], g22[2][2], g12[2][2];   // [q: xi][p: eta]
 #pragma unroll
-    for (int a = 0; a < 4; a++) {
-        long long id = (long long)(cj + (a >> 1)) * n + (ci + (a & 1));
-        xa[a] = X[id];
-        ya[a] = Y[id];
+    for (int p = 0; p < 2; p++)
+#pragma unroll
+        for (int q = 0; q < 2; q++) {
+            const double J11 = M.x.u[p], J12 = M.x.v[q], J21 = M.y.u[p], J22 = M.y.v[q];
+            const double det = J11 * J22 - J12 * J21;
+            if (!(det > 0.0)) ok = false;
+            coef.metric(J11, J12, J21, J22, det, g11[q][p], g12[q][p], g22[q][p]);
+        }
+#pragma unroll
+    for (int t = 0; t < 2; t++) {
+        s11[t] = g11[0][t] + g11[1][t];
+        s22[t] = g22[t][0] + g22[t][1];
+    }
+    double M11[3], M22[3];
+    pair3(s11[0], s11[1], M11);
+    pair3(s22[0], s22[1], M22);
+    double N[2][2];
+#pragma unroll
+    for (int b = 0; b < 2; b++) {
+        const double wa = b ? kG0 : kG1, wb = b ? kG1 : kG0;   // the xi factor of corner bit b at xi_0, xi_1
+        const double n0 = wa * g12[0][0] + wb * g12[1][0], n1 = wa * g12[0][1] + wb * g12[1][1];
+        N[0][b] = kG1 * n0 + kG0 * n1;
+        N[1][b] = kG0 * n0 + kG1 * n1;
     }
 #pragma unroll
     for (int a = 0; a < 4; a++)
 #pragma unroll
-        for (int b = 0; b < 4; b++) K[a][b] = 0.0;
-    bool ok = true;
-#pragma unroll
-    for (int q = 0; q < 4; q++) {
-        const double xi = (q & 1) ? kG1 : kG0, eta = (q & 2) ? kG1 : kG0;
-        const double dxi[4] = {-(1.0 - eta), 1.0 - eta, -eta, eta};
-        const double det_[4] = {-(1.0 - xi), -xi, 1.0 - xi, xi};
-        double J11 = 0, J12 = 0, J21 = 0, J22 = 0;
-#pragma unroll
-        for (int a = 0; a < 4; a++) {
-            J11 += xa[a] * dxi[a];
-            J12 += xa[a] * det_[a];
-            J21 += ya[a] * dxi[a];
-            J22 += ya[a] * det_[a];
+        for (int b = a; b < 4; b++) {
+            const int ax = a & 1, ay = a >> 1, bx = b & 1, by = b >> 1;
+            const double m1 = M11[ay + by], m2 = M22[ax + bx], c1 = N[ay][bx], c2 = N[by][ax];
+            double v = ax == bx ? m1 : -m1;
+            v = ay == by ? v + m2 : v - m2;
+            v = ax == by ? v + c1 : v - c1;
+            v = bx == ay ? v + c2 : v - c2;
+            K[sym4(a, b)] = v;
         }
-        const double det = J11 * J22 - J12 * J21;
-        if (!(det > 0.0)) ok = false;
-        double G11, G12, G22;
-        coef.metric(J11, J12, J21, J22, det, G11, G12, G22);
-#pragma unroll
-        for (int a = 0; a < 4; a++) {
-            const double ga = G11 * dxi[a] + G12 * det_[a];
-            const double gb = G12 * dxi[a] + G22 * det_[a];
-#pragma unroll
-            for (int b = 0; b < 4; b++) K[a][b] += ga * dxi[b] + gb * det_[b];
-        }
-    }
     return ok;
 }
 
@@ -93,83 +144,106 @@ __device__ __forceinline__ auto cell_coef2(const double* __restrict__ c, long lo
         return Scalar2{c[e]};
 }
 
-// Gather assembly (no atomics), tiled so that each cell's element matrix is
-// formed once per tile rather than once per node of the cell: a CTA of 256
-// threads owns kAsmTX x kAsmTY nodes, first forms the element matrices of
-// the (kAsmTX+1) x (kAsmTY+1) cells around them (one cell per thread) into
-// shared memory, then each node sums its four cells' entries in a fixed
-// order.  Couplings to boundary nodes are dropped; boundary rows are zero.
-constexpr int kAsmTX = 31, kAsmTY = 7;
-constexpr int kAsmCX = kAsmTX + 1, kAsmCells = (kAsmTX + 1) * (kAsmTY + 1);   // 256
-// the ten entries of a cell matrix the gather uses
-enum AsmEntry { E00, E11, E22, E33, E10, E12, E20, E30, E31, E32, NE2 };
+// Gather assembly (no atomics).  A CTA owns a strip of kAsmN node columns and
+// a band of H node rows and marches up one row of cells at a time: each of
+// its kAsmC threads forms one cell's matrix into shared memory, then the node
+// threads add the row's entries to the node row below it, which that
+// completes, and start the row above.  Couplings to boundary nodes are
+// dropped; boundary rows are zero.  FP64 arithmetic bounds the kernel (two
+// FMA per SM and clock), so the redundant cells count (one column in kAsmC,
+// one row per band) and the 64 bytes per node do not.  Narrow strips keep
+// the bands tall enough on small grids to give every SM work.
+constexpr int kAsmC = 64, kAsmN = kAsmC - 1;
 
 template <bool TENSOR>
-__global__ void __launch_bounds__(kAsmCells) k_assemble2d(int n, int ld, long long pl,
-                                                          const double* __restrict__ coords,
-                                                          const double* __restrict__ kappa, double* __restrict__ A,
-                                                          KState* st) {
-    __shared__ double sK[NE2][kAsmCells];
+__global__ void __launch_bounds__(kAsmC) k_assemble2d(int n, int ld, long long pl, int H,
+                                                      const double* __restrict__ coords,
+                                                      const double* __restrict__ kappa, double* __restrict__ A,
+                                                      KState* st) {
+    __shared__ double sK[10][kAsmC];
     const long long ne = (long long)(n - 1) * (n - 1);
-    const int i0 = blockIdx.x * kAsmTX, j0 = blockIdx.y * kAsmTY;    // first node of the tile
     const int t = threadIdx.x;
-    {
-        // cell (ci, cj) lies between nodes ci, ci+1 and cj, cj+1
-        const int ci = i0 - 1 + t % kAsmCX, cj = j0 - 1 + t / kAsmCX;
-        if (ci >= 0 && cj >= 0 && ci <= n - 2 && cj <= n - 2) {
-            double K[4][4];
-            const double* X = coords;
-            const double* Y = coords + (long long)n * n;
-            if (!element2d(X, Y, n, ci, cj, cell_coef2<TENSOR>(kappa, ne, (long long)cj * (n - 1) + ci), K))
+    const int i0 = blockIdx.x * kAsmN;
+    const int j0 = blockIdx.y * H, j1 = min(j0 + H, n);             // node rows [j0, j1)
+    const int ci = i0 - 1 + t;                                      // cell column between nodes ci, ci + 1
+    const int i = i0 + t;                                           // node column; its cells are slots t, t + 1
+    const bool node = t < kAsmN && i < n;
+    const bool in1 = node && i >= 1 && i <= n - 2;
+    double C = 0, W = 0;                                            // of the row in progress
+    for (int cj = j0 - 1; cj < j1; cj++) {
+        if (cj >= 0 && cj <= n - 2 && ci >= 0 && ci <= n - 2) {
+            CellMap2 M;
+            M.load(coords, coords + (long long)n * n, n, ci, cj);
+            double K[10];
+            if (!element2d(M, cell_coef2<TENSOR>(kappa, ne, (long long)cj * (n - 1) + ci), K))
                 set_err(st, BMG_ERR_MAP_FOLDED);
-            sK[E00][t] = K[0][0];
-            sK[E11][t] = K[1][1];
-            sK[E22][t] = K[2][2];
-            sK[E33][t] = K[3][3];
-            sK[E10][t] = K[1][0];
-            sK[E12][t] = K[1][2];
-            sK[E20][t] = K[2][0];
-            sK[E30][t] = K[3][0];
-            sK[E31][t] = K[3][1];
-            sK[E32][t] = K[3][2];
+#pragma unroll
+            for (int q = 0; q < 10; q++) sK[q][t] = K[q];
         }
+        __syncthreads();
+        if (cj >= j0 && node) {   // row cj: the cells above it, (i-1, cj) and (i, cj)
+            const bool in = in1 && cj >= 1 && cj <= n - 2;
+            const long long o = (long long)cj * ld + i;
+            double NW = 0;
+            if (in) {
+                C += sK[sym4(1, 1)][t];
+                if (i >= 2) {
+                    W += sK[sym4(0, 1)][t];
+                    if (cj + 1 <= n - 2) NW = sK[sym4(1, 2)][t];
+                }
+                C += sK[sym4(0, 0)][t + 1];
+            }
+            A[C2 * pl + o] = in ? C : 0.0;
+            A[W2 * pl + o] = in ? W : 0.0;
+            A[NW2 * pl + o] = NW;
+        }
+        if (cj + 1 < j1 && node) {   // row cj + 1: the cells below it, (i-1, cj) and (i, cj)
+            const int j = cj + 1;
+            const bool in = in1 && j >= 1 && j <= n - 2;
+            const long long o = (long long)j * ld + i;
+            double S = 0, SW = 0;
+            C = W = 0;
+            if (in) {
+                C = sK[sym4(3, 3)][t];
+                if (i >= 2) W = sK[sym4(2, 3)][t];
+                if (j >= 2) {
+                    S = sK[sym4(1, 3)][t];
+                    if (i >= 2) SW = sK[sym4(0, 3)][t];
+                }
+                C += sK[sym4(2, 2)][t + 1];
+                if (j >= 2) S += sK[sym4(0, 2)][t + 1];
+            }
+            A[S2 * pl + o] = S;
+            A[SW2 * pl + o] = SW;
+        }
+        __syncthreads();
     }
-    __syncthreads();
-    if (t >= kAsmTX * kAsmTY) return;
-    const int i = i0 + t % kAsmTX, j = j0 + t / kAsmTX;
-    if (i >= n || j >= n) return;
-    const long long o = (long long)j * ld + i;
-    double C = 0, W = 0, S = 0, SW = 0, NW = 0;
-    if (i >= 1 && j >= 1 && i <= n - 2 && j <= n - 2) {
-        // shared-memory slot of the cell whose lower-left node is (ci, cj)
-        auto cell = [&](int ci, int cj) { return (ci - i0 + 1) + kAsmCX * (cj - j0 + 1); };
-        // cell (i-1,j-1): node is corner 3
-        int e = cell(i - 1, j - 1);
-        C += sK[E33][e];
-        if (i - 1 >= 1) W += sK[E32][e];
-        if (j - 1 >= 1) S += sK[E31][e];
-        if (i - 1 >= 1 && j - 1 >= 1) SW += sK[E30][e];
-        // cell (i,j-1): node is corner 2
-        e = cell(i, j - 1);
-        C += sK[E22][e];
-        if (j - 1 >= 1) S += sK[E20][e];
-        // cell (i-1,j): node is corner 1
-        e = cell(i - 1, j);
-        C += sK[E11][e];
-        if (i - 1 >= 1) W += sK[E10][e];
-        if (i - 1 >= 1 && j + 1 <= n - 2) NW += sK[E12][e];
-        // cell (i,j): node is corner 0
-        e = cell(i, j);
-        C += sK[E00][e];
-    }
-    A[C2 * pl + o] = C;
-    A[W2 * pl + o] = W;
-    A[S2 * pl + o] = S;
-    A[SW2 * pl + o] = SW;
-    A[NW2 * pl + o] = NW;
 }
 
-inline dim3 grid_asm(int n) { return dim3(cdiv(n, kAsmTX), cdiv(n, kAsmTY)); }
+// Launches k_assemble2d; rows per band: the ones that minimise (warps per
+// scheduler) x (rows + 1 pre-roll row).  One warp's FP64 instruction holds its
+// scheduler's unit for 64 cycles, so a row of cells costs each warp the same
+// few microseconds whether or not the other schedulers have work.
+template <bool TENSOR>
+bmg_status launch_assemble2d(int n, int ld, long long pl, const double* coords, const double* coef, double* A,
+                             KState* st, cudaStream_t s) {
+    int dev = 0, sms = 0;
+    BMG_CUDA(cudaGetDevice(&dev));
+    BMG_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+    const int tx = cdiv(n, kAsmN);
+    int H = 1;
+    long long best = -1;
+    for (int h = 1; h <= 64 && h <= n; h++) {
+        const long long cost = (long long)cdiv(tx * cdiv(n, h) * (kAsmC / 32), 4 * sms) * (h + 1);
+        if (best < 0 || cost < best) {
+            best = cost;
+            H = h;
+        }
+    }
+    k_assemble2d<TENSOR><<<dim3(tx, cdiv(n, H)), kAsmC, 0, s>>>(n, ld, pl, H, coords, coef, A, st);
+    BMG_CUDA(cudaGetLastError());
+    return BMG_OK;
+}
 
 // Full 9-entry rows -> symmetric half planes; couplings to boundary nodes
 // and boundary rows are forced to zero.
@@ -300,8 +374,27 @@ __device__ __forceinline__ double pweight2(const double* __restrict__ P, int ldc
     return P[p * plc + o];
 }
 
-// Galerkin coarse operator A_c = P^T A P, one thread per coarse node, five
-// stored entries: A_c(K, K+d) = sum_i P(i,K) sum_{j in N(i)} A(i,j) P(j,K+d).
+// Weight of the fine point at offset (gx, gy) in [-2, 2]^2 from the fine point
+// 2(I,J) to the coarse node (I+ex, J+ey); all offsets are compile-time constants
+// at the call, so this is one load at a fixed offset from oc = (I,J).
+__host__ __device__ constexpr int half_floor(int g) { return g >= 0 ? g / 2 : -((1 - g) / 2); }
+__host__ __device__ constexpr bool parent1(int g, int e) {
+    return e - half_floor(g) >= 0 && e - half_floor(g) <= (g & 1);
+}
+__device__ __forceinline__ double weight2(const double* __restrict__ P, int ldc, long long plc, long long oc, int gx,
+                                          int gy, int ex, int ey) {
+    const int qx = half_floor(gx), qy = half_floor(gy), dI = ex - qx, dJ = ey - qy;
+    if (!(gx & 1) && !(gy & 1)) return 1.0;
+    const int p = !(gy & 1) ? (dI ? PXR : PXL) : !(gx & 1) ? (dJ ? PYN : PYS) : dJ ? (dI ? PNE : PNW) : (dI ? PSE : PSW);
+    return P[(long long)p * plc + oc + qx + (long long)ldc * qy];
+}
+
+// Galerkin coarse operator A_c = P^T A P, one thread per coarse node: the five
+// stored entries A_c(K, K+e) = sum_f P(f,K) (A P)(f, K+e) over the fine points
+// f = 2K + d, d in {-1,0,1}^2.  The four f with both coordinates odd are left
+// out: their interpolation solves their own fine equation, so (A P)(f, .) is
+// zero there (to rounding).  The offsets are constants, so the loops unroll to
+// plain loads and about 120 FP64 operations a coarse node.
 __global__ void k_rap2d(Sten2<double> F, int nf, const double* __restrict__ P, int nc, int ldc,
                         long long plc, double* __restrict__ Ac, KState* st) {
     const int I = blockIdx.x * blockDim.x + threadIdx.x;
@@ -310,26 +403,30 @@ __global__ void k_rap2d(Sten2<double> F, int nf, const double* __restrict__ P, i
     const long long o = (long long)J * ldc + I;
     double out[NS2] = {0, 0, 0, 0, 0};
     if (I >= 1 && J >= 1 && I <= nc - 2 && J <= nc - 2) {
-        const int tdx[NS2] = {0, -1, 0, -1, -1};
-        const int tdy[NS2] = {0, 0, -1, -1, 1};
-#pragma unroll 1
-        for (int t = 0; t < NS2; t++) {
-            const int LI = I + tdx[t], LJ = J + tdy[t];
-            if (LI < 1 || LJ < 1 || LI > nc - 2 || LJ > nc - 2) continue;
-            double acc = 0.0;
-            for (int fj = 2 * J - 1; fj <= 2 * J + 1; fj++)
-                for (int fi = 2 * I - 1; fi <= 2 * I + 1; fi++) {
-                    const double wK = pweight2(P, ldc, plc, nf, fi, fj, I, J);
-                    if (wK == 0.0) continue;
-                    for (int dy = -1; dy <= 1; dy++)
-                        for (int dx = -1; dx <= 1; dx++) {
-                            const double a = F.full(fi, fj, dx, dy);
-                            if (a == 0.0) continue;
-                            const double wL = pweight2(P, ldc, plc, nf, fi + dx, fj + dy, LI, LJ);
-                            acc += wK * a * wL;
-                        }
+        constexpr int tdx[NS2] = {0, -1, 0, -1, -1};
+        constexpr int tdy[NS2] = {0, 0, -1, -1, 1};
+#pragma unroll
+        for (int f = 0; f < 9; f++) {
+            const int fx = f % 3 - 1, fy = f / 3 - 1;
+            if (fx != 0 && fy != 0) continue;
+            const double wK = weight2(P, ldc, plc, o, fx, fy, 0, 0);
+#pragma unroll
+            for (int e = 0; e < 9; e++) {
+                const int dx = e % 3 - 1, dy = e / 3 - 1;
+                const double a = wK * F.full(2 * I + fx, 2 * J + fy, dx, dy);
+#pragma unroll
+                for (int t = 0; t < NS2; t++) {
+                    const int ex = t == 0 || t == 2 ? 0 : -1, ey = t == 2 || t == 3 ? -1 : t == 4 ? 1 : 0;
+                    if (parent1(fx + dx, ex) && parent1(fy + dy, ey))
+                        out[t] += a * weight2(P, ldc, plc, o, fx + dx, fy + dy, ex, ey);
                 }
-            out[t] = acc;
+            }
+        }
+        // couplings to boundary coarse nodes are dropped
+#pragma unroll
+        for (int t = 1; t < NS2; t++) {
+            const int LI = I + tdx[t], LJ = J + tdy[t];
+            if (LI < 1 || LJ < 1 || LI > nc - 2 || LJ > nc - 2) out[t] = 0.0;
         }
         if (!(out[0] > 0.0)) set_err(st, BMG_ERR_SETUP_BREAKDOWN);
     }
@@ -370,16 +467,21 @@ __global__ void k_boundary_rhs2d(int n, const double* __restrict__ coords, const
         const double* X = coords;
         const double* Y = coords + (long long)n * n;
         bool ok = true;
+#pragma unroll
         for (int cy = 0; cy < 2; cy++)
+#pragma unroll
             for (int cx = 0; cx < 2; cx++) {
                 const int ci = i - 1 + cx, cj = j - 1 + cy;
                 const int a = (1 - cx) + 2 * (1 - cy);      // the node's corner in the cell
-                double K[4][4];
-                ok &= element2d(X, Y, n, ci, cj, Scalar2{kappa[(long long)cj * (n - 1) + ci]}, K);
+                CellMap2 M;
+                M.load(X, Y, n, ci, cj);
+                double K[10];
+                ok &= element2d(M, Scalar2{kappa[(long long)cj * (n - 1) + ci]}, K);
+#pragma unroll
                 for (int b = 0; b < 4; b++) {
                     const int bi = ci + (b & 1), bj = cj + (b >> 1);
                     if (bi >= 1 && bj >= 1 && bi <= n - 2 && bj <= n - 2) continue;
-                    acc -= K[a][b] * g[(long long)bj * n + bi];
+                    acc -= K[a < b ? sym4(a, b) : sym4(b, a)] * g[(long long)bj * n + bi];
                 }
             }
         if (!ok) set_err(st, BMG_ERR_MAP_FOLDED);
@@ -387,14 +489,15 @@ __global__ void k_boundary_rhs2d(int n, const double* __restrict__ coords, const
     out[(long long)j * n + i] = acc;
 }
 
-// dL/dkappa_e = -lambda_e^T K_e^0 u_e (u, lambda in the caller's n^2 layout).
+// dL/dkappa_e = -lambda_e^T K_e^0 u_e (u, lambda in the caller's n^2 layout) =
+// -sum_q 1/4 (adj^T grad lambda) . (adj^T grad u) / det: the two fields'
+// gradients at the Gauss points instead of the element matrix, about 130 FP64
+// operations a cell.
 __global__ void k_adjoint_cells2d(int n, const double* __restrict__ coords, const double* __restrict__ u,
                                   const double* __restrict__ lam, double* __restrict__ g, KState* st) {
     const int ci = blockIdx.x * blockDim.x + threadIdx.x;
     const int cj = blockIdx.y;
     if (ci >= n - 1) return;
-    double K[4][4];
-    if (!element2d(coords, coords + (long long)n * n, n, ci, cj, Scalar2{1.0}, K)) set_err(st, BMG_ERR_MAP_FOLDED);
     double ue[4], le[4];
 #pragma unroll
     for (int a = 0; a < 4; a++) {
@@ -404,14 +507,25 @@ __global__ void k_adjoint_cells2d(int n, const double* __restrict__ coords, cons
         ue[a] = in ? u[id] : 0.0;
         le[a] = in ? lam[id] : 0.0;
     }
+    CellMap2 M;
+    EdgeMap2 U, L;
+    M.load(coords, coords + (long long)n * n, n, ci, cj);
+    U.set(ue);
+    L.set(le);
+    bool ok = true;
     double s = 0.0;
 #pragma unroll
-    for (int a = 0; a < 4; a++) {
-        double t = 0.0;
+    for (int p = 0; p < 2; p++)
 #pragma unroll
-        for (int b = 0; b < 4; b++) t += K[a][b] * ue[b];
-        s += le[a] * t;
-    }
+        for (int q = 0; q < 2; q++) {
+            const double J11 = M.x.u[p], J12 = M.x.v[q], J21 = M.y.u[p], J22 = M.y.v[q];
+            const double det = J11 * J22 - J12 * J21;
+            if (!(det > 0.0)) ok = false;
+            const double ux = J22 * U.u[p] - J21 * U.v[q], uy = J11 * U.v[q] - J12 * U.u[p];
+            const double lx = J22 * L.u[p] - J21 * L.v[q], ly = J11 * L.v[q] - J12 * L.u[p];
+            s += (ux * lx + uy * ly) * (0.25 / det);
+        }
+    if (!ok) set_err(st, BMG_ERR_MAP_FOLDED);
     g[(long long)cj * (n - 1) + ci] = -s;
 }
 
@@ -421,9 +535,8 @@ inline dim3 grid_rows(int ni, int nj) { return dim3(cdiv(ni, 128), nj); }
 
 bmg_status assemble2d(Ctx& c, const double* coords, const double* kappa) {
     Level& L = c.lev[0];
-    k_assemble2d<false><<<grid_asm(L.n), kAsmCells, 0, c.stream>>>(L.n, L.ld, L.plane, coords, kappa, L.A64, c.st);
+    BMG_TRY(launch_assemble2d<false>(L.n, L.ld, L.plane, coords, kappa, L.A64, c.st, c.stream));
     c.launches++;
-    BMG_CUDA(cudaGetLastError());
     return BMG_OK;
 }
 
@@ -431,8 +544,7 @@ bmg_status assemble2d(Ctx& c, const double* coords, const double* kappa) {
 // storage: half planes A (row length ld, plane stride pl) and error word st.
 bmg_status assemble_export2d(int n, int ld, long long pl, const double* coords, const double* kappa, double* A,
                              KState* st, double* out, cudaStream_t s) {
-    k_assemble2d<false><<<grid_asm(n), kAsmCells, 0, s>>>(n, ld, pl, coords, kappa, A, st);
-    BMG_CUDA(cudaGetLastError());
+    BMG_TRY(launch_assemble2d<false>(n, ld, pl, coords, kappa, A, st, s));
     k_export_stencil2d<<<grid_rows(n, n), 128, 0, s>>>(Sten2<double>{A, ld, pl}, n, out);
     BMG_CUDA(cudaGetLastError());
     return BMG_OK;
@@ -440,9 +552,8 @@ bmg_status assemble_export2d(int n, int ld, long long pl, const double* coords, 
 
 bmg_status assemble_tensor2d(Ctx& c, const double* coords, const double* D) {
     Level& L = c.lev[0];
-    k_assemble2d<true><<<grid_asm(L.n), kAsmCells, 0, c.stream>>>(L.n, L.ld, L.plane, coords, D, L.A64, c.st);
+    BMG_TRY(launch_assemble2d<true>(L.n, L.ld, L.plane, coords, D, L.A64, c.st, c.stream));
     c.launches++;
-    BMG_CUDA(cudaGetLastError());
     return BMG_OK;
 }
 
