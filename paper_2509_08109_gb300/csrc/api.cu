@@ -44,7 +44,8 @@ size_t carve(Ctx& c, char* base) {
     const size_t vt = f32 ? sizeof(float) : sizeof(double);
     for (int l = 0; l < c.nlev; l++) {
         Level& L = c.lev[l];
-        L.A64 = (double*)take(sizeof(double) * c.ns * L.plane);
+        // an FP64 V-cycle keeps the reciprocal diagonal behind the operator
+        L.A64 = (double*)take(sizeof(double) * (c.ns + (f32 ? 0 : 1)) * L.plane);
         L.A32 = f32 ? (float*)take(sizeof(float) * c.ns * L.plane) : nullptr;
         if (l < c.nlev - 1) {
             const Level& K = c.lev[l + 1];
@@ -531,6 +532,7 @@ bmg_status bmg_setup(bmg_ctx* ctx) {
     BMG_TRY(reset_state(c));
     for (int l = 0; l < c.nlev - 1; l++) BMG_TRY(c.dim == 2 ? setup_level2d(c, l) : setup_level3d(c, l));
     BMG_TRY(demote_levels(c));
+    BMG_TRY(invert_diagonals(c));
     if (c.use_fused) BMG_TRY(tail_pack(c));
     if (c.rs32) BMG_TRY(k_row_sums32(c));
     BMG_TRY(pspmv_prepare(c));

@@ -391,6 +391,7 @@ bmg_status fused_prepare(Ctx& c);
 bmg_status fused_configure(Ctx& c, int l, int wc, int hc, int hc_up);
 bmg_status fused_autotune(Ctx& c, int reps, double* best_ms_total);
 bmg_status demote_levels(Ctx& c);
+bmg_status invert_diagonals(Ctx& c);   // FP64 contexts: 1 / diagonal into the plane behind every level's operator
 // krylov.cu
 bmg_status k_pack(Ctx& c, const double* src, double* dst);      // n^d -> padded, boundary zeroed
 bmg_status k_unpack(Ctx& c, const double* src, double* dst);    // padded -> n^d

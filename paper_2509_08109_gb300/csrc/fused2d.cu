@@ -137,10 +137,25 @@ struct AccN;
 // ------------------------------------------------------------------ layout
 __host__ __device__ constexpr int r128(int b) { return (b + 127) & ~127; }
 
+// Streamed stencil planes.  FP32: C, W, S, SW, NW, and an update divides by C
+// (one reciprocal and a product).  FP64: W, S, SW, NW and the diagonal's
+// reciprocal, the plane bmg_setup adds behind the operator: an FP64 division
+// costs about nine of the FMA slots that bound these kernels (a point's whole
+// update has eight products), a product costs one.  Measured on the 1025^2
+// FP64 solve: k_vdown2d 56.9 -> 37.8 us, k_vup2d 62.9 -> 45.3 us, the tail
+// 46.6 -> 32.9 us.
 template <typename T>
-__device__ __forceinline__ T divide(T s, T d) { return s / d; }
+struct Pl {
+    static constexpr int C = C2, W = W2, S = S2, SW = SW2, NW = NW2;
+};
 template <>
-__device__ __forceinline__ float divide<float>(float s, float d) { return __fdividef(s, d); }
+struct Pl<double> {
+    static constexpr int W = W2 - 1, S = S2 - 1, SW = SW2 - 1, NW = NW2 - 1, C = NS2 - 1;
+};
+
+// s over the diagonal d (FP64: d is its reciprocal)
+__device__ __forceinline__ double divide(double s, double d) { return s * d; }
+__device__ __forceinline__ float divide(float s, float d) { return __fdividef(s, d); }
 __device__ __forceinline__ float4 divide(float4 s, float d) {
     return make_float4(__fdividef(s.x, d), __fdividef(s.y, d), __fdividef(s.z, d), __fdividef(s.w, d));
 }
@@ -259,31 +274,32 @@ struct AccN<4> {
 // NW(j,c) couples (c-1, j+1), NW(j-1,c+1) (c+1, j-1).
 template <typename T, typename V, typename XA>
 struct Rows {
+    using Q = Pl<T>;
     const T *a, *an, *as;          // stencil rows j, j+1, j-1 (plane 0)
     XA x, xn, xs;                  // iterate rows j, j+1, j-1
     int PL;                        // plane stride
     __device__ __forceinline__ V offdiag(int c) const {
-        V s = a[W2 * PL + c] * x[c - 1];
-        s += a[W2 * PL + c + 1] * x[c + 1];
-        s += a[S2 * PL + c] * xs[c];
-        s += an[S2 * PL + c] * xn[c];
-        s += a[SW2 * PL + c] * xs[c - 1];
-        s += an[SW2 * PL + c + 1] * xn[c + 1];
-        s += a[NW2 * PL + c] * xn[c - 1];
-        s += as[NW2 * PL + c + 1] * xs[c + 1];
+        V s = a[Q::W * PL + c] * x[c - 1];
+        s += a[Q::W * PL + c + 1] * x[c + 1];
+        s += a[Q::S * PL + c] * xs[c];
+        s += an[Q::S * PL + c] * xn[c];
+        s += a[Q::SW * PL + c] * xs[c - 1];
+        s += an[Q::SW * PL + c + 1] * xn[c + 1];
+        s += a[Q::NW * PL + c] * xn[c - 1];
+        s += as[Q::NW * PL + c + 1] * xs[c + 1];
         return s;
     }
     // forward sweep, colour 2: the (c +- 1, j) neighbours are still zero
     __device__ __forceinline__ V offdiag_no_row(int c) const {
-        V s = a[S2 * PL + c] * xs[c];
-        s += an[S2 * PL + c] * xn[c];
-        s += a[SW2 * PL + c] * xs[c - 1];
-        s += an[SW2 * PL + c + 1] * xn[c + 1];
-        s += a[NW2 * PL + c] * xn[c - 1];
-        s += as[NW2 * PL + c + 1] * xs[c + 1];
+        V s = a[Q::S * PL + c] * xs[c];
+        s += an[Q::S * PL + c] * xn[c];
+        s += a[Q::SW * PL + c] * xs[c - 1];
+        s += an[Q::SW * PL + c + 1] * xn[c + 1];
+        s += a[Q::NW * PL + c] * xn[c - 1];
+        s += as[Q::NW * PL + c + 1] * xs[c + 1];
         return s;
     }
-    __device__ __forceinline__ T diag(int c) const { return a[C2 * PL + c]; }
+    __device__ __forceinline__ T diag(int c) const { return a[Q::C * PL + c]; }
 };
 
 // ------------------------------------------------------------------ down kernel
@@ -389,7 +405,7 @@ __global__ void __launch_bounds__((WC + 8) * K, sizeof(T) == 4 ? 3 : 1)
         const Rows<T, V, XA> r = rows(j);
         V v = z0;
         if (vo && inrow(j)) {
-            const V s = vcast<V>(rg.F(j)[co]) - r.a[W2 * PL + co] * r.x[co - 1] - r.a[W2 * PL + co + 1] * r.x[co + 1];
+            const V s = vcast<V>(rg.F(j)[co]) - r.a[Pl<T>::W * PL + co] * r.x[co - 1] - r.a[Pl<T>::W * PL + co + 1] * r.x[co + 1];
             v = divide(s, r.diag(co));
         }
         X(j)[co] = v;
@@ -418,7 +434,7 @@ __global__ void __launch_bounds__((WC + 8) * K, sizeof(T) == 4 ? 3 : 1)
             Rj[ce] = (ve && rj) ? -r.offdiag(ce) : z0;
             Rj[co] = (vo && rj) ? -r.offdiag_no_row(co) : z0;
         } else {
-            Rj[ce] = (ve && rj) ? -(r.a[W2 * PL + ce] * r.x[ce - 1] + r.a[W2 * PL + ce + 1] * r.x[ce + 1]) : z0;
+            Rj[ce] = (ve && rj) ? -(r.a[Pl<T>::W * PL + ce] * r.x[ce - 1] + r.a[Pl<T>::W * PL + ce + 1] * r.x[ce + 1]) : z0;
             Rj[co] = z0;
         }
     };

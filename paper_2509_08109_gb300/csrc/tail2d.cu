@@ -31,13 +31,10 @@ namespace {
 constexpr int kTailThreads = 256;      // one thread per node of a colour at n = 33
 constexpr unsigned kTailChunk = 16384;    // bytes per bulk copy
 
-template <typename T>
-__device__ __forceinline__ T tdiv(T s, T d) { return s / d; }
-template <>
-__device__ __forceinline__ float tdiv<float>(float s, float d) { return __fdividef(s, d); }
-
 // Packed image, per level l: A (5 planes of n_l^2, compact rows of length
-// n_l), then P (8 planes of n_{l+1}^2) unless l is the last level.  The
+// n_l; the C plane holds the diagonal's reciprocal, so an update is a product
+// in the chain of dependent phases instead of a division), then P (8 planes
+// of n_{l+1}^2) unless l is the last level.  The
 // vectors (b, x, r per level) follow the image in shared memory.
 __host__ __device__ inline long long tail_pack_elems(const int* n, int nlev) {
     long long e = 0;
@@ -60,15 +57,18 @@ __host__ __device__ inline unsigned tail_pack_bytes_of(const int* n, int nlev) {
 }
 
 // Copies plane-strided planes (row length ld, plane stride pl) of an m x m
-// grid into compact planes (row length m).
+// grid into compact planes (row length m); plane inv (none if negative) as
+// reciprocals.
 template <typename T>
-__global__ void k_tail_pack(const T* __restrict__ src, int planes, int m, int ld, long long pl, T* __restrict__ dst) {
+__global__ void k_tail_pack(const T* __restrict__ src, int planes, int m, int ld, long long pl, int inv,
+                            T* __restrict__ dst) {
     const int total = planes * m * m;
     for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < total; k += gridDim.x * blockDim.x) {
         const int p = k / (m * m);
         const int r = k - p * m * m;
         const int j = r / m, i = r - j * m;
-        dst[k] = src[p * pl + (long long)j * ld + i];
+        const T v = src[p * pl + (long long)j * ld + i];
+        dst[k] = p == inv && v != (T)0 ? (T)1 / v : v;
     }
 }
 
@@ -171,7 +171,7 @@ __global__ void __launch_bounds__(kTailThreads) k_vtail2d(TailArgs a0, const Tai
             const int jj = k / ni, ii = k - jj * ni;
             const int i = i0 + 2 * ii, j = j0 + 2 * jj;
             const int o = j * m + i;
-            x[o * NR + rh] = tdiv<T>(f[o * NR + rh] - offdiag(A, m, m2, x, i, j, rh), A[C2 * m2 + o]);
+            x[o * NR + rh] = (f[o * NR + rh] - offdiag(A, m, m2, x, i, j, rh)) * A[C2 * m2 + o];
         }
     };
 
@@ -196,12 +196,12 @@ __global__ void __launch_bounds__(kTailThreads) k_vtail2d(TailArgs a0, const Tai
             const int k = kk / NR, rh = kk - k * NR;
             const int J = 1 + k / nb, I = k - (J - 1) * nb;
             const int o = 2 * J * m + 2 * I + 1;
-            const T xl = I >= 1 ? tdiv<T>(f[(o - 1) * NR + rh], A[C2 * m2 + o - 1]) : (T)0;
-            const T xr = I + 1 < nb ? tdiv<T>(f[(o + 1) * NR + rh], A[C2 * m2 + o + 1]) : (T)0;
+            const T xl = I >= 1 ? (f[(o - 1) * NR + rh]) * A[C2 * m2 + o - 1] : (T)0;
+            const T xr = I + 1 < nb ? (f[(o + 1) * NR + rh]) * A[C2 * m2 + o + 1] : (T)0;
             T sum = A[W2 * m2 + o] * xl;
             sum += A[W2 * m2 + o + 1] * xr;
             if (I >= 1) x[(o - 1) * NR + rh] = xl;
-            x[o * NR + rh] = tdiv<T>(f[o * NR + rh] - sum, A[C2 * m2 + o]);
+            x[o * NR + rh] = (f[o * NR + rh] - sum) * A[C2 * m2 + o];
         }
         __syncthreads();
         // colours 2 and 3, one thread per colour-3 point: the colour-2 row
@@ -217,7 +217,7 @@ __global__ void __launch_bounds__(kTailThreads) k_vtail2d(TailArgs a0, const Tai
             sum += A[SW2 * m2 + o + m + 1] * X(o + m + 1);
             sum += A[NW2 * m2 + o] * X(o + m - 1);
             sum += A[NW2 * m2 + o - m + 1] * X(o - m + 1);
-            return tdiv<T>(f[o * NR + rh] - sum, A[C2 * m2 + o]);
+            return (f[o * NR + rh] - sum) * A[C2 * m2 + o];
         };
         for (int kk = tid; kk < nb * nb * NR; kk += nth) {
             const int k = kk / NR, rh = kk - k * NR;
@@ -235,7 +235,7 @@ __global__ void __launch_bounds__(kTailThreads) k_vtail2d(TailArgs a0, const Tai
             sum += A[NW2 * m2 + o] * X(o + m - 1);
             sum += A[NW2 * m2 + o - m + 1] * X(o - m + 1);
             if (I >= 1) x[(o - 1) * NR + rh] = xl;
-            x[o * NR + rh] = tdiv<T>(f[o * NR + rh] - sum, A[C2 * m2 + o]);
+            x[o * NR + rh] = (f[o * NR + rh] - sum) * A[C2 * m2 + o];
         }
         __syncthreads();
         // residual and restriction, one thread per interior coarse node.
@@ -322,7 +322,7 @@ __global__ void __launch_bounds__(kTailThreads) k_vtail2d(TailArgs a0, const Tai
             if (I >= 1 && J >= 1) x[(o - m - 1) * NR + rh] = sw;
             if (J >= 1) x[(o - m) * NR + rh] = so;
             if (I >= 1) x[(o - 1) * NR + rh] = w;
-            x[o * NR + rh] = tdiv<T>(f[o * NR + rh] - sum, A[C2 * m2 + o]);
+            x[o * NR + rh] = (f[o * NR + rh] - sum) * A[C2 * m2 + o];
         }
         __syncthreads();
         for (int c = 2; c >= 0; c--) {
@@ -386,13 +386,13 @@ bmg_status tail_pack_impl(Ctx& c) {
     for (int l = 0; l < L; l++) {
         const Level& Lv = c.lev[t + l];
         const T* A = std::is_same<T, float>::value ? (const T*)Lv.A32 : (const T*)Lv.A64;
-        k_tail_pack<T><<<cdiv(NS2 * Lv.n * Lv.n, 256), 256, 0, c.stream>>>(A, NS2, Lv.n, Lv.ld, Lv.plane, q);
+        k_tail_pack<T><<<cdiv(NS2 * Lv.n * Lv.n, 256), 256, 0, c.stream>>>(A, NS2, Lv.n, Lv.ld, Lv.plane, C2, q);
         c.launches++;
         q += (long long)NS2 * Lv.n * Lv.n;
         if (l + 1 < L) {
             const Level& K = c.lev[t + l + 1];
             const T* P = std::is_same<T, float>::value ? (const T*)Lv.P32 : (const T*)Lv.P64;
-            k_tail_pack<T><<<cdiv(NP2 * K.n * K.n, 256), 256, 0, c.stream>>>(P, NP2, K.n, K.ld, K.plane, q);
+            k_tail_pack<T><<<cdiv(NP2 * K.n * K.n, 256), 256, 0, c.stream>>>(P, NP2, K.n, K.ld, K.plane, -1, q);
             c.launches++;
             q += (long long)NP2 * K.n * K.n;
         }

@@ -96,7 +96,8 @@ bmg_status fused_configure(Ctx& c, int l, int wc, int hc, int hc_up) {
     F.hc_up = hc_up;
     F.tiles_y_up = cdiv(m, hc_up);
     const int WW = 2 * F.wc + 16, WWc = F.wc + 8;
-    const void* A = f32 ? (const void*)Lf.A32 : (const void*)Lf.A64;
+    // FP64 streams W, S, SW, NW and the reciprocal diagonal, the plane behind them
+    const void* A = f32 ? (const void*)Lf.A32 : (const void*)(Lf.A64 + Lf.plane);
     const void* P = f32 ? (const void*)Lf.P32 : (const void*)Lf.P64;
     const void* f = l == 0 ? (const void*)c.r : Lf.b;
     const bool f_is64 = l == 0 || !f32;

@@ -115,6 +115,21 @@ __global__ void k_convert(long long count, const S* __restrict__ src, D* __restr
         dst[k] = (D)src[k];
 }
 
+// Reciprocal diagonals of every level (blockIdx.y) in one launch; the zero
+// diagonal of boundary and padding nodes gives zero.
+struct DiagLevels {
+    const double* diag[kMaxLevels];
+    double* inv[kMaxLevels];
+    long long count[kMaxLevels];
+};
+__global__ void k_invert_diagonals(DiagLevels a) {
+    const double* __restrict__ d = a.diag[blockIdx.y];
+    double* __restrict__ r = a.inv[blockIdx.y];
+    for (long long k = blockIdx.x * (long long)blockDim.x + threadIdx.x; k < a.count[blockIdx.y];
+         k += (long long)gridDim.x * blockDim.x)
+        r[k] = d[k] != 0.0 ? 1.0 / d[k] : 0.0;
+}
+
 inline dim3 rows(int ni, int nj) { return dim3(cdiv(ni, 128), nj); }
 
 template <typename T>
@@ -237,6 +252,22 @@ bmg_status demote_levels(Ctx& c) {
     }
     BMG_CUDA(cudaGetLastError());
     if (c.dim == 3) BMG_TRY(colour_blocks3d(c));
+    return BMG_OK;
+}
+
+bmg_status invert_diagonals(Ctx& c) {
+    if (c.opts.precision != BMG_PREC_FP64) return BMG_OK;
+    DiagLevels a{};
+    for (int l = 0; l < c.nlev; l++) {
+        const Level& L = c.lev[l];
+        a.diag[l] = L.A64 + (c.dim == 2 ? (long long)C2 : 13LL) * L.plane;
+        a.inv[l] = L.A64 + (long long)c.ns * L.plane;
+        a.count[l] = L.plane;
+    }
+    k_invert_diagonals<<<dim3(cdiv(c.lev[0].plane, 4 * 256) < 1216 ? cdiv(c.lev[0].plane, 4 * 256) : 1216, c.nlev), 256, 0,
+                         c.stream>>>(a);
+    c.launches++;
+    BMG_CUDA(cudaGetLastError());
     return BMG_OK;
 }
 
