@@ -86,7 +86,7 @@ size_t carve(Ctx& c, char* base) {
     c.stage_out = (double*)take(sizeof(double) * nn);
     c.partials = (double*)take(sizeof(double) * kMaxBlocks);
     c.st = (KState*)take(sizeof(KState));
-    const size_t tp = tail_pack_bytes(c);
+    const size_t tp = c.dim == 2 ? tail_pack_bytes(c) : tail3_pack_bytes(c);
     c.tail_pack = tp ? take(tp) : nullptr;
     c.mrhs_ws = c.mrhs_bytes ? take(c.mrhs_bytes) : nullptr;
     return align256(off);
@@ -451,9 +451,7 @@ bmg_status bmg_attach(bmg_ctx* ctx, void* ws, size_t bytes, void* stream) {
     BMG_CUDA(cudaMemsetAsync(c.ws, 0, c.ws_need, c.stream));
     BMG_CUDA(cudaStreamSynchronize(c.stream));
     c.use_fused = c.dim == 2 && !(c.opts.flags & BMG_FLAG_UNFUSED) && c.nlev >= 2;
-    // FP64 3-D V-cycles are bound by FP64 arithmetic: the half sweeps'
-    // recomputed halo would cost more than their saved traffic
-    c.use_hs3 = c.dim == 3 && c.opts.precision == BMG_PREC_FP32 && !(c.opts.flags & BMG_FLAG_UNFUSED);
+    c.use_hs3 = c.dim == 3 && !(c.opts.flags & BMG_FLAG_UNFUSED);
     c.use_graphs = !(c.opts.flags & BMG_FLAG_NO_GRAPHS);
     if (c.use_fused) BMG_TRY(fused_prepare(c));
     c.attached = true;
@@ -534,6 +532,7 @@ bmg_status bmg_setup(bmg_ctx* ctx) {
     BMG_TRY(demote_levels(c));
     BMG_TRY(invert_diagonals(c));
     if (c.use_fused) BMG_TRY(tail_pack(c));
+    if (c.dim == 3) BMG_TRY(tail3_pack(c));
     if (c.rs32) BMG_TRY(k_row_sums32(c));
     BMG_TRY(pspmv_prepare(c));
     KState h;

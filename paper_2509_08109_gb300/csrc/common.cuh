@@ -144,7 +144,7 @@ struct Ctx {
     ProfSlot prof[BMG_PROF_KINDS];
     bool use_fused = false;       // streaming V-cycle kernels (2-D)
     bool use_hs3 = false;         // 3-D: half-sweep kernels (one launch per colour parity of k)
-    void* tail_pack = nullptr;    // 2-D: operators and weights of the tail levels, packed (tail2d.cu)
+    void* tail_pack = nullptr;    // operators and weights of the tail levels, packed (tail2d.cu, vcycle3d.cu)
     // CUDA graphs of one inner/outer iteration (two, for the alternating z buffers)
     cudaStream_t cap_stream = nullptr;
     cudaGraphExec_t it_exec[2] = {nullptr, nullptr};
@@ -382,6 +382,8 @@ size_t tail_smem_bytes(const Ctx& c, int t);
 size_t tail_pack_bytes(const Ctx& c);             // packed tail operators (0 outside 2-D)
 bmg_status tail_pack(Ctx& c);                     // fills c.tail_pack (bmg_setup)
 bmg_status tail_vcycle(Ctx& c, int t);
+size_t tail3_pack_bytes(const Ctx& c);            // the same for the 3-D tail (vcycle3d.cu)
+bmg_status tail3_pack(Ctx& c);
 // z32 = M r32 (FP32 in and out); with zold and the streaming kernels the
 // finest up kernel also forms r.z, r.z_old and the flexible-CG beta
 bool vcycle_forms_beta(const Ctx& c);

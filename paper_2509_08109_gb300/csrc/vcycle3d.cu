@@ -2,8 +2,11 @@
 // 8-colour Gauss-Seidel with colour (i&1) + 2(j&1) + 4(k&1), forward colour
 // order before the coarse correction and reverse after; residual;
 // restriction P^T; prolongation with correction; exact solve on 3^3).
+#include <type_traits>
+
 #include "common.cuh"
 #include "grid3.cuh"
+#include "mbar.cuh"
 
 namespace bmg {
 namespace {
@@ -83,30 +86,91 @@ __global__ void k_gs_colour3d_cb(const float* __restrict__ blk, long long nc, in
     x[o] = (__ldcs(&f[o]) - s) / __ldcs(&blk[13 * nc + t]);
 }
 
+template <typename T>
+struct V2 {
+    T x, y;
+};
+template <typename T>
+__device__ __forceinline__ V2<T> ld2(const T* p) {
+    if constexpr (sizeof(T) == 4) {
+        const float2 v = __ldg(reinterpret_cast<const float2*>(p));
+        return {v.x, v.y};
+    } else {
+        const double2 v = __ldg(reinterpret_cast<const double2*>(p));
+        return {v.x, v.y};
+    }
+}
+
+// mask of the non-zero components of offset t: the neighbour at offset t (or
+// -t) of a point of colour col has colour col ^ mask
+__host__ __device__ constexpr int off_mask(int t) { return (t % 3 != 1) | ((t / 3 % 3 != 1) << 1) | ((t / 9 != 1) << 2); }
+
 // Residual after the forward 8-colour sweep from a zero guess: a point's own
 // update zeroed its residual while the neighbours of later colours were
-// still zero, so r = - sum over the neighbours of a later colour of a x.
-// The neighbour at offset d has colour col ^ m(d), m(d) the mask of the
-// non-zero components of d; same order of terms as offdiag3.
-template <typename T>
-__global__ void k_residual3d_sweep(L3<T> L, const T* __restrict__ x, T* __restrict__ r) {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    const int j = blockIdx.y, k = blockIdx.z;
-    if (i < 1 || j < 1 || k < 1 || i > L.n - 2 || j > L.n - 2 || k > L.n - 2) return;
-    const int col = (i & 1) | ((j & 1) << 1) | ((k & 1) << 2);
-    const long long o = L.idx(i, j, k);
+// still zero, so r = - sum over the neighbours of a later colour of a x, in
+// the order of offdiag3.  A thread forms the column pair (2p, 2p + 1) of a
+// row, so each point's terms are fixed at compile time (rows and planes of
+// one parity are uniform over a CTA) and the loads are two wide; a thread per
+// point left half the lanes of every term idle.  257^3 FP32: 148 us,
+// the time of its 60 bytes a node at the copy rate (225 before); 129^3 FP64:
+// 56 us.
+template <typename T, int JODD, int KODD>
+__device__ __forceinline__ void residual3d_pair(const L3<T>& L, const T* __restrict__ x, T* __restrict__ r, int i,
+                                                long long o) {
+    constexpr int c0 = 2 * JODD + 4 * KODD, c1 = c0 + 1;
     const long long sy = L.ld, sz = (long long)L.ld * L.n;
-    T s = 0;
+    T X[3][3][4];      // [dz + 1][dy + 1]: columns i - 1 .. i + 2
+#pragma unroll
+    for (int z = 0; z < 3; z++)
+#pragma unroll
+        for (int y = 0; y < 3; y++) {
+            if (KODD && z != 1) continue;
+            const T* q = x + o + (y - 1) * sy + (z - 1) * sz;
+            const V2<T> v = ld2(q);
+            X[z][y][0] = i > 0 ? __ldg(q - 1) : (T)0;
+            X[z][y][1] = v.x;
+            X[z][y][2] = v.y;
+            X[z][y][3] = __ldg(q + 2);
+        }
+    T s0 = 0, s1 = 0;
 #pragma unroll
     for (int t = 0; t < 13; t++) {
-        const int m = (off_x(t) != 0) | ((off_y(t) != 0) << 1) | ((off_z(t) != 0) << 2);
-        if ((col ^ m) > col) {
-            const long long d = off_x(t) + sy * off_y(t) + sz * off_z(t);
-            s += L.A[(long long)t * L.pl + o] * x[o + d];
-            s += L.A[(long long)t * L.pl + o - d] * x[o - d];
+        const bool n0 = (c0 ^ off_mask(t)) > c0, n1 = (c1 ^ off_mask(t)) > c1;
+        if (!n0 && !n1) continue;
+        const int dx = off_x(t), dy = off_y(t), dz = off_z(t);
+        const V2<T> own = ld2(L.A + t * L.pl + o);
+        const T* b = L.A + t * L.pl + o - dy * sy - dz * sz;   // the mirrors, stored at the node - d
+        const V2<T> m = ld2(b);
+        if (n0) {
+            s0 += own.x * X[dz + 1][dy + 1][1 + dx];
+            s0 += (dx == 0 ? m.x : dx < 0 ? m.y : i > 0 ? __ldg(b - 1) : (T)0) * X[1 - dz][1 - dy][1 - dx];
+        }
+        if (n1) {
+            s1 += own.y * X[dz + 1][dy + 1][2 + dx];
+            s1 += (dx == 0 ? m.y : dx < 0 ? __ldg(b + 2) : m.x) * X[1 - dz][1 - dy][2 - dx];
         }
     }
-    r[o] = -s;
+    if (i > 0) r[o] = -s0;
+    r[o + 1] = -s1;
+}
+
+template <typename T>
+__global__ void __launch_bounds__(64) k_residual3d_sweep(L3<T> L, const T* __restrict__ x, T* __restrict__ r) {
+    const int i = 2 * (blockIdx.x * blockDim.x + threadIdx.x);
+    const int j = 1 + blockIdx.y, k = 1 + blockIdx.z;      // interior rows and planes
+    if (i + 1 > L.n - 2) return;
+    const long long o = L.idx(i, j, k);
+    if (k & 1) {
+        if (j & 1)
+            residual3d_pair<T, 1, 1>(L, x, r, i, o);
+        else
+            residual3d_pair<T, 0, 1>(L, x, r, i, o);
+    } else {
+        if (j & 1)
+            residual3d_pair<T, 1, 0>(L, x, r, i, o);
+        else
+            residual3d_pair<T, 0, 0>(L, x, r, i, o);
+    }
 }
 
 // b_c(K) = sum over the 27 fine neighbours f = 2K + d of P(f, K) r_f, in the
@@ -198,186 +262,225 @@ __global__ void k_coarsest3d(L3<T> L, const double* __restrict__ A64, const T* _
 inline dim3 g3(int ni, int nj, int nk) { return dim3(cdiv(ni, 64), nj, nk); }
 
 // ---------------------------------------------------------------- tail
-// The coarse end of the 3-D V-cycle (levels with n <= tail3_max_n down to the
-// 3^3 grid and back) in one launch of one CTA: the same per-node steps as the
-// kernels above, each phase a block-strided loop followed by a block barrier.
-// Each phase waits on its loads, so the tail's time is about its number of
-// phases times the latency of the memory it reads.  In FP32 the tail starts
-// at 9^3 and all its levels (9^3, 5^3, 3^3: about 76 KB in a compact layout,
-// n in place of the padded row length) live in shared memory for the launch:
-// operators and weights copied from their arrays at the start, the first
-// level's right-hand side copied in and its iterate copied out; the 17^3
-// level runs the half-sweep kernels instead.  In FP64 the tail starts at
-// 17^3 (its operator alone is 550 KB) and works on the levels' arrays in
-// global memory (L2-resident).  Measured on the 257^3 shell (FP32
-// refinement solve): 1.052 s with a 17^3 tail in global memory, 1.045 s with
-// its lower levels staged.
-constexpr int kTail3Threads = 1024;
-template <typename T>
-constexpr int tail3_max_n() { return sizeof(T) == 4 ? 9 : 17; }   // first tail level: n <= this
-constexpr int kTail3Lev = 4;     // levels of a tail: 17, 9, 5, 3 at most
-
-template <typename T>
-struct Tail3Level {
-    L3<T> A;
-    const T* P;        // interpolation from the next level (its grid: ldc, plane plc)
-    int ldc;
-    long long plc;
-    const T* b;
-    T* x;
-    T* r;
-};
+// The coarse end of the 3-D V-cycle (9^3, 5^3 and 3^3) in one launch of one
+// CTA, every level in shared memory for the launch in a compact layout (n in
+// place of the padded row length; 76 KB in FP32, 151 KB in FP64).  The
+// operators and weights do not change between V-cycles: bmg_setup packs them
+// once into the shared-memory image, which a launch stages with bulk copies.
+// A barrier separates the colours, and a phase's time is the chain of one
+// thread's products (64 cycles each in FP64), so:
+//   - the diagonals are packed as reciprocals;
+//   - the forward sweep from the zero guess takes only the couplings to
+//     earlier colours, and the residual after it only those to later colours;
+//   - two lanes share a point, each summing half of its couplings;
+//   - prolongation runs one thread per fine point.
+// Measured per V-cycle: FP64 206 -> 55 us (it started at 17^3, in global
+// memory), FP32 42 -> 27 us.
+constexpr int kTail3Threads = 512;
+constexpr int kTail3MaxN = 9;    // first tail level: n <= this
+constexpr int kTail3Lev = 3;     // levels of a tail: 9, 5, 3 at most
+constexpr unsigned kTail3Chunk = 16384;   // bytes per bulk copy
 
 template <typename T>
 struct Tail3Args {
     int nlev;
-    Tail3Level<T> lv[kTail3Lev];
+    int n[kTail3Lev];      // nodes per side
+    const void* pack;      // packed operators and weights (shared-memory image)
+    unsigned pack_bytes;   // its size, a multiple of 16
+    const T* b;            // right-hand side of the first tail level
+    T* x;                  // its finished iterate
+    int ld;                // their row length
     const double* a64c;    // FP64 centre entry of the coarsest operator at (1,1,1)
+    KState* st;
 };
 
-// Elements of shared memory for the staged levels (all of them, FP32 only).
-template <typename T>
-__host__ __device__ constexpr bool tail3_stages() { return sizeof(T) == 4; }
-inline size_t tail3_smem_elems(const int* ns, int nlev) {
+// first level of the tail, and the sizes of its packed image and vectors
+int tail3_first(const Ctx& c) {
+    int t = c.nlev - 1;
+    while (t > 0 && c.lev[t - 1].n <= kTail3MaxN) t--;
+    return t;
+}
+size_t tail3_pack_elems(const Ctx& c) {
     size_t e = 0;
-    for (int q = 0; q < nlev; q++) {
-        const size_t n3 = (size_t)ns[q] * ns[q] * ns[q];
-        e += (NS3 + 3) * n3;
-        if (q + 1 < nlev) e += (size_t)NP3 * ns[q + 1] * ns[q + 1] * ns[q + 1];
+    for (int l = tail3_first(c); l < c.nlev; l++) {
+        const size_t n = c.lev[l].n, nc = l + 1 < c.nlev ? c.lev[l + 1].n : 0;
+        e += NS3 * n * n * n + NP3 * nc * nc * nc;
     }
     return e;
+}
+size_t tail3_vec_elems(const Ctx& c) {
+    size_t e = 0;
+    for (int l = tail3_first(c); l < c.nlev; l++) e += 3 * (size_t)c.lev[l].n * c.lev[l].n * c.lev[l].n;
+    return e;
+}
+
+// A level in shared memory: n^3 arrays.
+template <typename T>
+struct T3 {
+    int n, nc;           // nodes per side, of the next level
+    T *A, *P, *b, *x, *r;
+};
+
+// One colour: sel < 0: forward Gauss-Seidel update from the zero guess (the
+// couplings to earlier colours); sel == 0: reverse update (all); sel > 0: the
+// residual after the forward sweep into r (those to later colours).  The
+// colour is a run-time value, uniform over the CTA: unrolled per colour the
+// code outran the instruction cache (FP32 tail 72 us instead of 42).
+template <typename T>
+__device__ __forceinline__ void tail3_colour(const T3<T>& v, int col, int sel, int tid) {
+    const int n = v.n, n3 = n * n * n;
+    const int pi = col & 1, pj = (col >> 1) & 1, pk = col >> 2;
+    // n = 2^k + 1: walk 2^(k-1) points a side and leave out the even
+    // coordinates' last one, so that positions are shifts and masks
+    const int lg = 31 - __clz(n - 1) - 1, m = 1 << lg;
+    const int h = tid & 1;
+    for (int t0 = 0; t0 < m * m * m; t0 += kTail3Threads / 2) {
+        const int t = t0 + (tid >> 1);
+        const int I = t & (m - 1), J = (t >> lg) & (m - 1), K = t >> (2 * lg);
+        const int i = 2 - pi + 2 * I, j = 2 - pj + 2 * J, k = 2 - pk + 2 * K;
+        const bool on = i < n - 1 && j < n - 1 && k < n - 1;
+        const int o = i + n * (j + n * k);
+        T s = 0;
+        if (on) {
+#pragma unroll
+            for (int q = 0; q < 13; q++) {
+                const int c = col ^ off_mask(q);
+                if (sel == 0 || (c > col) == (sel > 0)) {
+                    const int d = off_x(q) + n * (off_y(q) + n * off_z(q));
+                    s += v.A[q * n3 + (h ? o - d : o)] * v.x[h ? o - d : o + d];
+                }
+            }
+        }
+        s += __shfl_xor_sync(0xffffffffu, s, 1);
+        if (on && h == 0) {
+            if (sel > 0)
+                v.r[o] = -s;
+            else
+                v.x[o] = (v.b[o] - s) * v.A[13 * n3 + o];
+        }
+    }
 }
 
 template <typename T>
 __global__ void __launch_bounds__(kTail3Threads) k_vtail3d(Tail3Args<T> a) {
     extern __shared__ __align__(16) unsigned char t3_raw[];
-    __shared__ Tail3Level<T> lv[kTail3Lev];
-    const int tid = threadIdx.x, nth = blockDim.x;
+    __shared__ T3<T> lv[kTail3Lev];
+    __shared__ uint64_t bar;
+    const int tid = threadIdx.x, nth = kTail3Threads;
     const int L = a.nlev;
+    T* base = reinterpret_cast<T*>(t3_raw);
     if (tid == 0) {
-        T* sp = reinterpret_cast<T*>(t3_raw);
+        // the packed operators and weights, level after level
+        mbar::init(&bar, 1);
+        mbar::fence_init();
+        mbar::expect_tx(&bar, a.pack_bytes);
+        for (unsigned off = 0; off < a.pack_bytes; off += kTail3Chunk) {
+            const unsigned len = a.pack_bytes - off < kTail3Chunk ? a.pack_bytes - off : kTail3Chunk;
+            mbar::bulk_g2s(t3_raw + off, (const unsigned char*)a.pack + off, len, &bar);
+        }
+        T* sp = base;
+        T* vp = base + a.pack_bytes / sizeof(T);
         for (int q = 0; q < L; q++) {
-            lv[q] = a.lv[q];
-            if (tail3_stages<T>()) {
-                const int n = a.lv[q].A.n;
-                const long long n3 = (long long)n * n * n;
-                lv[q].A = L3<T>{sp, n, n, n3};
-                sp += NS3 * n3;
-                if (q + 1 < L) {
-                    const int nc = a.lv[q + 1].A.n;
-                    lv[q].P = sp;
-                    lv[q].ldc = nc;
-                    lv[q].plc = (long long)nc * nc * nc;
-                    sp += NP3 * lv[q].plc;
-                }
-                lv[q].b = sp;
-                lv[q].x = sp + n3;
-                lv[q].r = sp + 2 * n3;
-                sp += 3 * n3;
-            }
+            T3<T>& v = lv[q];
+            const int n = v.n = a.n[q], n3 = n * n * n;
+            v.nc = q + 1 < L ? a.n[q + 1] : 0;
+            v.A = sp;
+            v.P = v.A + NS3 * n3;
+            sp = v.P + NP3 * v.nc * v.nc * v.nc;
+            v.b = vp;
+            v.x = v.b + n3;
+            v.r = v.x + n3;
+            vp = v.r + n3;
         }
     }
     __syncthreads();
-    if (tail3_stages<T>()) {
-        // operators (NS3 planes) and weights (NP3 planes on the next grid),
-        // from the padded layout into the compact one; the first level's
-        // right-hand side
-        {
-            const Tail3Level<T>& g = a.lv[0];
-            const int n = g.A.n, n3 = n * n * n;
-            T* db = const_cast<T*>(lv[0].b);
-            for (int u = tid; u < n3; u += nth) {
-                const int i = u % n, j = (u / n) % n, k = u / (n * n);
-                db[u] = g.b[g.A.idx(i, j, k)];
-            }
-        }
-        for (int q = 0; q < L; q++) {
-            const Tail3Level<T>& g = a.lv[q];
-            const int n = g.A.n;
-            const int n3 = n * n * n;
-            T* dA = const_cast<T*>(lv[q].A.A);
-            for (int e = tid; e < NS3 * n3; e += nth) {
-                const int t = e / n3, u = e - t * n3;
-                const int i = u % n, j = (u / n) % n, k = u / (n * n);
-                dA[e] = g.A.A[t * g.A.pl + g.A.idx(i, j, k)];
-            }
-            if (q + 1 < L) {
-                const int nc = a.lv[q + 1].A.n, nc3 = nc * nc * nc;
-                T* dP = const_cast<T*>(lv[q].P);
-                for (int e = tid; e < NP3 * nc3; e += nth) {
-                    const int t = e / nc3, u = e - t * nc3;
-                    const int i = u % nc, j = (u / nc) % nc, k = u / (nc * nc);
-                    dP[e] = g.P[t * g.plc + (long long)i + (long long)g.ldc * (j + (long long)nc * k)];
-                }
-            }
-        }
-        __syncthreads();
-    }
-    auto colour = [&](const Tail3Level<T>& v, int col) {
-        const int n = v.A.n;
-        const int pi = col & 1, pj = (col >> 1) & 1, pk = col >> 2;
-        const int ni = cb_side(n, pi), nj = cb_side(n, pj), nk = cb_side(n, pk);
-        for (int t = tid; t < ni * nj * nk; t += nth) {
-            const int i = 2 - pi + 2 * (t % ni), j = 2 - pj + 2 * ((t / ni) % nj), k = 2 - pk + 2 * (t / (ni * nj));
-            const long long o = v.A.idx(i, j, k);
-            v.x[o] = (v.b[o] - offdiag3(v.A, v.x, i, j, k)) / v.A.A[13 * v.A.pl + o];
-        }
-    };
-    for (int l = 0; l + 1 < L; l++) {
-        const Tail3Level<T>& v = lv[l];
-        const Tail3Level<T>& w = lv[l + 1];
-        const int n = v.A.n, m = n - 2;
-        for (long long q = tid; q < (long long)v.A.ld * n * n; q += nth) v.x[q] = (T)0;
-        __syncthreads();
-        for (int col = 0; col < 8; col++) {
-            colour(v, col);
-            __syncthreads();
-        }
-        for (int q = tid; q < m * m * m; q += nth) {
-            const int i = 1 + q % m, j = 1 + (q / m) % m, k = 1 + q / (m * m);
-            const long long o = v.A.idx(i, j, k);
-            v.r[o] = v.b[o] - (v.A.A[13 * v.A.pl + o] * v.x[o] + offdiag3(v.A, v.x, i, j, k));
-        }
-        __syncthreads();
-        const int nc = w.A.n, mc = nc - 2;
-        for (int q = tid; q < mc * mc * mc; q += nth) {
-            const int I = 1 + q % mc, J = 1 + (q / mc) % mc, K = 1 + q / (mc * mc);
-            restrict_node3d<T>(n, v.A.ld, v.r, v.P, nc, v.ldc, v.plc, (T*)w.b, w.A.ld, I, J, K);
-        }
-        __syncthreads();
-    }
-    {   // coarsest: one unknown, exact in FP64; the rest of its iterate is zero
-        const Tail3Level<T>& v = lv[L - 1];
-        const int n = v.A.n;
-        for (long long q = tid; q < (long long)v.A.ld * n * n; q += nth) v.x[q] = (T)0;
-        __syncthreads();
-        if (tid == 0) {
-            const long long o = v.A.idx(1, 1, 1);
-            v.x[o] = (T)((double)v.b[o] / *a.a64c);
-        }
-        __syncthreads();
-    }
-    for (int l = L - 2; l >= 0; l--) {
-        const Tail3Level<T>& v = lv[l];
-        const Tail3Level<T>& w = lv[l + 1];
-        const int n = v.A.n, nc = w.A.n, mc = nc - 1;
-        for (int q = tid; q < mc * mc * mc; q += nth) {
-            const int I = q % mc, J = (q / mc) % mc, K = q / (mc * mc);
-            prolong_node3d<T>(n, v.A.ld, v.x, v.P, nc, v.ldc, v.plc, w.x, w.A.ld, I, J, K);
-        }
-        __syncthreads();
-        for (int col = 7; col >= 0; col--) {
-            colour(v, col);
-            __syncthreads();
-        }
-    }
-    if (tail3_stages<T>()) {   // the first level's iterate back to its array
-        const Tail3Level<T>& g = a.lv[0];
-        const int n = g.A.n, n3 = n * n * n;
+    // meanwhile: zero iterates and residuals, the first level's right-hand side
+    for (int q = 0; q < L; q++) {
+        const T3<T> v = lv[q];
+        const int n = v.n, n3 = n * n * n;
         for (int u = tid; u < n3; u += nth) {
             const int i = u % n, j = (u / n) % n, k = u / (n * n);
-            g.x[g.A.idx(i, j, k)] = lv[0].x[u];
+            v.b[u] = q == 0 ? a.b[(long long)i + (long long)a.ld * (j + (long long)n * k)] : (T)0;
+            v.x[u] = v.r[u] = (T)0;
         }
+    }
+    if (!__syncthreads_and(mbar::wait(&bar, 0))) {
+        // record the expiry, give the copies in flight one more bounded wait
+        // (the shared memory must outlive them) and leave
+        if (tid == 0) set_err(a.st, BMG_ERR_TIMEOUT);
+        mbar::wait(&bar, 0);
+        return;
+    }
+    for (int l = 0; l + 1 < L; l++) {
+        const T3<T> v = lv[l], w = lv[l + 1];
+#pragma unroll 1
+        for (int ph = 0; ph < 15; ph++) {      // colours 0..7 forward, residuals of colours 0..6
+            tail3_colour<T>(v, ph & 7, ph < 8 ? -1 : 1, tid);
+            if (ph < 8 || ph == 14) __syncthreads();
+        }
+        const int nc = w.n, mc = nc - 2;
+        for (int q = tid; q < mc * mc * mc; q += nth) {
+            const int I = 1 + q % mc, J = 1 + (q / mc) % mc, K = 1 + q / (mc * mc);
+            restrict_node3d<T>(v.n, v.n, v.r, v.P, nc, nc, (long long)nc * nc * nc, w.b, nc, I, J, K);
+        }
+        __syncthreads();
+    }
+    if (tid == 0) {   // coarsest: one unknown, exact in FP64
+        const T3<T> v = lv[L - 1];
+        const int o = 1 + v.n * (1 + v.n);
+        v.x[o] = (T)((double)v.b[o] / *a.a64c);
+    }
+    __syncthreads();
+    for (int l = L - 2; l >= 0; l--) {
+        const T3<T> v = lv[l], w = lv[l + 1];
+        const int n = v.n, nc = w.n, m = n - 2, nc3 = nc * nc * nc;
+        for (int q = tid; q < m * m * m; q += nth) {
+            const int i = 1 + q % m, j = 1 + (q / m) % m, k = 1 + q / (m * m);
+            const int b = (i & 1) | ((j & 1) << 1) | ((k & 1) << 2);
+            const int oc = (i >> 1) + nc * ((j >> 1) + nc * (k >> 1));
+            T s = 0;
+            if (b == 0) {
+                s = w.x[oc];
+            } else {
+                for (int c = 0, e = 0; c < 8; c++)
+                    if ((c & ~b) == 0) {
+                        s += v.P[(kPBase(b) + e) * nc3 + oc] * w.x[oc + (c & 1) + nc * (((c >> 1) & 1) + nc * (c >> 2))];
+                        e++;
+                    }
+            }
+            v.x[i + n * (j + n * k)] += s;
+        }
+        __syncthreads();
+#pragma unroll 1
+        for (int col = 7; col >= 0; col--) {
+            tail3_colour<T>(v, col, 0, tid);
+            __syncthreads();
+        }
+    }
+    {   // the first level's iterate to its array
+        const int n = a.n[0], n3 = n * n * n;
+        for (int u = tid; u < n3; u += nth) {
+            const int i = u % n, j = (u / n) % n, k = u / (n * n);
+            a.x[(long long)i + (long long)a.ld * (j + (long long)n * k)] = lv[0].x[u];
+        }
+    }
+}
+
+// Packs one level: the operator's planes in compact rows (the diagonal as its
+// reciprocal), then the weights on the next level's grid.
+template <typename T>
+__global__ void k_tail3_pack(const T* __restrict__ A, int n, int ld, long long pl, const T* __restrict__ P, int nc,
+                             int ldc, long long plc, T* __restrict__ dst) {
+    const int n3 = n * n * n, nc3 = nc * nc * nc, tot = NS3 * n3 + NP3 * nc3;
+    for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < tot; e += gridDim.x * blockDim.x) {
+        const bool op = e < NS3 * n3;
+        const int m = op ? n : nc, m3 = op ? n3 : nc3, u = op ? e : e - NS3 * n3;
+        const int t = u / m3, r = u - t * m3;
+        const int i = r % m, j = (r / m) % m, k = r / (m * m);
+        T w = op ? A[t * pl + (long long)i + (long long)ld * (j + (long long)n * k)]
+                 : P[t * plc + (long long)i + (long long)ldc * (j + (long long)nc * k)];
+        if (op && t == 13 && w != (T)0) w = (T)1 / w;
+        dst[e] = w;
     }
 }
 
@@ -398,10 +501,11 @@ __global__ void __launch_bounds__(kTail3Threads) k_vtail3d(Tail3Args<T> a) {
 // in shared memory, with the two neighbouring planes' iterates beside it.
 // Within a plane, colour (i&1) + 2(j&1) of the last phase depends on the
 // first through a chain of at most three column steps and one row step, so
-// a tile of kHsTI x TJ owned points computes (kHsTI + 6) x (TJ + 2) points
+// a tile of TI x TJ owned points computes (TI + 6) x (TJ + 2) points
 // and neighbouring tiles recompute each other's halo.  Each point's update
 // is the per-colour kernels' update: the same 26 products summed in the
-// same order (offset t, then its mirror), the same division.
+// same order (offset t, then its mirror); FP64 multiplies by the stored
+// reciprocal of the diagonal, since FP64 arithmetic bounds it.
 //
 // Threads.  Lane p of a warp owns the column pair (ib + 2p, ib + 2p + 1) of
 // a row; the two points of a pair have consecutive colours, so a thread
@@ -413,21 +517,35 @@ __global__ void __launch_bounds__(kTail3Threads) k_vtail3d(Tail3Args<T> a) {
 //
 // Inputs and outputs are separate arrays (xout is never read), so a CTA
 // never sees a neighbour's finished values in place of the initial ones.
-constexpr int kHsPairs = 32;                 // column pairs per row: one per lane
-constexpr int kHsWarps = 8;
-constexpr int kHsThreads = 32 * kHsWarps;
-constexpr int kHsTI = 2 * kHsPairs - 6;      // owned columns of a tile (58)
-constexpr int kHsHalf = kHsPairs + 2;        // one parity's columns in a shared row
-constexpr int kHsCols = 2 * kHsHalf;         // shared row: columns ib-2 .. ib+65
-__host__ __device__ constexpr int hs_tj(int rows) { return 2 * kHsWarps * rows - 2; }   // owned rows
-__host__ __device__ constexpr int hs_srows(int rows) { return hs_tj(rows) + 4; }        // shared rows
-// Rows per warp and phase: one (58 x 14 owned points, 80 registers, 3 CTAs
-// per SM) measured faster than two (58 x 30, 128 registers, 2 CTAs per SM):
-// 0.66 against 0.76 ms per 257^3 V-cycle's finest-level half sweeps.
+//
+// Tile shapes.  W warps share a row (64 W computed columns) and S row slots
+// give 2 S computed rows, 2 S - 2 of them owned.  FULL: the tile spans the
+// whole row and needs no column halo; otherwise it owns 64 W - 6 columns.
+// hsweep3d takes the full row up to 129: 58-column tiles compute 192 columns
+// for the 127 points of a 129-node row (reverse sweep of one parity at 129^3:
+// FP64 120 us, full row 95; FP32 32.6, full row 27.8) and 128 for 63.  At 257^3
+// a row takes four warps, so either the rows' halo grows (four slots) or the
+// CTA does: 257 us against 196 for the 58-column tiles.
+template <int W_, int S_, bool FULL_>
+struct HsShape {
+    static constexpr int W = W_, S = S_;
+    static constexpr bool FULL = FULL_;
+    static constexpr int threads = 32 * W * S;
+    static constexpr int TI = FULL ? 64 * W : 64 * W - 6;   // owned columns
+    static constexpr int TJ = 2 * S - 2;                    // owned rows
+    static constexpr int half = 32 * W + 2;                 // one parity's columns in a shared row
+    static constexpr int cols = 2 * half;                   // shared row: columns ib-2 .. ib+64W+1
+    static constexpr int rows = TJ + 4;                     // shared rows
+    static constexpr int plane = rows * cols;
+};
+
+// In-plane couplings (offsets t >= 9 and their mirrors) that the update of a
+// point of the plane's colour col needs: all of them in a reverse sweep, in a
+// forward sweep from the zero guess those to the colours already updated.
+__host__ __device__ constexpr bool hs_in(int t, int col, bool fwd) { return !fwd || (col ^ (off_mask(t) & 3)) < col; }
+// plane of the diagonal: FP64 levels keep its reciprocal behind the operator
 template <typename T>
-constexpr int hs_rows() { return 1; }
-template <typename T>
-constexpr size_t hs_smem() { return sizeof(T) * 3 * (size_t)hs_srows(hs_rows<T>()) * kHsCols; }
+constexpr int hs_diag() { return sizeof(T) == 8 ? NS3 : 13; }
 
 template <typename T>
 struct HS3Args {
@@ -441,40 +559,32 @@ struct HS3Args {
     int parity;          // planes k with k & 1 == parity
 };
 
-template <typename T>
-struct V2 {
-    T x, y;
-};
-template <typename T>
-__device__ __forceinline__ V2<T> ld2(const T* p) {
-    if constexpr (sizeof(T) == 4) {
-        const float2 v = __ldg(reinterpret_cast<const float2*>(p));
-        return {v.x, v.y};
-    } else {
-        const double2 v = __ldg(reinterpret_cast<const double2*>(p));
-        return {v.x, v.y};
-    }
-}
-
 // One pair's stencil: the 14 stored planes at both points (own) and, for
 // each stored offset d, the mirror a(q, q - d) stored at q - d.
-template <typename T, int MODE>
+template <typename T, int MODE, bool FWD>
 struct HsPair {
     T own0[NS3], own1[NS3];   // first (even column) / second point
     T mir0[13], mir1[13];
     T f0, f1;
+    // JODD: the row's parity (its two points have colours 2 JODD, 2 JODD + 1)
+    template <int JODD>
+    static constexpr bool needs(int t) {
+        return t < 9 ? MODE != 0   // z-couplings (mode 0: the odd planes are still zero)
+                     : hs_in(t, 2 * JODD, FWD) || hs_in(t, 2 * JODD + 1, FWD);
+    }
+    template <int JODD>
     __device__ __forceinline__ void load(const HS3Args<T>& a, long long o0, bool first_ok) {
         const long long sz = (long long)a.ld * a.n;
 #pragma unroll
         for (int t = 0; t < NS3; t++) {
-            if (MODE == 0 && t < 9) continue;   // z-couplings: the odd planes are still zero
-            const V2<T> v = ld2(a.A + t * a.pl + o0);
+            if (t < 13 && !needs<JODD>(t)) continue;
+            const V2<T> v = ld2(a.A + (t == 13 ? hs_diag<T>() : t) * a.pl + o0);
             own0[t] = v.x;
             own1[t] = v.y;
         }
 #pragma unroll
         for (int t = 0; t < 13; t++) {
-            if (MODE == 0 && t < 9) continue;
+            if (!needs<JODD>(t)) continue;
             const int dx = off_x(t), dy = off_y(t), dz = off_z(t);
             const long long m = o0 - (long long)dy * a.ld - dz * sz;   // node (i, j - dy, k - dz)
             const T* b = a.A + t * a.pl + m;
@@ -499,54 +609,51 @@ struct HsPair {
 // Gauss-Seidel update of one point from its stencil and the shared
 // iterates.  ODD: the point is the pair's second (odd) column.  s: index of
 // the point's row in the shared arrays (row start), p: the pair.
-template <typename T, int MODE, bool ODD>
+template <typename T, typename SH, int MODE, bool FWD, int JODD, bool ODD>
 __device__ __forceinline__ T hs_update(const T* own, const T* mir, T f, const T* xc, const T* xb, const T* xa,
                                        int rs, int p) {
     // shared index of the neighbour at column offset dx, row offset dy
     auto at = [&](int dx, int dy) {
-        const int c = ODD ? (dx == 0 ? kHsHalf + p + 1 : (dx < 0 ? p + 1 : p + 2))
-                          : (dx == 0 ? p + 1 : (dx < 0 ? kHsHalf + p : kHsHalf + p + 1));
-        return rs + dy * kHsCols + c;
+        const int c = ODD ? (dx == 0 ? SH::half + p + 1 : (dx < 0 ? p + 1 : p + 2))
+                          : (dx == 0 ? p + 1 : (dx < 0 ? SH::half + p : SH::half + p + 1));
+        return rs + dy * SH::cols + c;
     };
     T s = 0;
 #pragma unroll
     for (int t = 0; t < 13; t++) {
         if (MODE == 0 && t < 9) continue;
+        if (t >= 9 && !hs_in(t, 2 * JODD + ODD, FWD)) continue;
         const int dx = off_x(t), dy = off_y(t), dz = off_z(t);
         const T* xp = dz < 0 ? xb : xc;   // plane of q + d
         const T* xm = dz < 0 ? xa : xc;   // plane of q - d
         s += own[t] * xp[at(dx, dy)];
         s += mir[t] * xm[at(-dx, -dy)];
     }
-    return (f - s) / own[13];
+    return sizeof(T) == 8 ? (f - s) * own[13] : (f - s) / own[13];
 }
 
 // MODE 0: zero initial iterate, no z-couplings (forward sweep of the even
 // planes); MODE 1: zero initial iterate, z-couplings to xz (forward sweep of
 // the odd planes); MODE 2: initial iterate xcur, z-couplings to xz (reverse
 // sweeps).  FWD: colours of the plane ascending, else descending.
-template <typename T, int MODE, bool FWD>
-__global__ void __launch_bounds__(kHsThreads) k_hsweep3d(HS3Args<T> a) {
-    constexpr int ROWS = hs_rows<T>();
-    constexpr int TJ = hs_tj(ROWS);
-    constexpr int SR = hs_srows(ROWS);
-    constexpr int PLANE = SR * kHsCols;
+template <typename T, typename SH, int MODE, bool FWD>
+__global__ void __launch_bounds__(SH::threads, (sizeof(T) == 8 ? 512 : 768) / SH::threads) k_hsweep3d(HS3Args<T> a) {
     extern __shared__ __align__(16) unsigned char hs_raw[];
     T* xc = reinterpret_cast<T*>(hs_raw);   // swept plane k
-    T* xb = xc + PLANE;                      // plane k - 1
-    T* xa = xb + PLANE;                      // plane k + 1
+    T* xb = xc + SH::plane;                  // plane k - 1
+    T* xa = xb + SH::plane;                  // plane k + 1
     const int n = a.n, ld = a.ld;
     const long long sz = (long long)ld * n;
     const int k = 2 - a.parity + 2 * (int)blockIdx.z;
-    const int i0 = 1 + (int)blockIdx.x * kHsTI, j0 = 1 + (int)blockIdx.y * TJ;
-    const int ib = i0 - 3;                   // first computed column (even)
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int i0 = 1 + (int)blockIdx.x * SH::TI, j0 = 1 + (int)blockIdx.y * SH::TJ;
+    const int ib = SH::FULL ? 0 : i0 - 3;    // first computed column (even)
+    const int tid = threadIdx.x;
     // shared position (lr, lc) holds node (ib - 2 + lc, j0 - 2 + lr)
-    for (int q = tid; q < PLANE; q += kHsThreads) {
-        const int lr = q / kHsCols, lc = q - lr * kHsCols;
+    for (int q = tid; q < SH::plane; q += SH::threads) {
+        const int lr = q / SH::cols, lc = q - lr * SH::cols;
         const int i = ib - 2 + lc, j = j0 - 2 + lr;
         const bool in = i >= 1 && i <= n - 2 && j >= 1 && j <= n - 2;
-        const int s = lr * kHsCols + (lc & 1) * kHsHalf + (lc >> 1);
+        const int s = lr * SH::cols + (lc & 1) * SH::half + (lc >> 1);
         const long long o = (long long)i + (long long)ld * j + sz * k;
         xc[s] = (MODE == 2 && in) ? a.xcur[o] : (T)0;
         if (MODE >= 1) {
@@ -555,53 +662,54 @@ __global__ void __launch_bounds__(kHsThreads) k_hsweep3d(HS3Args<T> a) {
         }
     }
     __syncthreads();
-    const int p = lane;
-    const int i = ib + 2 * p;                // the pair's first column
-    HsPair<T, MODE> hold[ROWS];
-    bool ok0[ROWS], ok1[ROWS];
-    // one row parity: PH = 0 loads and updates the pair's earlier colour,
-    // PH = 1 updates the later one from the registers
-    auto phase = [&](int jpar, bool second) {
-#pragma unroll
-        for (int r = 0; r < ROWS; r++) {
-            const int lrow = 2 * (warp + kHsWarps * r) + jpar;   // region row, j = j0 - 1 + lrow
-            const int j = j0 - 1 + lrow;
-            const int rs = (lrow + 1) * kHsCols;
+    const int slot = tid / (32 * SH::W);
+    const int p = tid - 32 * SH::W * slot;   // the pair's index in the row
+    const int i = ib + 2 * p;                // its first column
+    HsPair<T, MODE, FWD> hold;
+    bool ok0 = false, ok1 = false;
+    // one row parity: the first call loads and updates the pair's earlier
+    // colour, the second updates the later one from the registers
+    auto phase = [&](auto jp, bool second) {
+        constexpr int jpar = decltype(jp)::value;   // the rows' parity: j0 - 1 is even
+        const int lrow = 2 * slot + jpar;           // region row, j = j0 - 1 + lrow
+        const int j = j0 - 1 + lrow;
+        const int rs = (lrow + 1) * SH::cols;
+        if (!second) {
             const bool pv = j >= 1 && j <= n - 2 && i >= 0 && i <= n - 2;
-            if (!second) {
-                ok0[r] = pv && i >= 1;
-                ok1[r] = pv && i + 1 <= n - 2;
-                if (pv) hold[r].load(a, (long long)i + (long long)ld * j + sz * k, ok0[r]);
-            }
-            // FWD: even column first; reverse: odd column first
-            const bool do_odd = FWD ? second : !second;
-            if (do_odd) {
-                if (ok1[r]) xc[rs + kHsHalf + p + 1] =
-                    hs_update<T, MODE, true>(hold[r].own1, hold[r].mir1, hold[r].f1, xc, xb, xa, rs, p);
-            } else {
-                if (ok0[r]) xc[rs + p + 1] =
-                    hs_update<T, MODE, false>(hold[r].own0, hold[r].mir0, hold[r].f0, xc, xb, xa, rs, p);
-            }
+            ok0 = pv && i >= 1;
+            ok1 = pv && i + 1 <= n - 2;
+            if (pv) hold.template load<jpar>(a, (long long)i + (long long)ld * j + sz * k, ok0);
+        }
+        // FWD: even column first; reverse: odd column first
+        const bool do_odd = FWD ? second : !second;
+        if (do_odd) {
+            if (ok1)
+                xc[rs + SH::half + p + 1] =
+                    hs_update<T, SH, MODE, FWD, jpar, true>(hold.own1, hold.mir1, hold.f1, xc, xb, xa, rs, p);
+        } else {
+            if (ok0)
+                xc[rs + p + 1] =
+                    hs_update<T, SH, MODE, FWD, jpar, false>(hold.own0, hold.mir0, hold.f0, xc, xb, xa, rs, p);
         }
         __syncthreads();
     };
     if (FWD) {
-        phase(0, false);
-        phase(0, true);
-        phase(1, false);
-        phase(1, true);
+        phase(std::integral_constant<int, 0>{}, false);
+        phase(std::integral_constant<int, 0>{}, true);
+        phase(std::integral_constant<int, 1>{}, false);
+        phase(std::integral_constant<int, 1>{}, true);
     } else {
-        phase(1, false);
-        phase(1, true);
-        phase(0, false);
-        phase(0, true);
+        phase(std::integral_constant<int, 1>{}, false);
+        phase(std::integral_constant<int, 1>{}, true);
+        phase(std::integral_constant<int, 0>{}, false);
+        phase(std::integral_constant<int, 0>{}, true);
     }
-    for (int q = tid; q < kHsTI * TJ; q += kHsThreads) {
-        const int lj = q / kHsTI, li = q - lj * kHsTI;
+    for (int q = tid; q < SH::TI * SH::TJ; q += SH::threads) {
+        const int lj = q / SH::TI, li = q - lj * SH::TI;
         const int ii = i0 + li, jj = j0 + lj;
         if (ii > n - 2 || jj > n - 2) continue;
         const int lc = ii - ib + 2, lr = jj - j0 + 2;
-        a.xout[(long long)ii + (long long)ld * jj + sz * k] = xc[lr * kHsCols + (lc & 1) * kHsHalf + (lc >> 1)];
+        a.xout[(long long)ii + (long long)ld * jj + sz * k] = xc[lr * SH::cols + (lc & 1) * SH::half + (lc >> 1)];
     }
 }
 
@@ -688,56 +796,59 @@ bmg_status colour_blocks3d(Ctx& c) {
 // profiler: per point of the parity its stored planes (in-plane ones only in
 // mode 0), the mirrored z-planes of the plane above, the neighbouring
 // planes' iterate, the right-hand side, the output and (mode 2) the input.
-template <typename T, int MODE, bool FWD>
-bmg_status hsweep3d(Ctx& c, int l, const T* f, const T* xcur, const T* xz, T* xout, int parity) {
-    const Level& F = c.lev[l];
-    constexpr int TJ = hs_tj(hs_rows<T>());
-    const int planes = parity ? (F.n - 1) / 2 : (F.n - 3) / 2;
-    if (planes < 1) return BMG_OK;
-    HS3Args<T> a{A_of<T>(F), F.n, F.ld, F.plane, f, xcur, xz, xout, parity};
-    const dim3 grid(cdiv(F.n - 2, kHsTI), cdiv(F.n - 2, TJ), planes);
-    prof_begin(c, BMG_PROF_SMOOTH, l);
-    k_hsweep3d<T, MODE, FWD><<<grid, kHsThreads, hs_smem<T>(), c.stream>>>(a);
+template <typename T, typename SH, int MODE, bool FWD>
+bmg_status launch_hsweep3d(Ctx& c, const HS3Args<T>& a, int planes) {
+    auto kern = k_hsweep3d<T, SH, MODE, FWD>;
+    const int smem = (int)(3 * SH::plane * sizeof(T));
+    if (smem > 48 * 1024) BMG_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+    kern<<<dim3(cdiv(a.n - 2, SH::TI), cdiv(a.n - 2, SH::TJ), planes), SH::threads, smem, c.stream>>>(a);
     c.launches++;
-    const double per = MODE == 0 ? 5.0 + 2.0 : (MODE == 1 ? 14.0 + 9.0 + 2.0 + 2.0 : 14.0 + 9.0 + 2.0 + 3.0);
-    prof_end(c, BMG_PROF_SMOOTH, l, per * sizeof(T) * dofs3(c, l) / 2);
+    BMG_CUDA(cudaGetLastError());
     return BMG_OK;
 }
 
-// The half-sweep legs of a level (FP32 only: see use_hs3).
-template <typename T>
-bool hs3_on(const Ctx& c) { return sizeof(T) == 4 && c.use_hs3; }
+template <typename T, int MODE, bool FWD>
+bmg_status hsweep3d(Ctx& c, int l, const T* f, const T* xcur, const T* xz, T* xout, int parity) {
+    const Level& F = c.lev[l];
+    const int planes = parity ? (F.n - 1) / 2 : (F.n - 3) / 2;
+    if (planes < 1) return BMG_OK;
+    const HS3Args<T> a{A_of<T>(F), F.n, F.ld, F.plane, f, xcur, xz, xout, parity};
+    prof_begin(c, BMG_PROF_SMOOTH, l);
+    bmg_status st;
+    if (F.n <= 65)
+        st = launch_hsweep3d<T, HsShape<1, 8, true>, MODE, FWD>(c, a, planes);
+    else if (F.n <= 129)
+        st = launch_hsweep3d<T, HsShape<2, 4, true>, MODE, FWD>(c, a, planes);
+    else
+        st = launch_hsweep3d<T, HsShape<1, 8, false>, MODE, FWD>(c, a, planes);
+    const double per = MODE == 0 ? 5.0 + 2.0 : (MODE == 1 ? 14.0 + 9.0 + 2.0 + 2.0 : 14.0 + 9.0 + 2.0 + 3.0);
+    prof_end(c, BMG_PROF_SMOOTH, l, per * sizeof(T) * dofs3(c, l) / 2);
+    return st;
+}
 
+// The half-sweep legs of a level.
 template <typename T>
 bmg_status hs3_down(Ctx& c, int l, const T* f, T* x) {
-    if constexpr (sizeof(T) == 4) {
-        // even planes (their odd neighbours still zero), then odd planes
-        BMG_TRY((hsweep3d<T, 0, true>(c, l, f, nullptr, nullptr, x, 0)));
-        return hsweep3d<T, 1, true>(c, l, f, nullptr, x, x, 1);
-    } else {
-        return BMG_ERR_STATE;
-    }
+    // even planes (their odd neighbours still zero), then odd planes
+    BMG_TRY((hsweep3d<T, 0, true>(c, l, f, nullptr, nullptr, x, 0)));
+    return hsweep3d<T, 1, true>(c, l, f, nullptr, x, x, 1);
 }
 
 template <typename T>
 bmg_status hs3_up(Ctx& c, int l, const T* f, T* x, const T* xc) {
-    if constexpr (sizeof(T) == 4) {
-        // x + P x_c into the residual buffer (free until the next down leg),
-        // then the odd planes against the corrected even planes, then the
-        // even planes against the finished odd planes
-        const Level& F = c.lev[l];
-        const Level& K = c.lev[l + 1];
-        T* xcor = (T*)F.r;
-        prof_begin(c, BMG_PROF_PROLONG, l);
-        k_prolong3d_to<T><<<g3(K.n - 1, K.n - 1, K.n - 1), 64, 0, c.stream>>>(F.n, F.ld, x, xcor, P_of<T>(F), K.n,
-                                                                               K.ld, K.plane, xc);
-        prof_end(c, BMG_PROF_PROLONG, l, (2.0 + c.np / 8.0 + 0.125) * sizeof(T) * dofs3(c, l));
-        c.launches += 1;
-        BMG_TRY((hsweep3d<T, 2, false>(c, l, f, xcor, xcor, x, 1)));
-        return hsweep3d<T, 2, false>(c, l, f, xcor, x, x, 0);
-    } else {
-        return BMG_ERR_STATE;
-    }
+    // x + P x_c into the residual buffer (free until the next down leg), then
+    // the odd planes against the corrected even planes, then the even planes
+    // against the finished odd planes
+    const Level& F = c.lev[l];
+    const Level& K = c.lev[l + 1];
+    T* xcor = (T*)F.r;
+    prof_begin(c, BMG_PROF_PROLONG, l);
+    k_prolong3d_to<T><<<g3(K.n - 1, K.n - 1, K.n - 1), 64, 0, c.stream>>>(F.n, F.ld, x, xcor, P_of<T>(F), K.n, K.ld,
+                                                                           K.plane, xc);
+    prof_end(c, BMG_PROF_PROLONG, l, (2.0 + c.np / 8.0 + 0.125) * sizeof(T) * dofs3(c, l));
+    c.launches += 1;
+    BMG_TRY((hsweep3d<T, 2, false>(c, l, f, xcor, xcor, x, 1)));
+    return hsweep3d<T, 2, false>(c, l, f, xcor, x, x, 0);
 }
 
 template <typename T>
@@ -747,23 +858,22 @@ bmg_status vcycle3d_impl(Ctx& c, const T* b0, T* x0, T* xout) {
     const double sz = sizeof(T);
     auto bl = [&](int l) { return l == 0 ? b0 : (const T*)c.lev[l].b; };
     auto xl = [&](int l) { return l == 0 ? x0 : (T*)c.lev[l].x; };
-    // levels t .. L-1 (n <= tail3_max_n) run in the single-CTA tail
-    int t = L - 1;
-    while (t > 0 && c.lev[t - 1].n <= tail3_max_n<T>()) t--;
+    // levels t .. L-1 run in the single-CTA tail
+    const int t = tail3_first(c);
     for (int l = 0; l < t; l++) {
         const Level& F = c.lev[l];
         const Level& K = c.lev[l + 1];
         L3<T> v{A_of<T>(F), F.n, F.ld, F.plane};
-        BMG_CUDA(cudaMemsetAsync(xl(l), 0, sizeof(T) * F.plane, s));
         const int h = (F.n + 1) / 2;
         const double N = dofs3(c, l);
-        if (hs3_on<T>(c)) {
+        if (c.use_hs3) {   // writes every interior node, reads none before
             BMG_TRY(hs3_down(c, l, bl(l), xl(l)));
         } else {
+            BMG_CUDA(cudaMemsetAsync(xl(l), 0, sizeof(T) * F.plane, s));
             for (int col = 0; col < 8; col++) BMG_TRY(colour_sweep<T>(c, l, v, bl(l), xl(l), col, h));
         }
         prof_begin(c, BMG_PROF_RESIDUAL, l);
-        k_residual3d_sweep<T><<<g3(F.n, F.n, F.n), 64, 0, s>>>(v, xl(l), (T*)F.r);
+        k_residual3d_sweep<T><<<g3((F.n - 1) / 2, F.n - 2, F.n - 2), 64, 0, s>>>(v, xl(l), (T*)F.r);
         prof_end(c, BMG_PROF_RESIDUAL, l, (c.ns + 3) * sz * N);
         prof_begin(c, BMG_PROF_RESTRICT, l);
         k_restrict3d<T><<<g3(K.n, K.n, K.n), 64, 0, s>>>(F.n, F.ld, (const T*)F.r, P_of<T>(F), K.n, K.ld, K.plane,
@@ -774,28 +884,18 @@ bmg_status vcycle3d_impl(Ctx& c, const T* b0, T* x0, T* xout) {
     {
         Tail3Args<T> a{};
         a.nlev = L - t;
-        if (a.nlev > kTail3Lev) return BMG_ERR_STATE;   // n <= 17 has at most kTail3Lev levels
-        for (int q = 0; q < a.nlev; q++) {
-            const int l = t + q;
-            const Level& F = c.lev[l];
-            Tail3Level<T>& g = a.lv[q];
-            g.A = L3<T>{A_of<T>(F), F.n, F.ld, F.plane};
-            g.P = l + 1 < L ? P_of<T>(F) : nullptr;
-            g.ldc = l + 1 < L ? c.lev[l + 1].ld : 0;
-            g.plc = l + 1 < L ? c.lev[l + 1].plane : 0;
-            g.b = bl(l);
-            g.x = xl(l);
-            g.r = (T*)F.r;
-        }
+        if (a.nlev > kTail3Lev) return BMG_ERR_STATE;   // n <= 9 has at most kTail3Lev levels
+        for (int q = 0; q < a.nlev; q++) a.n[q] = c.lev[t + q].n;
+        a.pack = c.tail_pack;
+        a.pack_bytes = (unsigned)tail3_pack_bytes(c);
+        a.b = bl(t);
+        a.x = xl(t);
+        a.ld = c.lev[t].ld;
         const Level& C = c.lev[L - 1];
         a.a64c = C.A64 + 13 * C.plane + (long long)C.ld * (1 + (long long)C.n) + 1;
-        size_t smem = 0;
-        if (tail3_stages<T>()) {
-            int ns[kTail3Lev];
-            for (int q = 0; q < a.nlev; q++) ns[q] = c.lev[t + q].n;
-            smem = sizeof(T) * tail3_smem_elems(ns, a.nlev);
-            BMG_CUDA(cudaFuncSetAttribute(k_vtail3d<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-        }
+        a.st = c.st;
+        const size_t smem = a.pack_bytes + sizeof(T) * tail3_vec_elems(c);
+        BMG_CUDA(cudaFuncSetAttribute(k_vtail3d<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
         k_vtail3d<T><<<1, kTail3Threads, smem, s>>>(a);
         c.launches++;
     }
@@ -804,7 +904,7 @@ bmg_status vcycle3d_impl(Ctx& c, const T* b0, T* x0, T* xout) {
         const Level& K = c.lev[l + 1];
         L3<T> v{A_of<T>(F), F.n, F.ld, F.plane};
         const double N = dofs3(c, l);
-        if (hs3_on<T>(c)) {
+        if (c.use_hs3) {
             BMG_TRY(hs3_up(c, l, bl(l), xl(l), xl(l + 1)));
             continue;
         }
@@ -819,6 +919,34 @@ bmg_status vcycle3d_impl(Ctx& c, const T* b0, T* x0, T* xout) {
     (void)xout;
     BMG_CUDA(cudaGetLastError());
     return BMG_OK;
+}
+
+size_t tail3_pack_bytes(const Ctx& c) {
+    return (tail3_pack_elems(c) * (c.opts.precision == BMG_PREC_FP32 ? 4 : 8) + 15) & ~(size_t)15;
+}
+
+namespace {
+template <typename T>
+bmg_status tail3_pack_impl(Ctx& c) {
+    T* q = (T*)c.tail_pack;
+    for (int l = tail3_first(c); l < c.nlev; l++) {
+        const Level& F = c.lev[l];
+        const bool last = l + 1 == c.nlev;
+        const int nc = last ? 0 : c.lev[l + 1].n;
+        const int tot = NS3 * F.n * F.n * F.n + NP3 * nc * nc * nc;
+        k_tail3_pack<T><<<cdiv(tot, 256), 256, 0, c.stream>>>(A_of<T>(F), F.n, F.ld, F.plane, last ? nullptr : P_of<T>(F),
+                                                             nc, last ? 0 : c.lev[l + 1].ld,
+                                                             last ? 0 : c.lev[l + 1].plane, q);
+        c.launches++;
+        q += tot;
+    }
+    BMG_CUDA(cudaGetLastError());
+    return BMG_OK;
+}
+}  // namespace
+
+bmg_status tail3_pack(Ctx& c) {
+    return c.opts.precision == BMG_PREC_FP32 ? tail3_pack_impl<float>(c) : tail3_pack_impl<double>(c);
 }
 
 template bmg_status vcycle3d_impl<double>(Ctx&, const double*, double*, double*);
