@@ -102,8 +102,9 @@ void drop_mrhs(Ctx& c) {
 }
 
 bmg_status read_state(Ctx& c, KState& h) {
-    BMG_CUDA(cudaMemcpyAsync(&h, c.st, sizeof(KState), cudaMemcpyDeviceToHost, c.stream));
+    BMG_CUDA(cudaMemcpyAsync(c.st_host, c.st, sizeof(KState), cudaMemcpyDeviceToHost, c.stream));
     BMG_CUDA(cudaStreamSynchronize(c.stream));
+    h = *c.st_host;
     return BMG_OK;
 }
 
@@ -453,6 +454,7 @@ bmg_status bmg_attach(bmg_ctx* ctx, void* ws, size_t bytes, void* stream) {
     c.use_fused = c.dim == 2 && !(c.opts.flags & BMG_FLAG_UNFUSED) && c.nlev >= 2;
     c.use_hs3 = c.dim == 3 && !(c.opts.flags & BMG_FLAG_UNFUSED);
     c.use_graphs = !(c.opts.flags & BMG_FLAG_NO_GRAPHS);
+    BMG_TRY(node_tiles_prepare(c));
     if (c.use_fused) BMG_TRY(fused_prepare(c));
     c.attached = true;
     c.have_op = c.have_setup = false;

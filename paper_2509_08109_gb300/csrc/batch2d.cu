@@ -48,7 +48,6 @@ namespace {
 constexpr int R = kBatchR;
 constexpr int kBThreads = 256;                 // batched vector kernels: 64 columns x R
 constexpr int kBCols = kBThreads / R;
-constexpr int kRowBlocks = 32;                 // blocks per problem of the row-parallel kernels
 
 size_t a256(size_t v) { return (v + 255) & ~(size_t)255; }
 
@@ -244,17 +243,28 @@ __global__ void k_bunpack_all(const BProbDev* __restrict__ probs, const PackEnt*
 // ||r||^2 (and, with bb, ||b||^2) per system; the last block of the problem
 // stores them and restarts the inner CG of its active systems.  Rows whose x
 // neighbourhood is zero take r = b without the FP64 products.
+// A block takes kResRows rows, so a problem has blocks in proportion to its
+// rows (the grid's width is the largest problem's count, the blocks past a
+// problem's own leave at once): FP64 arithmetic, 12 operations a value, bounds
+// the kernel, and with a fixed 32 blocks for every problem the largest ones
+// ran on a fraction of the SMs (16 problems of 65..1025 x 4: mean of a
+// solve's four calls 1.12 ms, now 0.63 ms).
+constexpr int kResRows = 8;
+__host__ __device__ inline int res_blocks(int n) { return (n - 2 + kResRows - 1) / kResRows; }
+
 __global__ void __launch_bounds__(kBThreads) k_bresidual(const BProbDev* __restrict__ probs, SysState* sys,
                                                          double* partials, unsigned* counters, int bb) {
     __shared__ double red[kBThreads];
     __shared__ bool last;
     const int pi = blockIdx.y;
     const BProbDev P = probs[pi];
+    const int n = P.n, ld = P.ld, nb = res_blocks(n);
+    if ((int)blockIdx.x >= nb) return;
     const int rh = threadIdx.x % R, col = threadIdx.x / R;
-    const int n = P.n, ld = P.ld;
     const long long pl = P.plane;
     double acc = 0.0, accb = 0.0;
-    for (int j = 1 + blockIdx.x; j <= n - 2; j += gridDim.x) {
+    const int j1 = min(1 + ((int)blockIdx.x + 1) * kResRows, n - 1);
+    for (int j = 1 + (int)blockIdx.x * kResRows; j < j1; j++) {
         for (int i = 1 + col; i <= n - 2; i += kBCols) {
             const long long o = (long long)j * ld + i;
             const double* A = P.A64;
@@ -279,29 +289,32 @@ __global__ void __launch_bounds__(kBThreads) k_bresidual(const BProbDev* __restr
             }
             P.r[o * R + rh] = (float)v;
             acc += v * v;
-            accb += bv * bv;
+            if (bb) accb += bv * bv;
         }
     }
     const double t1 = block_sum_r(acc, red);
     const double t2 = bb ? block_sum_r(accb, red) : 0.0;
-    double* part = partials + ((long long)pi * gridDim.x + blockIdx.x) * 2 * R;
+    double* base = partials + (long long)pi * gridDim.x * 2 * R;
+    double* part = base + (long long)blockIdx.x * 2 * R;
     if (threadIdx.x < R) {
         part[2 * threadIdx.x] = t1;
         part[2 * threadIdx.x + 1] = t2;
     }
     __threadfence();
     __syncthreads();
-    if (threadIdx.x == 0) last = atomicAdd(&counters[pi], 1u) == gridDim.x - 1;
+    if (threadIdx.x == 0) last = atomicAdd(&counters[pi], 1u) == (unsigned)nb - 1;
     __syncthreads();
     if (!last) return;
     __threadfence();
+    // the problem's blocks in a fixed order
+    double s1 = 0.0, s2 = 0.0;
+    for (int k = col; k < nb; k += kBCols) {
+        s1 += ((volatile const double*)base)[(long long)k * 2 * R + 2 * rh];
+        if (bb) s2 += ((volatile const double*)base)[(long long)k * 2 * R + 2 * rh + 1];
+    }
+    s1 = block_sum_r(s1, red);
+    s2 = bb ? block_sum_r(s2, red) : 0.0;
     if (threadIdx.x < R) {
-        const double* base = partials + (long long)pi * gridDim.x * 2 * R;
-        double s1 = 0.0, s2 = 0.0;
-        for (int k = 0; k < (int)gridDim.x; k++) {
-            s1 += ((volatile const double*)base)[(long long)k * 2 * R + 2 * threadIdx.x];
-            s2 += ((volatile const double*)base)[(long long)k * 2 * R + 2 * threadIdx.x + 1];
-        }
         SysState& sy = sys[(long long)pi * R + threadIdx.x];
         sy.rr = s1;
         if (bb) sy.bb = s2;
@@ -573,7 +586,7 @@ struct Batch {
     unsigned* counters = nullptr;       // count (finest up) + count (product) + count (residual)
     double* part_up = nullptr;          // finest up kernel partials
     double* part_sp = nullptr;          // operator product partials
-    double* part_res = nullptr;         // residual partials (count * kRowBlocks * 2R)
+    double* part_res = nullptr;         // residual partials (count * the largest problem's blocks * 2R)
     double* stage = nullptr;            // host staging (largest n^2 * R doubles)
     PackEnt* ptab = nullptr;            // device: 3 * count pack/unpack entries
     PackEnt* ptab_h = nullptr;          // pinned mirror
@@ -587,6 +600,12 @@ struct Batch {
 };
 
 namespace {
+
+int max_res_blocks(const Batch& B) {
+    int m = 1;
+    for (const BProbDev& P : B.prob_h) m = std::max(m, res_blocks(P.n));
+    return m;
+}
 
 // Walks the workspace layout; with base == nullptr it only measures.
 size_t carve_batch(Batch& B, char* base) {
@@ -640,7 +659,7 @@ size_t carve_batch(Batch& B, char* base) {
     B.counters = (unsigned*)take(sizeof(unsigned) * 3 * B.count);
     B.part_up = (double*)take(sizeof(double) * 2 * R * (parts_up > 0 ? parts_up : 1));
     B.part_sp = (double*)take(sizeof(double) * R * (parts_sp > 0 ? parts_sp : 1));
-    B.part_res = (double*)take(sizeof(double) * 2 * R * kRowBlocks * B.count);
+    B.part_res = (double*)take(sizeof(double) * 2 * R * max_res_blocks(B) * B.count);
     B.stage = (double*)take(sizeof(double) * B.stage_elems);
     B.ptab = (PackEnt*)take(sizeof(PackEnt) * 3 * B.count);
     return a256(off);
@@ -834,7 +853,7 @@ bmg_status run_iteration(Batch& B, int parity) {
 }
 
 bmg_status residual(Batch& B, bool bb) {
-    k_bresidual<<<dim3(kRowBlocks, B.count), kBThreads, 0, B.stream>>>(B.prob_d, B.sys, B.part_res,
+    k_bresidual<<<dim3(max_res_blocks(B), B.count), kBThreads, 0, B.stream>>>(B.prob_d, B.sys, B.part_res,
                                                                        B.counters + 2 * B.count, bb ? 1 : 0);
     B.launches++;
     BMG_CUDA(cudaGetLastError());

@@ -139,6 +139,8 @@ struct Ctx {
     KState* st_host = nullptr;    // pinned mirror
     long long launches = 0;
     int red_blocks = 0;           // fixed grid of the reducing kernels (deterministic)
+    int sms = 0;                  // SMs of the device
+    int nt_h = 0, nt_i = 0, nt_j = 0, nt_tiles = 0;   // node tiles of the FP64 products and residuals
     int spmv_h = 0, spmv_tiles_x = 0, spmv_tiles = 0;   // tiles of the 2-D refinement-mode operator product
     bool prof_on = false;
     ProfSlot prof[BMG_PROF_KINDS];
@@ -223,79 +225,72 @@ struct Sten2 {
     }
 };
 
-// Block-wide sum (blockDim.x == kThreads), result valid in thread 0.
+// Block-wide sum (blockDim.x == kThreads) in a fixed order, valid in lane 0 of
+// warp sum_warp(): one warp adds the other warps' values lane by lane and
+// folds the lanes, 12 FP64 adds, where a shuffle tree in every warp takes 45 of
+// the units' slots.  The warp rotates with the block, so that the blocks of an
+// SM use different schedulers.
+__device__ __forceinline__ int sum_warp() { return blockIdx.x % (kThreads / 32); }
 __device__ __forceinline__ double block_sum(double v) {
-    __shared__ double sh[kThreads / 32];
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
-    int w = threadIdx.x >> 5, l = threadIdx.x & 31;
+    __shared__ double sh[kThreads];
     __syncthreads();
-    if (l == 0) sh[w] = v;
+    sh[threadIdx.x] = v;
     __syncthreads();
     double s = 0.0;
-    if (w == 0) {
-        s = l < kThreads / 32 ? sh[l] : 0.0;
+    if ((int)(threadIdx.x >> 5) == sum_warp()) {
+        const int l = threadIdx.x & 31;
+        s = sh[l];
+#pragma unroll
+        for (int w = 1; w < kThreads / 32; w++) s += sh[l + 32 * w];
         for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
     }
     return s;
 }
 
-// Two sums at once (same scheme as grid_sum; partials holds 2 per block).
-__device__ __forceinline__ bool grid_sum2(double v1, double v2, double* partials, unsigned int* counter,
-                                          double* t1, double* t2) {
-    __shared__ bool last2;
-    double b1 = block_sum(v1);
-    double b2 = block_sum(v2);
-    if (threadIdx.x == 0) {
-        partials[2 * blockIdx.x] = b1;
-        partials[2 * blockIdx.x + 1] = b2;
-        __threadfence();
-        unsigned int t = atomicAdd(counter, 1u);
-        last2 = (t == gridDim.x - 1);
-    }
-    __syncthreads();
-    if (!last2) return false;
-    __threadfence();
-    double s1 = 0.0, s2 = 0.0;
-    for (int k = threadIdx.x; k < (int)gridDim.x; k += blockDim.x) {
-        s1 += ((volatile double*)partials)[2 * k];
-        s2 += ((volatile double*)partials)[2 * k + 1];
-    }
-    s1 = block_sum(s1);
-    s2 = block_sum(s2);
-    if (threadIdx.x == 0) {
-        *counter = 0u;
-        *t1 = s1;
-        *t2 = s2;
-        return true;
-    }
-    return false;
-}
-
-// Deterministic grid reduction: each block stores its partial; the last
-// block to arrive sums the partials in a fixed order.  Returns true (in
-// thread 0 of the last block only) with the total in *total.
-__device__ __forceinline__ bool grid_sum(double v, double* partials, unsigned int* counter,
-                                         double* total) {
+// Deterministic grid reduction of N sums at once: each block stores its
+// partials (N per block); the last block to arrive sums them in a fixed order.
+// Returns true (in one thread of the last block only) with the totals in t.
+template <int N>
+__device__ __forceinline__ bool grid_sum_n(const double (&v)[N], double* partials, unsigned int* counter,
+                                           double (&t)[N]) {
     __shared__ bool last;
-    double b = block_sum(v);
-    if (threadIdx.x == 0) {
-        partials[blockIdx.x] = b;
+    const bool lead = (int)threadIdx.x == 32 * sum_warp();
+    double b[N];
+#pragma unroll
+    for (int q = 0; q < N; q++) b[q] = block_sum(v[q]);
+    if (lead) {
+#pragma unroll
+        for (int q = 0; q < N; q++) partials[N * blockIdx.x + q] = b[q];
         __threadfence();
-        unsigned int t = atomicAdd(counter, 1u);
-        last = (t == gridDim.x - 1);
+        last = atomicAdd(counter, 1u) == gridDim.x - 1;
     }
     __syncthreads();
     if (!last) return false;
     __threadfence();
-    double s = 0.0;
-    for (int k = threadIdx.x; k < (int)gridDim.x; k += blockDim.x) s += ((volatile double*)partials)[k];
-    s = block_sum(s);
-    if (threadIdx.x == 0) {
-        *counter = 0u;
-        *total = s;
-        return true;
+#pragma unroll
+    for (int q = 0; q < N; q++) {
+        double s = 0.0;
+        for (int k = threadIdx.x; k < (int)gridDim.x; k += blockDim.x) s += ((volatile double*)partials)[N * k + q];
+        t[q] = block_sum(s);
     }
-    return false;
+    if (lead) *counter = 0u;
+    return lead;
+}
+
+__device__ __forceinline__ bool grid_sum2(double v1, double v2, double* partials, unsigned int* counter,
+                                          double* t1, double* t2) {
+    double t[2];
+    if (!grid_sum_n<2>({v1, v2}, partials, counter, t)) return false;
+    *t1 = t[0];
+    *t2 = t[1];
+    return true;
+}
+
+__device__ __forceinline__ bool grid_sum(double v, double* partials, unsigned int* counter, double* total) {
+    double t[1];
+    if (!grid_sum_n<1>({v}, partials, counter, t)) return false;
+    *total = t[0];
+    return true;
 }
 
 // ------------------------------------------------------------------ host launchers
@@ -408,6 +403,7 @@ bmg_status k_row_sums32(Ctx& c);                // rs32 = row sums of A (compute
 bmg_status k_residual_to32(Ctx& c);             // r32 = (float)(b - A x); rr; resets the inner CG state
 bmg_status k_rz_beta32(Ctx& c, const float* z, const float* zo);
 bmg_status k_update_dr32(Ctx& c, int parity);    // x (FP64) += alpha p; r32 -= alpha q
+bmg_status node_tiles_prepare(Ctx& c);           // tile shape of the FP64 products and residuals
 bmg_status pspmv_prepare(Ctx& c);                // tile shape of the 2-D operator product
 bmg_status k_pspmv32(Ctx& c, const float* z, int parity);   // p = z + beta p_old; q = A p; alpha
 

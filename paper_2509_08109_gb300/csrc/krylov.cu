@@ -63,16 +63,14 @@ __device__ __forceinline__ bool row_x_zero(const T* __restrict__ x, int ld, int 
         return sizeof(T) == 8 ? (unsigned long long)__double_as_longlong((double)v) << 1
                               : (unsigned long long)__float_as_uint((float)v) << 1;
     };
-    unsigned long long m = bits(x[o]);
-    if (DIM == 2) {
-        m |= bits(x[o - 1]) | bits(x[o + 1]) | bits(x[o - ld]) | bits(x[o + ld]);
-        m |= bits(x[o - ld - 1]) | bits(x[o + ld + 1]) | bits(x[o + ld - 1]) | bits(x[o - ld + 1]);
-    } else {
-#pragma unroll
-        for (int t = 0; t < 13; t++) {
-            const long long d = d3(t, ld, n);
-            m |= bits(x[o + d]) | bits(x[o - d]);
-        }
+    unsigned long long m = 0;
+    // row by row and not unrolled: holding the neighbourhood in registers for
+    // the products that follow costs more occupancy than reading it again
+    const int rows = DIM == 2 ? 3 : 9;
+#pragma unroll 1
+    for (int q = 0; q < rows && m == 0; q++) {
+        const T* r = x + o + (long long)ld * ((q % 3 - 1) + (DIM == 2 ? 0LL : (long long)n * (q / 3 - 1)));
+        m = bits(r[-1]) | bits(r[0]) | bits(r[1]);
     }
     return m == 0;
 }
@@ -132,6 +130,36 @@ struct Acc32 {
     for (int r_ = blockIdx.x; r_ < (g).rows(); r_ += gridDim.x)           \
         for (int i_ = threadIdx.x; i_ < (g).ld; i_ += blockDim.x)
 
+// Interior nodes in tiles of 32 columns x 8 rows, H steps of a tile per CTA
+// (2-D: the next 8 rows; 3-D: the next plane).  A row-strided loop left up to
+// 40% of the FP64 lanes idle (127 interior columns on 160 padded ones and 256
+// threads), and FP64 lanes are what bounds the products below.  Boundary and
+// padding entries are zero in every array and stay as they are.
+template <int DIM>
+struct NodeTiles {
+    int n, ld, H, ti, tj;
+    template <class F>
+    __device__ __forceinline__ void each(F&& f) const {
+        const int t = (int)blockIdx.x;
+        const int i = 1 + 32 * (t % ti) + (int)(threadIdx.x & 31);
+        const int ty = (int)(threadIdx.x >> 5);
+        if (i > n - 2) return;
+        if (DIM == 2) {
+            const int j0 = 1 + 8 * H * (t / ti) + ty;
+            for (int s = 0; s < H; s++) {
+                const int j = j0 + 8 * s;
+                if (j > n - 2) break;
+                f((long long)j * ld + i);
+            }
+        } else {
+            const int j = 1 + 8 * (t / ti % tj) + ty;
+            if (j > n - 2) return;
+            const int k0 = 1 + H * (t / (ti * tj));
+            for (int k = k0; k < k0 + H && k <= n - 2; k++) f((long long)i + (long long)ld * (j + (long long)n * k));
+        }
+    }
+};
+
 // ---------------------------------------------------------------- layout
 template <int DIM>
 __global__ void k_pack_t(int n, int ld, const double* __restrict__ src, double* __restrict__ dst) {
@@ -153,43 +181,50 @@ __global__ void k_unpack_t(int n, int ld, const double* __restrict__ src, double
 // ---------------------------------------------------------------- FP64 outer CG
 // r = b - A x ; st.rr = ||r||^2 (rows with a zero x neighbourhood: r = b)
 template <int DIM>
-__global__ void k_residual64(RowGrid<DIM> g, const double* __restrict__ A, long long pl, const double* __restrict__ b,
-                             const double* __restrict__ x, double* __restrict__ r, double* partials, KState* st) {
+__global__ void __launch_bounds__(kThreads) k_residual64(NodeTiles<DIM> g, const double* __restrict__ A, long long pl,
+                                                         const double* __restrict__ b, const double* __restrict__ x,
+                                                         double* __restrict__ r, double* partials, KState* st) {
     double acc = 0.0;
-    FOR_ROWS(g) {
-        const long long k = (long long)r_ * g.ld + i_;
-        double v = 0.0;
-        if (g.row_inner(r_) && i_ >= 1 && i_ <= g.n - 2)
-            v = row_x_zero<DIM, double>(x, g.ld, g.n, k) ? b[k] : b[k] - apply_row<DIM, double>(A, pl, g.ld, g.n, x, k);
+    g.each([&](long long k) {
+        const double v =
+            row_x_zero<DIM, double>(x, g.ld, g.n, k) ? b[k] : b[k] - apply_row<DIM, double>(A, pl, g.ld, g.n, x, k);
         r[k] = v;
         acc += v * v;
-    }
+    });
     double t;
     if (grid_sum(acc, partials, &st->counter[0], &t)) st->rr = t;
 }
 
-__global__ void k_dot64(long long tot, const double* __restrict__ a, const double* __restrict__ b, double* partials,
-                        KState* st, double* slot) {
+// The vector kernels below read pairs (planes hold a multiple of 32 values)
+// on four CTAs per SM: every CTA's sum costs FP64 slots of its own, and with
+// eight per SM, a shuffle tree in every warp, those took as long as the
+// vectors (1025^2: r.z 17.5 us, update 16.4 us; now 11.4
+// and 14.7 us).
+__global__ void __launch_bounds__(kThreads) k_dot64(long long pairs, const double2* __restrict__ a,
+                                                    const double2* __restrict__ b, double* partials, KState* st,
+                                                    double* slot) {
     double acc = 0.0;
-    for (long long k = blockIdx.x * (long long)blockDim.x + threadIdx.x; k < tot;
-         k += (long long)gridDim.x * blockDim.x)
-        acc += a[k] * b[k];
+    for (long long k = blockIdx.x * (long long)blockDim.x + threadIdx.x; k < pairs;
+         k += (long long)gridDim.x * blockDim.x) {
+        const double2 u = a[k], v = b[k];
+        acc += u.x * v.x;
+        acc += u.y * v.y;
+    }
     double t;
     if (grid_sum(acc, partials, &st->counter[1], &t)) *slot = t;
 }
 
 // q = A p; st.pq = p.q; alpha = rz / pq
 template <int DIM>
-__global__ void k_spmv_pq64(RowGrid<DIM> g, const double* __restrict__ A, long long pl, const double* __restrict__ p,
-                            double* __restrict__ q, double* partials, KState* st) {
+__global__ void __launch_bounds__(kThreads) k_spmv_pq64(NodeTiles<DIM> g, const double* __restrict__ A, long long pl,
+                                                        const double* __restrict__ p, double* __restrict__ q,
+                                                        double* partials, KState* st) {
     double acc = 0.0;
-    FOR_ROWS(g) {
-        const long long k = (long long)r_ * g.ld + i_;
-        double v = 0.0;
-        if (g.row_inner(r_) && i_ >= 1 && i_ <= g.n - 2) v = apply_row<DIM, double>(A, pl, g.ld, g.n, p, k);
+    g.each([&](long long k) {
+        const double v = apply_row<DIM, double>(A, pl, g.ld, g.n, p, k);
         q[k] = v;
         acc += p[k] * v;
-    }
+    });
     double t;
     if (grid_sum(acc, partials, &st->counter[2], &t)) {
         st->pq = t;
@@ -203,17 +238,24 @@ __global__ void k_spmv_pq64(RowGrid<DIM> g, const double* __restrict__ A, long l
 }
 
 // x += alpha p; r -= alpha q; st.rr = ||r||^2
-__global__ void k_update_xr64(long long tot, double* __restrict__ x, double* __restrict__ r,
-                              const double* __restrict__ p, const double* __restrict__ q, double* partials,
-                              KState* st) {
+__global__ void __launch_bounds__(kThreads) k_update_xr64(long long pairs, double2* __restrict__ x,
+                                                          double2* __restrict__ r, const double2* __restrict__ p,
+                                                          const double2* __restrict__ q, double* partials,
+                                                          KState* st) {
     const double alpha = st->alpha;
     double acc = 0.0;
-    for (long long k = blockIdx.x * (long long)blockDim.x + threadIdx.x; k < tot;
+    for (long long k = blockIdx.x * (long long)blockDim.x + threadIdx.x; k < pairs;
          k += (long long)gridDim.x * blockDim.x) {
-        x[k] += alpha * p[k];
-        const double rv = r[k] - alpha * q[k];
+        double2 xv = x[k], rv = r[k];
+        const double2 pv = p[k], qv = q[k];
+        xv.x += alpha * pv.x;
+        xv.y += alpha * pv.y;
+        rv.x -= alpha * qv.x;
+        rv.y -= alpha * qv.y;
+        x[k] = xv;
         r[k] = rv;
-        acc += rv * rv;
+        acc += rv.x * rv.x;
+        acc += rv.y * rv.y;
     }
     double t;
     if (grid_sum(acc, partials, &st->counter[3], &t)) st->rr = t;
@@ -221,33 +263,49 @@ __global__ void k_update_xr64(long long tot, double* __restrict__ x, double* __r
 
 // r.z and (flexible) r.z_old in one pass, then beta in the last block; the
 // first iteration has no beta.
-__global__ void k_rz_beta64(long long tot, const double* __restrict__ r, const double* __restrict__ z,
-                            const double* __restrict__ zo, int flexible, double* partials, KState* st) {
+template <bool FLEX>
+__global__ void __launch_bounds__(kThreads) k_rz_beta64(long long pairs, const double2* __restrict__ r,
+                                                        const double2* __restrict__ z,
+                                                        const double2* __restrict__ zo, double* partials,
+                                                        KState* st) {
     double a1 = 0.0, a2 = 0.0;
-    for (long long k = blockIdx.x * (long long)blockDim.x + threadIdx.x; k < tot;
+    for (long long k = blockIdx.x * (long long)blockDim.x + threadIdx.x; k < pairs;
          k += (long long)gridDim.x * blockDim.x) {
-        const double rv = r[k];
-        a1 += rv * z[k];
-        if (flexible) a2 += rv * zo[k];
+        const double2 rv = r[k], zv = z[k];
+        a1 += rv.x * zv.x;
+        a1 += rv.y * zv.y;
+        if (FLEX) {
+            const double2 ov = zo[k];
+            a2 += rv.x * ov.x;
+            a2 += rv.y * ov.y;
+        }
     }
-    double t1, t2;
-    if (grid_sum2(a1, a2, partials, &st->counter[5], &t1, &t2)) {
+    double t1 = 0.0, t2 = 0.0;
+    const bool lead = FLEX ? grid_sum2(a1, a2, partials, &st->counter[5], &t1, &t2)
+                           : grid_sum(a1, partials, &st->counter[5], &t1);
+    if (lead) {
         if (st->first) {
             st->beta = 0.0;
             st->first = 0;
         } else {
-            st->beta = (flexible ? t1 - t2 : t1) / st->rz;
+            st->beta = (FLEX ? t1 - t2 : t1) / st->rz;
         }
         st->rz = t1;
     }
 }
 
 // p = z + beta p
-__global__ void k_p_update64(long long tot, const double* __restrict__ z, double* __restrict__ p, KState* st) {
+__global__ void __launch_bounds__(kThreads) k_p_update64(long long pairs, const double2* __restrict__ z,
+                                                         double2* __restrict__ p, KState* st) {
     const double beta = st->beta;
-    for (long long k = blockIdx.x * (long long)blockDim.x + threadIdx.x; k < tot;
-         k += (long long)gridDim.x * blockDim.x)
-        p[k] = z[k] + beta * p[k];
+    for (long long k = blockIdx.x * (long long)blockDim.x + threadIdx.x; k < pairs;
+         k += (long long)gridDim.x * blockDim.x) {
+        const double2 zv = z[k];
+        double2 pv = p[k];
+        pv.x = zv.x + beta * pv.x;
+        pv.y = zv.y + beta * pv.y;
+        p[k] = pv;
+    }
 }
 
 // ---------------------------------------------------------------- refinement (FP32 inner CG)
@@ -255,18 +313,17 @@ __global__ void k_p_update64(long long tot, const double* __restrict__ z, double
 // Rows whose x neighbourhood is zero take r = b without the FP64 products
 // (the FP64 rate, not HBM, bounds this kernel otherwise).
 template <int DIM>
-__global__ void k_residual_to32_t(RowGrid<DIM> g, const double* __restrict__ A, long long pl,
-                                  const double* __restrict__ b, const double* __restrict__ x,
-                                  float* __restrict__ r32, double* partials, KState* st) {
+__global__ void __launch_bounds__(kThreads) k_residual_to32_t(NodeTiles<DIM> g, const double* __restrict__ A,
+                                                              long long pl, const double* __restrict__ b,
+                                                              const double* __restrict__ x, float* __restrict__ r32,
+                                                              double* partials, KState* st) {
     double acc = 0.0;
-    FOR_ROWS(g) {
-        const long long k = (long long)r_ * g.ld + i_;
-        double v = 0.0;
-        if (g.row_inner(r_) && i_ >= 1 && i_ <= g.n - 2)
-            v = row_x_zero<DIM, double>(x, g.ld, g.n, k) ? b[k] : b[k] - apply_row<DIM, double>(A, pl, g.ld, g.n, x, k);
+    g.each([&](long long k) {
+        const double v =
+            row_x_zero<DIM, double>(x, g.ld, g.n, k) ? b[k] : b[k] - apply_row<DIM, double>(A, pl, g.ld, g.n, x, k);
         r32[k] = (float)v;
         acc += v * v;
-    }
+    });
     double t;
     if (grid_sum(acc, partials, &st->counter[0], &t)) {
         st->rr = t;
@@ -339,26 +396,48 @@ __global__ void k_pspmv32_t(RowGrid<DIM> g, const float* __restrict__ A, const f
 // x += alpha p straight into the FP64 iterate (an FP32 correction would cap
 // the true residual near eps_32 ||A|| ||d|| / ||A d||, far above 1e-10 for a
 // smooth correction d); r -= alpha q in FP32.
-__global__ void k_update_xr32(long long tot, double* __restrict__ x, float* __restrict__ r,
-                              const float* __restrict__ p, const float* __restrict__ q, const KState* st) {
+__global__ void __launch_bounds__(kThreads) k_update_xr32(long long quads, double2* __restrict__ x,
+                                                          float4* __restrict__ r, const float4* __restrict__ p,
+                                                          const float4* __restrict__ q, const KState* st) {
     const double alpha = st->alpha;
     const float a32 = (float)alpha;
-    for (long long k = blockIdx.x * (long long)blockDim.x + threadIdx.x; k < tot;
+    for (long long k = blockIdx.x * (long long)blockDim.x + threadIdx.x; k < quads;
          k += (long long)gridDim.x * blockDim.x) {
-        x[k] += alpha * (double)p[k];
-        r[k] -= a32 * q[k];
+        const float4 pv = p[k], qv = q[k];
+        float4 rv = r[k];
+        double2 x0 = x[2 * k], x1 = x[2 * k + 1];
+        x0.x += alpha * (double)pv.x;
+        x0.y += alpha * (double)pv.y;
+        x1.x += alpha * (double)pv.z;
+        x1.y += alpha * (double)pv.w;
+        rv.x -= a32 * qv.x;
+        rv.y -= a32 * qv.y;
+        rv.z -= a32 * qv.z;
+        rv.w -= a32 * qv.w;
+        x[2 * k] = x0;
+        x[2 * k + 1] = x1;
+        r[k] = rv;
     }
 }
 
-// r.z and r.z_old in one pass; the last block forms the flexible-CG beta
-__global__ void k_rz_beta32_t(long long tot, const float* __restrict__ r, const float* __restrict__ z,
-                              const float* __restrict__ zo, double* partials, KState* st) {
+// r.z and r.z_old in one pass; the last block forms the flexible-CG beta.
+// Four values a load, two CTAs per SM (as the FP64 vector kernels).
+__global__ void __launch_bounds__(kThreads) k_rz_beta32_t(long long quads, const float4* __restrict__ r,
+                                                          const float4* __restrict__ z,
+                                                          const float4* __restrict__ zo, double* partials,
+                                                          KState* st) {
     Acc32 a1, a2;
-    for (long long k = blockIdx.x * (long long)blockDim.x + threadIdx.x; k < tot;
+    for (long long k = blockIdx.x * (long long)blockDim.x + threadIdx.x; k < quads;
          k += (long long)gridDim.x * blockDim.x) {
-        const float rv = r[k];
-        a1.add(rv * z[k]);
-        a2.add(rv * zo[k]);
+        const float4 rv = r[k], zv = z[k], ov = zo[k];
+        a1.add(rv.x * zv.x);
+        a2.add(rv.x * ov.x);
+        a1.add(rv.y * zv.y);
+        a2.add(rv.y * ov.y);
+        a1.add(rv.z * zv.z);
+        a2.add(rv.z * ov.z);
+        a1.add(rv.w * zv.w);
+        a2.add(rv.w * ov.w);
     }
     double t1, t2;
     if (grid_sum2(a1.value(), a2.value(), partials, &st->counter[4], &t1, &t2)) {
@@ -387,7 +466,51 @@ inline double dofs0(const Ctx& c) {
         (c).launches++;                                                                                   \
     } while (0)
 
+// The same for the node-tile kernels.
+#define DISPATCH_TILES(c, KERNEL, ...)                                                                     \
+    do {                                                                                                   \
+        const Level& L_ = (c).lev[0];                                                                      \
+        if ((c).dim == 2)                                                                                  \
+            KERNEL<2><<<(c).nt_tiles, kThreads, 0, (c).stream>>>(                                          \
+                NodeTiles<2>{L_.n, L_.ld, (c).nt_h, (c).nt_i, (c).nt_j}, __VA_ARGS__);                     \
+        else                                                                                               \
+            KERNEL<3><<<(c).nt_tiles, kThreads, 0, (c).stream>>>(                                          \
+                NodeTiles<3>{L_.n, L_.ld, (c).nt_h, (c).nt_i, (c).nt_j}, __VA_ARGS__);                     \
+        (c).launches++;                                                                                    \
+    } while (0)
+
+// CTAs of the reducing vector kernels: four per SM, fewer where a CTA would
+// get less than two pairs a thread.
+inline int vec_blocks(const Ctx& c) {
+    const int want = cdiv(c.lev[0].plane / 2, 2 * kThreads);
+    return want < 4 * c.sms ? want : 4 * c.sms;
+}
+
 }  // namespace
+
+// Steps per tile of the node-tile kernels: the CTAs of an SM share its FP64
+// units, so minimise CTAs per SM x steps (each CTA's reduction counted as
+// one more), within the partials' buffer.
+bmg_status node_tiles_prepare(Ctx& c) {
+    BMG_CUDA(cudaDeviceGetAttribute(&c.sms, cudaDevAttrMultiProcessorCount, c.device));
+    const int m = c.lev[0].n - 2;
+    const int ti = cdiv(m, 32), tj = cdiv(m, 8), steps = c.dim == 2 ? tj : m;
+    const long long cols = c.dim == 2 ? ti : (long long)ti * tj;
+    long long best = -1;
+    for (int h = 1; h <= steps; h++) {
+        const long long tiles = cols * cdiv(steps, h);
+        if (tiles > kMaxBlocks) continue;
+        const long long cost = (long long)cdiv(tiles, c.sms) * (h + 1);
+        if (best < 0 || cost < best) {
+            best = cost;
+            c.nt_h = h;
+            c.nt_tiles = (int)tiles;
+        }
+    }
+    c.nt_i = ti;
+    c.nt_j = tj;
+    return best < 0 ? BMG_ERR_SHAPE : BMG_OK;
+}
 
 bmg_status k_pack(Ctx& c, const double* src, double* dst) {
     const Level& L = c.lev[0];
@@ -413,14 +536,15 @@ bmg_status k_unpack(Ctx& c, const double* src, double* dst) {
 
 bmg_status k_residual(Ctx& c, const double* b, const double* x, double* r) {
     const Level& L = c.lev[0];
-    DISPATCH_DIM(c, k_residual64, L.A64, L.plane, b, x, r, c.partials, c.st);
+    DISPATCH_TILES(c, k_residual64, L.A64, L.plane, b, x, r, c.partials, c.st);
     BMG_CUDA(cudaGetLastError());
     return BMG_OK;
 }
 
 bmg_status k_dot(Ctx& c, const double* a, const double* b, double* slot) {
     const Level& L = c.lev[0];
-    k_dot64<<<c.red_blocks, kThreads, 0, c.stream>>>(L.plane, a, b, c.partials, c.st, slot);
+    k_dot64<<<vec_blocks(c), kThreads, 0, c.stream>>>(L.plane / 2, (const double2*)a, (const double2*)b, c.partials, c.st,
+                                                      slot);
     c.launches++;
     BMG_CUDA(cudaGetLastError());
     return BMG_OK;
@@ -429,7 +553,7 @@ bmg_status k_dot(Ctx& c, const double* a, const double* b, double* slot) {
 bmg_status k_spmv_pq(Ctx& c, const double* p, double* q) {
     const Level& L = c.lev[0];
     prof_begin(c, BMG_PROF_SPMV, 0);
-    DISPATCH_DIM(c, k_spmv_pq64, L.A64, L.plane, p, q, c.partials, c.st);
+    DISPATCH_TILES(c, k_spmv_pq64, L.A64, L.plane, p, q, c.partials, c.st);
     prof_end(c, BMG_PROF_SPMV, 0, (c.ns + 2) * 8.0 * dofs0(c));
     BMG_CUDA(cudaGetLastError());
     return BMG_OK;
@@ -438,7 +562,9 @@ bmg_status k_spmv_pq(Ctx& c, const double* p, double* q) {
 bmg_status k_update_xr(Ctx& c) {
     const Level& L = c.lev[0];
     prof_begin(c, BMG_PROF_UPDATE, 0);
-    k_update_xr64<<<c.red_blocks, kThreads, 0, c.stream>>>(L.plane, c.x, c.r, c.p, c.q, c.partials, c.st);
+    k_update_xr64<<<vec_blocks(c), kThreads, 0, c.stream>>>(L.plane / 2, (double2*)c.x, (double2*)c.r,
+                                                            (const double2*)c.p, (const double2*)c.q, c.partials,
+                                                            c.st);
     prof_end(c, BMG_PROF_UPDATE, 0, 6 * 8.0 * dofs0(c));
     c.launches++;
     BMG_CUDA(cudaGetLastError());
@@ -447,7 +573,11 @@ bmg_status k_update_xr(Ctx& c) {
 
 bmg_status k_rz_beta(Ctx& c, const double* z, const double* zold, bool flexible) {
     const Level& L = c.lev[0];
-    k_rz_beta64<<<c.red_blocks, kThreads, 0, c.stream>>>(L.plane, c.r, z, zold, flexible ? 1 : 0, c.partials, c.st);
+    const double2 *r2 = (const double2*)c.r, *z2 = (const double2*)z, *o2 = (const double2*)zold;
+    if (flexible)
+        k_rz_beta64<true><<<vec_blocks(c), kThreads, 0, c.stream>>>(L.plane / 2, r2, z2, o2, c.partials, c.st);
+    else
+        k_rz_beta64<false><<<vec_blocks(c), kThreads, 0, c.stream>>>(L.plane / 2, r2, z2, o2, c.partials, c.st);
     c.launches++;
     BMG_CUDA(cudaGetLastError());
     return BMG_OK;
@@ -455,7 +585,9 @@ bmg_status k_rz_beta(Ctx& c, const double* z, const double* zold, bool flexible)
 
 bmg_status k_p_update(Ctx& c, const double* z) {
     const Level& L = c.lev[0];
-    k_p_update64<<<c.red_blocks, kThreads, 0, c.stream>>>(L.plane, z, c.p, c.st);
+    const int blocks = cdiv(L.plane / 2, 2 * kThreads);
+    k_p_update64<<<blocks < c.red_blocks ? blocks : c.red_blocks, kThreads, 0, c.stream>>>(
+        L.plane / 2, (const double2*)z, (double2*)c.p, c.st);
     c.launches++;
     BMG_CUDA(cudaGetLastError());
     return BMG_OK;
@@ -463,7 +595,7 @@ bmg_status k_p_update(Ctx& c, const double* z) {
 
 bmg_status k_residual_to32(Ctx& c) {
     const Level& L = c.lev[0];
-    DISPATCH_DIM(c, k_residual_to32_t, L.A64, L.plane, c.bvec, c.x, c.r32, c.partials, c.st);
+    DISPATCH_TILES(c, k_residual_to32_t, L.A64, L.plane, c.bvec, c.x, c.r32, c.partials, c.st);
     BMG_CUDA(cudaGetLastError());
     return BMG_OK;
 }
@@ -594,7 +726,8 @@ bmg_status k_row_sums32(Ctx& c) {
 
 bmg_status k_rz_beta32(Ctx& c, const float* z, const float* zo) {
     const Level& L = c.lev[0];
-    k_rz_beta32_t<<<c.red_blocks, kThreads, 0, c.stream>>>(L.plane, c.r32, z, zo, c.partials, c.st);
+    k_rz_beta32_t<<<vec_blocks(c), kThreads, 0, c.stream>>>(L.plane / 4, (const float4*)c.r32, (const float4*)z,
+                                                            (const float4*)zo, c.partials, c.st);
     c.launches++;
     BMG_CUDA(cudaGetLastError());
     return BMG_OK;
@@ -785,7 +918,9 @@ bmg_status k_pspmv32(Ctx& c, const float* z, int parity) {
 bmg_status k_update_dr32(Ctx& c, int parity) {
     const Level& L = c.lev[0];
     prof_begin(c, BMG_PROF_UPDATE, 0);
-    k_update_xr32<<<c.red_blocks, kThreads, 0, c.stream>>>(L.plane, c.x, c.r32, c.p32s[parity], c.q32, c.st);
+    const int blocks = cdiv(L.plane / 4, kThreads);
+    k_update_xr32<<<blocks < 8 * c.sms ? blocks : 8 * c.sms, kThreads, 0, c.stream>>>(
+        L.plane / 4, (double2*)c.x, (float4*)c.r32, (const float4*)c.p32s[parity], (const float4*)c.q32, c.st);
     prof_end(c, BMG_PROF_UPDATE, 0, (4 * 4.0 + 2 * 8.0) * dofs0(c));
     c.launches++;
     BMG_CUDA(cudaGetLastError());
