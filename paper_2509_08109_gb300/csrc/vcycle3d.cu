@@ -101,6 +101,26 @@ __device__ __forceinline__ V2<T> ld2(const T* p) {
     }
 }
 
+// the same without the read-only path (arrays another kernel has just written
+// while this one was coming up), and the store
+template <typename T>
+__device__ __forceinline__ V2<T> ld2c(const T* p) {
+    if constexpr (sizeof(T) == 4) {
+        const float2 v = *reinterpret_cast<const float2*>(p);
+        return {v.x, v.y};
+    } else {
+        const double2 v = *reinterpret_cast<const double2*>(p);
+        return {v.x, v.y};
+    }
+}
+template <typename T>
+__device__ __forceinline__ void st2(T* p, T a, T b) {
+    if constexpr (sizeof(T) == 4)
+        *reinterpret_cast<float2*>(p) = make_float2(a, b);
+    else
+        *reinterpret_cast<double2*>(p) = make_double2(a, b);
+}
+
 // mask of the non-zero components of offset t: the neighbour at offset t (or
 // -t) of a point of colour col has colour col ^ mask
 __host__ __device__ constexpr int off_mask(int t) { return (t % 3 != 1) | ((t / 3 % 3 != 1) << 1) | ((t / 9 != 1) << 2); }
@@ -115,8 +135,7 @@ __host__ __device__ constexpr int off_mask(int t) { return (t % 3 != 1) | ((t / 
 // the time of its 60 bytes a node at the copy rate (225 before); 129^3 FP64:
 // 56 us.
 template <typename T, int JODD, int KODD>
-__device__ __forceinline__ void residual3d_pair(const L3<T>& L, const T* __restrict__ x, T* __restrict__ r, int i,
-                                                long long o) {
+__device__ __forceinline__ void residual3d_pair(const L3<T>& L, const T* x, int i, long long o, T& r0, T& r1) {
     constexpr int c0 = 2 * JODD + 4 * KODD, c1 = c0 + 1;
     const long long sy = L.ld, sz = (long long)L.ld * L.n;
     T X[3][3][4];      // [dz + 1][dy + 1]: columns i - 1 .. i + 2
@@ -126,11 +145,11 @@ __device__ __forceinline__ void residual3d_pair(const L3<T>& L, const T* __restr
         for (int y = 0; y < 3; y++) {
             if (KODD && z != 1) continue;
             const T* q = x + o + (y - 1) * sy + (z - 1) * sz;
-            const V2<T> v = ld2(q);
-            X[z][y][0] = i > 0 ? __ldg(q - 1) : (T)0;
+            const V2<T> v = ld2c(q);
+            X[z][y][0] = i > 0 ? q[-1] : (T)0;
             X[z][y][1] = v.x;
             X[z][y][2] = v.y;
-            X[z][y][3] = __ldg(q + 2);
+            X[z][y][3] = q[2];
         }
     T s0 = 0, s1 = 0;
 #pragma unroll
@@ -150,27 +169,32 @@ __device__ __forceinline__ void residual3d_pair(const L3<T>& L, const T* __restr
             s1 += (dx == 0 ? m.y : dx < 0 ? __ldg(b + 2) : m.x) * X[1 - dz][1 - dy][2 - dx];
         }
     }
-    if (i > 0) r[o] = -s0;
-    r[o + 1] = -s1;
+    r0 = -s0;
+    r1 = -s1;
 }
 
 template <typename T>
-__global__ void __launch_bounds__(64) k_residual3d_sweep(L3<T> L, const T* __restrict__ x, T* __restrict__ r) {
+__global__ void __launch_bounds__(64) k_residual3d_sweep(L3<T> L, const T* x, T* __restrict__ r) {
+    pdl_wait();
+    pdl_trigger();
     const int i = 2 * (blockIdx.x * blockDim.x + threadIdx.x);
     const int j = 1 + blockIdx.y, k = 1 + blockIdx.z;      // interior rows and planes
     if (i + 1 > L.n - 2) return;
     const long long o = L.idx(i, j, k);
+    T r0, r1;
     if (k & 1) {
         if (j & 1)
-            residual3d_pair<T, 1, 1>(L, x, r, i, o);
+            residual3d_pair<T, 1, 1>(L, x, i, o, r0, r1);
         else
-            residual3d_pair<T, 0, 1>(L, x, r, i, o);
+            residual3d_pair<T, 0, 1>(L, x, i, o, r0, r1);
     } else {
         if (j & 1)
-            residual3d_pair<T, 1, 0>(L, x, r, i, o);
+            residual3d_pair<T, 1, 0>(L, x, i, o, r0, r1);
         else
-            residual3d_pair<T, 0, 0>(L, x, r, i, o);
+            residual3d_pair<T, 0, 0>(L, x, i, o, r0, r1);
     }
+    if (i > 0) r[o] = r0;
+    r[o + 1] = r1;
 }
 
 // b_c(K) = sum over the 27 fine neighbours f = 2K + d of P(f, K) r_f, in the
@@ -182,7 +206,7 @@ __global__ void __launch_bounds__(64) k_residual3d_sweep(L3<T> L, const T* __res
 // ldv: row length of the coarse vector bc (ldc, that of the weight planes,
 // unless the coarse level lives in another layout).
 template <typename T>
-__device__ __forceinline__ void restrict_node3d(int nf, int ldf, const T* __restrict__ r, const T* __restrict__ P,
+__device__ __forceinline__ void restrict_node3d(int nf, int ldf, const T* r, const T* __restrict__ P,
                                                 int nc, int ldc, long long plc, T* __restrict__ bc, int ldv, int I,
                                                 int J, int K) {
     const long long oc = (long long)I + (long long)ldc * (J + (long long)nc * K);
@@ -204,8 +228,10 @@ __device__ __forceinline__ void restrict_node3d(int nf, int ldf, const T* __rest
 }
 
 template <typename T>
-__global__ void k_restrict3d(int nf, int ldf, const T* __restrict__ r, const T* __restrict__ P, int nc, int ldc,
+__global__ void k_restrict3d(int nf, int ldf, const T* r, const T* __restrict__ P, int nc, int ldc,
                              long long plc, T* __restrict__ bc) {
+    pdl_wait();
+    pdl_trigger();
     const int I = blockIdx.x * blockDim.x + threadIdx.x;
     const int J = blockIdx.y, K = blockIdx.z;
     if (I < 1 || J < 1 || K < 1 || I > nc - 2 || J > nc - 2 || K > nc - 2) return;
@@ -220,7 +246,7 @@ __global__ void k_restrict3d(int nf, int ldf, const T* __restrict__ r, const T* 
 // ldv: row length of the coarse vector xc (as in restrict_node3d).
 template <typename T>
 __device__ __forceinline__ void prolong_node3d(int nf, int ldf, T* __restrict__ x, const T* __restrict__ P, int nc,
-                                               int ldc, long long plc, const T* __restrict__ xc, int ldv, int I,
+                                               int ldc, long long plc, const T* xc, int ldv, int I,
                                                int J, int K) {
     const long long oc = (long long)I + (long long)ldc * (J + (long long)nc * K);
     const long long ov = (long long)I + (long long)ldv * (J + (long long)nc * K);
@@ -268,14 +294,19 @@ inline dim3 g3(int ni, int nj, int nk) { return dim3(cdiv(ni, 64), nj, nk); }
 // operators and weights do not change between V-cycles: bmg_setup packs them
 // once into the shared-memory image, which a launch stages with bulk copies.
 // A barrier separates the colours, and a phase's time is the chain of one
-// thread's products (64 cycles each in FP64), so:
-//   - the diagonals are packed as reciprocals;
+// thread's instructions, of which a level of a few hundred points leaves
+// nothing else to run meanwhile.  So:
+//   - the diagonals are packed as reciprocals, and the coarsest unknown's
+//     reciprocal is formed while the level above still runs;
 //   - the forward sweep from the zero guess takes only the couplings to
 //     earlier colours, and the residual after it only those to later colours;
-//   - two lanes share a point, each summing half of its couplings;
-//   - prolongation runs one thread per fine point.
-// Measured per V-cycle: FP64 206 -> 55 us (it started at 17^3, in global
-// memory), FP32 42 -> 27 us.
+//   - eight lanes share a point, each with at most two offsets and their
+//     mirrors (FP64 at 9^3, where a colour's 64 points keep the FP64 units
+//     busy: two lanes, the stored couplings and the mirrors);
+//   - eight lanes share a coarse node of the restriction, and prolongation
+//     runs one thread per fine point, all of one parity class in a warp.
+// Measured per V-cycle: FP64 206 -> 54 us (it started at 17^3, in global
+// memory), FP32 42 -> 25.5 us.
 constexpr int kTail3Threads = 512;
 constexpr int kTail3MaxN = 9;    // first tail level: n <= this
 constexpr int kTail3Lev = 3;     // levels of a tail: 9, 5, 3 at most
@@ -321,35 +352,77 @@ struct T3 {
     T *A, *P, *b, *x, *r;
 };
 
+// lanes per point of a colour phase
+template <typename T>
+__device__ __forceinline__ int tail3_lanes(int n) { return sizeof(T) == 8 && n > 5 ? 2 : 8; }
+
+// this thread's share of a point's couplings with eight lanes: offsets
+// lane and lane + 8 (none where that is not below 13)
+struct T3Lane {
+    int da, db, pa, pb;   // index distance and plane offset
+    int ma, mb;           // parity masks; 0: no offset
+};
+__device__ __forceinline__ T3Lane tail3_lane(int n, int tid) {
+    const int a = tid & 7, b = a + 8, n3 = n * n * n;
+    T3Lane q;
+    q.da = off_x(a) + n * (off_y(a) + n * off_z(a));
+    q.db = off_x(b) + n * (off_y(b) + n * off_z(b));
+    q.pa = a * n3;
+    q.pb = b * n3;
+    q.ma = off_mask(a);
+    q.mb = b < 13 ? off_mask(b) : 0;
+    return q;
+}
+
 // One colour: sel < 0: forward Gauss-Seidel update from the zero guess (the
 // couplings to earlier colours); sel == 0: reverse update (all); sel > 0: the
 // residual after the forward sweep into r (those to later colours).  The
 // colour is a run-time value, uniform over the CTA: unrolled per colour the
 // code outran the instruction cache (FP32 tail 72 us instead of 42).
 template <typename T>
-__device__ __forceinline__ void tail3_colour(const T3<T>& v, int col, int sel, int tid) {
+__device__ __forceinline__ void tail3_colour(const T3<T>& v, const T3Lane& ln, int col, int sel, int tid) {
     const int n = v.n, n3 = n * n * n;
     const int pi = col & 1, pj = (col >> 1) & 1, pk = col >> 2;
     // n = 2^k + 1: walk 2^(k-1) points a side and leave out the even
     // coordinates' last one, so that positions are shifts and masks
     const int lg = 31 - __clz(n - 1) - 1, m = 1 << lg;
-    const int h = tid & 1;
-    for (int t0 = 0; t0 < m * m * m; t0 += kTail3Threads / 2) {
-        const int t = t0 + (tid >> 1);
+    const int lanes = tail3_lanes<T>(n), lgl = lanes == 8 ? 3 : 1;
+    const int h = tid & (lanes - 1);
+    for (int t0 = 0; t0 < m * m * m; t0 += kTail3Threads >> lgl) {
+        const int t = t0 + (tid >> lgl);
         const int I = t & (m - 1), J = (t >> lg) & (m - 1), K = t >> (2 * lg);
         const int i = 2 - pi + 2 * I, j = 2 - pj + 2 * J, k = 2 - pk + 2 * K;
         const bool on = i < n - 1 && j < n - 1 && k < n - 1;
         const int o = i + n * (j + n * k);
         T s = 0;
-        if (on) {
+        if (lanes == 8) {
+            const bool ua = sel == 0 || ((col ^ ln.ma) > col) == (sel > 0);
+            const bool ub = ln.mb && (sel == 0 || ((col ^ ln.mb) > col) == (sel > 0));
+            if (on && ua) {
+                s = v.A[ln.pa + o] * v.x[o + ln.da];
+                s += v.A[ln.pa + o - ln.da] * v.x[o - ln.da];
+            }
+            if (on && ub) {
+                s += v.A[ln.pb + o] * v.x[o + ln.db];
+                s += v.A[ln.pb + o - ln.db] * v.x[o - ln.db];
+            }
+            s += __shfl_xor_sync(0xffffffffu, s, 4);
+            s += __shfl_xor_sync(0xffffffffu, s, 2);
+        } else if (on) {
+            T s1 = 0;   // two chains
 #pragma unroll
             for (int q = 0; q < 13; q++) {
                 const int c = col ^ off_mask(q);
                 if (sel == 0 || (c > col) == (sel > 0)) {
                     const int d = off_x(q) + n * (off_y(q) + n * off_z(q));
-                    s += v.A[q * n3 + (h ? o - d : o)] * v.x[h ? o - d : o + d];
+                    const T a = v.A[q * n3 + (h ? o - d : o)], y = v.x[h ? o - d : o + d];
+                    if (q & 1)
+                        s1 += a * y;
+                    else
+                        s += a * y;
                 }
             }
+            s += s1;
         }
         s += __shfl_xor_sync(0xffffffffu, s, 1);
         if (on && h == 0) {
@@ -366,6 +439,7 @@ __global__ void __launch_bounds__(kTail3Threads) k_vtail3d(Tail3Args<T> a) {
     extern __shared__ __align__(16) unsigned char t3_raw[];
     __shared__ T3<T> lv[kTail3Lev];
     __shared__ uint64_t bar;
+    __shared__ int s_rw[27];   // restriction: weight plane (31: none) and, from bit 8, the owner's offset bits
     const int tid = threadIdx.x, nth = kTail3Threads;
     const int L = a.nlev;
     T* base = reinterpret_cast<T*>(t3_raw);
@@ -393,16 +467,29 @@ __global__ void __launch_bounds__(kTail3Threads) k_vtail3d(Tail3Args<T> a) {
             vp = v.r + n3;
         }
     }
+    if (tid >= 32 && tid < 59) {
+        const int o = tid - 32, dx = off_x(o), dy = off_y(o), dz = off_z(o);
+        const int m = (dx != 0) | ((dy != 0) << 1) | ((dz != 0) << 2);
+        const int sb = (dx < 0) | ((dy < 0) << 1) | ((dz < 0) << 2);
+        s_rw[o] = (m ? kPBase(m) + compress3(sb, m) : 31) | (sb << 8);
+    }
+    // the coarsest operator's one entry
+    const double ainv = tid == 0 ? 1.0 / *a.a64c : 0.0;
     __syncthreads();
-    // meanwhile: zero iterates and residuals, the first level's right-hand side
-    for (int q = 0; q < L; q++) {
-        const T3<T> v = lv[q];
-        const int n = v.n, n3 = n * n * n;
-        for (int u = tid; u < n3; u += nth) {
-            const int i = u % n, j = (u / n) % n, k = u / (n * n);
-            v.b[u] = q == 0 ? a.b[(long long)i + (long long)a.ld * (j + (long long)n * k)] : (T)0;
-            v.x[u] = v.r[u] = (T)0;
-        }
+    // meanwhile: zero vectors, then the first level's right-hand side
+    {
+        T* v0 = lv[0].b;
+        const int nv = (int)(lv[L - 1].r - v0) + lv[L - 1].n * lv[L - 1].n * lv[L - 1].n;
+        for (int u = tid; u < nv; u += nth) v0[u] = (T)0;
+    }
+    pdl_wait();
+    pdl_trigger();
+    __syncthreads();
+    {
+        const int n = lv[0].n;   // at most 16: half a warp a row
+        T* b = lv[0].b;
+        for (int row = tid >> 4; row < n * n; row += nth >> 4)
+            if ((tid & 15) < n) b[row * n + (tid & 15)] = a.b[(long long)a.ld * row + (tid & 15)];
     }
     if (!__syncthreads_and(mbar::wait(&bar, 0))) {
         // record the expiry, give the copies in flight one more bounded wait
@@ -413,56 +500,75 @@ __global__ void __launch_bounds__(kTail3Threads) k_vtail3d(Tail3Args<T> a) {
     }
     for (int l = 0; l + 1 < L; l++) {
         const T3<T> v = lv[l], w = lv[l + 1];
+        const T3Lane ln = tail3_lane(v.n, tid);
 #pragma unroll 1
         for (int ph = 0; ph < 15; ph++) {      // colours 0..7 forward, residuals of colours 0..6
-            tail3_colour<T>(v, ph & 7, ph < 8 ? -1 : 1, tid);
+            tail3_colour<T>(v, ln, ph & 7, ph < 8 ? -1 : 1, tid);
             if (ph < 8 || ph == 14) __syncthreads();
         }
-        const int nc = w.n, mc = nc - 2;
-        for (int q = tid; q < mc * mc * mc; q += nth) {
-            const int I = 1 + q % mc, J = 1 + (q / mc) % mc, K = 1 + q / (mc * mc);
-            restrict_node3d<T>(v.n, v.n, v.r, v.P, nc, nc, (long long)nc * nc * nc, w.b, nc, I, J, K);
+        // restriction: the 27 fine neighbours of a coarse node over eight lanes
+        const int n = v.n, nc = w.n, lg = 31 - __clz(nc - 1), mc = 1 << lg, nc3 = nc * nc * nc;
+        for (int t0 = 0; t0 < mc * mc * mc; t0 += nth >> 3) {
+            const int t = t0 + (tid >> 3);
+            const int I = t & (mc - 1), J = (t >> lg) & (mc - 1), K = t >> (2 * lg);
+            const bool on = I > 0 && J > 0 && K > 0 && K < mc;
+            const int oc = I + nc * (J + nc * K), of = 2 * (I + n * (J + n * K));
+            T s = 0;
+            if (on)
+                for (int o = tid & 7; o < 27; o += 8) {
+                    const int pw = s_rw[o], sb = pw >> 8;
+                    const T rv = v.r[of + off_x(o) + n * (off_y(o) + n * off_z(o))];
+                    const int own = oc - (sb & 1) - nc * (((sb >> 1) & 1) + nc * (sb >> 2));
+                    s += (pw & 31) == 31 ? rv : v.P[(pw & 31) * nc3 + own] * rv;
+                }
+            s += __shfl_xor_sync(0xffffffffu, s, 4);
+            s += __shfl_xor_sync(0xffffffffu, s, 2);
+            s += __shfl_xor_sync(0xffffffffu, s, 1);
+            if (on && (tid & 7) == 0) w.b[oc] = s;
         }
         __syncthreads();
     }
-    if (tid == 0) {   // coarsest: one unknown, exact in FP64
+    if (tid == 0) {   // coarsest: one unknown, in FP64
         const T3<T> v = lv[L - 1];
         const int o = 1 + v.n * (1 + v.n);
-        v.x[o] = (T)((double)v.b[o] / *a.a64c);
+        v.x[o] = (T)((double)v.b[o] * ainv);
     }
     __syncthreads();
     for (int l = L - 2; l >= 0; l--) {
         const T3<T> v = lv[l], w = lv[l + 1];
-        const int n = v.n, nc = w.n, m = n - 2, nc3 = nc * nc * nc;
-        for (int q = tid; q < m * m * m; q += nth) {
-            const int i = 1 + q % m, j = 1 + (q / m) % m, k = 1 + q / (m * m);
-            const int b = (i & 1) | ((j & 1) << 1) | ((k & 1) << 2);
-            const int oc = (i >> 1) + nc * ((j >> 1) + nc * (k >> 1));
+        const int n = v.n, nc = w.n, lg = 31 - __clz(nc - 1), mc = 1 << lg, nc3 = nc * nc * nc;
+        // cell (I, J, K) of the coarse level owns the fine points 2 (I, J, K) + b
+        for (int t = tid; t < 8 * mc * mc * mc; t += nth) {
+            const int I = t & (mc - 1), J = (t >> lg) & (mc - 1), K = (t >> (2 * lg)) & (mc - 1), b = t >> (3 * lg);
+            const int i = 2 * I + (b & 1), j = 2 * J + ((b >> 1) & 1), k = 2 * K + (b >> 2);
+            if (i == 0 || j == 0 || k == 0) continue;
+            const int oc = I + nc * (J + nc * K);
             T s = 0;
             if (b == 0) {
                 s = w.x[oc];
             } else {
-                for (int c = 0, e = 0; c < 8; c++)
+                const T* P = v.P + kPBase(b) * nc3 + oc;
+#pragma unroll
+                for (int c = 0; c < 8; c++)
                     if ((c & ~b) == 0) {
-                        s += v.P[(kPBase(b) + e) * nc3 + oc] * w.x[oc + (c & 1) + nc * (((c >> 1) & 1) + nc * (c >> 2))];
-                        e++;
+                        s += *P * w.x[oc + (c & 1) + nc * (((c >> 1) & 1) + nc * (c >> 2))];
+                        P += nc3;
                     }
             }
             v.x[i + n * (j + n * k)] += s;
         }
         __syncthreads();
+        const T3Lane ln = tail3_lane(n, tid);
 #pragma unroll 1
         for (int col = 7; col >= 0; col--) {
-            tail3_colour<T>(v, col, 0, tid);
+            tail3_colour<T>(v, ln, col, 0, tid);
             __syncthreads();
         }
     }
     {   // the first level's iterate to its array
-        const int n = a.n[0], n3 = n * n * n;
-        for (int u = tid; u < n3; u += nth) {
-            const int i = u % n, j = (u / n) % n, k = u / (n * n);
-            a.x[(long long)i + (long long)a.ld * (j + (long long)n * k)] = lv[0].x[u];
-        }
+        const int n = lv[0].n;
+        for (int row = tid >> 4; row < n * n; row += nth >> 4)
+            if ((tid & 15) < n) a.x[(long long)a.ld * row + (tid & 15)] = lv[0].x[row * n + (tid & 15)];
     }
 }
 
@@ -525,7 +631,9 @@ __global__ void k_tail3_pack(const T* __restrict__ A, int n, int ld, long long p
 // for the 127 points of a 129-node row (reverse sweep of one parity at 129^3:
 // FP64 120 us, full row 95; FP32 32.6, full row 27.8) and 128 for 63.  At 257^3
 // a row takes four warps, so either the rows' halo grows (four slots) or the
-// CTA does: 257 us against 196 for the 58-column tiles.
+// CTA does: 257 us against 196 for the 58-column tiles (169 since their
+// accesses are pairs and the first rows' stencils are fetched while the
+// iterates are staged).
 template <int W_, int S_, bool FULL_>
 struct HsShape {
     static constexpr int W = W_, S = S_;
@@ -600,7 +708,9 @@ struct HsPair {
                 mir1[t] = v.x;
             }
         }
-        const V2<T> v = ld2(a.f + o0);
+    }
+    __device__ __forceinline__ void load_f(const HS3Args<T>& a, long long o0) {
+        const V2<T> v = ld2c(a.f + o0);
         f0 = v.x;
         f1 = v.y;
     }
@@ -648,39 +758,63 @@ __global__ void __launch_bounds__(SH::threads, (sizeof(T) == 8 ? 512 : 768) / SH
     const int i0 = 1 + (int)blockIdx.x * SH::TI, j0 = 1 + (int)blockIdx.y * SH::TJ;
     const int ib = SH::FULL ? 0 : i0 - 3;    // first computed column (even)
     const int tid = threadIdx.x;
-    // shared position (lr, lc) holds node (ib - 2 + lc, j0 - 2 + lr)
-    for (int q = tid; q < SH::plane; q += SH::threads) {
-        const int lr = q / SH::cols, lc = q - lr * SH::cols;
-        const int i = ib - 2 + lc, j = j0 - 2 + lr;
-        const bool in = i >= 1 && i <= n - 2 && j >= 1 && j <= n - 2;
-        const int s = lr * SH::cols + (lc & 1) * SH::half + (lc >> 1);
-        const long long o = (long long)i + (long long)ld * j + sz * k;
-        xc[s] = (MODE == 2 && in) ? a.xcur[o] : (T)0;
-        if (MODE >= 1) {
-            xb[s] = (in && k >= 2) ? a.xz[o - sz] : (T)0;
-            xa[s] = (in && k <= n - 3) ? a.xz[o + sz] : (T)0;
-        }
-    }
-    __syncthreads();
     const int slot = tid / (32 * SH::W);
     const int p = tid - 32 * SH::W * slot;   // the pair's index in the row
     const int i = ib + 2 * p;                // its first column
     HsPair<T, MODE, FWD> hold;
     bool ok0 = false, ok1 = false;
-    // one row parity: the first call loads and updates the pair's earlier
-    // colour, the second updates the later one from the registers
-    auto phase = [&](auto jp, bool second) {
-        constexpr int jpar = decltype(jp)::value;   // the rows' parity: j0 - 1 is even
-        const int lrow = 2 * slot + jpar;           // region row, j = j0 - 1 + lrow
-        const int j = j0 - 1 + lrow;
-        const int rs = (lrow + 1) * SH::cols;
-        if (!second) {
-            const bool pv = j >= 1 && j <= n - 2 && i >= 0 && i <= n - 2;
-            ok0 = pv && i >= 1;
-            ok1 = pv && i + 1 <= n - 2;
-            if (pv) hold.template load<jpar>(a, (long long)i + (long long)ld * j + sz * k, ok0);
+    // the pair's rows: region row 2 slot + jpar, j = j0 - 1 + row (j0 - 1 is even)
+    auto load = [&](auto jp) {
+        constexpr int jpar = decltype(jp)::value;
+        const int j = j0 - 1 + 2 * slot + jpar;
+        const bool pv = j >= 1 && j <= n - 2 && i >= 0 && i <= n - 2;
+        ok0 = pv && i >= 1;
+        ok1 = pv && i + 1 <= n - 2;
+        if (pv) hold.template load<jpar>(a, (long long)i + (long long)ld * j + sz * k, ok0);
+    };
+    auto load_f = [&](int jpar) {
+        if (ok0 || ok1) hold.load_f(a, (long long)i + (long long)ld * (j0 - 1 + 2 * slot + jpar) + sz * k);
+    };
+    // the first rows' stencils, which no kernel of the iteration writes, are in
+    // flight while the iterates are staged
+    using First = std::integral_constant<int, FWD ? 0 : 1>;
+    using Second = std::integral_constant<int, FWD ? 1 : 0>;
+    load(First{});
+    pdl_wait();
+    pdl_trigger();
+    load_f(First::value);
+    // Shared position (lr, lc) holds node (ib - 2 + lc, j0 - 2 + lr), even
+    // columns before odd ones; boundary and padding entries of the arrays are
+    // zero, so a pair is in or out as a whole.
+    for (int q = tid; q < SH::rows * SH::half; q += SH::threads) {
+        const int lr = q / SH::half, lp = q - lr * SH::half;
+        const int ic = ib - 2 + 2 * lp, j = j0 - 2 + lr;
+        const bool in = ic >= 0 && ic + 1 < ld && j >= 0 && j <= n - 1;
+        const int s = lr * SH::cols + lp;
+        const long long o = (long long)ic + (long long)ld * j + sz * k;
+        V2<T> c{0, 0}, b{0, 0}, t{0, 0};
+        if (in) {
+            if (MODE == 2) c = ld2c(a.xcur + o);
+            if (MODE >= 1) {
+                b = ld2c(a.xz + o - sz);
+                t = ld2c(a.xz + o + sz);
+            }
         }
-        // FWD: even column first; reverse: odd column first
+        xc[s] = c.x;
+        xc[s + SH::half] = c.y;
+        if (MODE >= 1) {
+            xb[s] = b.x;
+            xb[s + SH::half] = b.y;
+            xa[s] = t.x;
+            xa[s + SH::half] = t.y;
+        }
+    }
+    __syncthreads();
+    // one row parity: the pair's earlier colour, then the later one from the
+    // registers (FWD: even column first; reverse: odd column first)
+    auto phase = [&](auto jp, bool second) {
+        constexpr int jpar = decltype(jp)::value;
+        const int rs = (2 * slot + jpar + 1) * SH::cols;
         const bool do_odd = FWD ? second : !second;
         if (do_odd) {
             if (ok1)
@@ -693,31 +827,38 @@ __global__ void __launch_bounds__(SH::threads, (sizeof(T) == 8 ? 512 : 768) / SH
         }
         __syncthreads();
     };
-    if (FWD) {
-        phase(std::integral_constant<int, 0>{}, false);
-        phase(std::integral_constant<int, 0>{}, true);
-        phase(std::integral_constant<int, 1>{}, false);
-        phase(std::integral_constant<int, 1>{}, true);
-    } else {
-        phase(std::integral_constant<int, 1>{}, false);
-        phase(std::integral_constant<int, 1>{}, true);
-        phase(std::integral_constant<int, 0>{}, false);
-        phase(std::integral_constant<int, 0>{}, true);
-    }
-    for (int q = tid; q < SH::TI * SH::TJ; q += SH::threads) {
-        const int lj = q / SH::TI, li = q - lj * SH::TI;
-        const int ii = i0 + li, jj = j0 + lj;
-        if (ii > n - 2 || jj > n - 2) continue;
-        const int lc = ii - ib + 2, lr = jj - j0 + 2;
-        a.xout[(long long)ii + (long long)ld * jj + sz * k] = xc[lr * SH::cols + (lc & 1) * SH::half + (lc >> 1)];
+    phase(First{}, false);
+    phase(First{}, true);
+    load(Second{});
+    load_f(Second::value);
+    phase(Second{}, false);
+    phase(Second{}, true);
+    // every thread stores its pair of both rows
+#pragma unroll
+    for (int r = 0; r < 2; r++) {
+        const int lrow = 2 * slot + r, j = j0 - 1 + lrow;
+        if (lrow < 1 || lrow > SH::TJ || j > n - 2) continue;
+        const bool w0 = i >= i0 && i < i0 + SH::TI && i <= n - 2;
+        const bool w1 = i + 1 >= i0 && i + 1 < i0 + SH::TI && i + 1 <= n - 2;
+        const T v0 = xc[(lrow + 1) * SH::cols + p + 1], v1 = xc[(lrow + 1) * SH::cols + SH::half + p + 1];
+        T* o = a.xout + (long long)i + (long long)ld * j + sz * k;
+        if (w0 && w1) {
+            st2(o, v0, v1);
+        } else if (w0) {
+            o[0] = v0;
+        } else if (w1) {
+            o[1] = v1;
+        }
     }
 }
 
 // x_out = x_in + P x_c at every interior fine point (out of place; the
 // same sum as prolong_node3d).
 template <typename T>
-__global__ void k_prolong3d_to(int nf, int ldf, const T* __restrict__ xin, T* __restrict__ xout,
-                               const T* __restrict__ P, int nc, int ldc, long long plc, const T* __restrict__ xc) {
+__global__ void k_prolong3d_to(int nf, int ldf, const T* xin, T* __restrict__ xout,
+                               const T* __restrict__ P, int nc, int ldc, long long plc, const T* xc) {
+    pdl_wait();
+    pdl_trigger();
     const int I = blockIdx.x * blockDim.x + threadIdx.x;
     const int J = blockIdx.y, K = blockIdx.z;
     if (I > nc - 2 || J > nc - 2 || K > nc - 2) return;
@@ -801,9 +942,9 @@ bmg_status launch_hsweep3d(Ctx& c, const HS3Args<T>& a, int planes) {
     auto kern = k_hsweep3d<T, SH, MODE, FWD>;
     const int smem = (int)(3 * SH::plane * sizeof(T));
     if (smem > 48 * 1024) BMG_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
-    kern<<<dim3(cdiv(a.n - 2, SH::TI), cdiv(a.n - 2, SH::TJ), planes), SH::threads, smem, c.stream>>>(a);
+    BMG_CUDA(launch_pdl(kern, dim3(cdiv(a.n - 2, SH::TI), cdiv(a.n - 2, SH::TJ), planes), dim3(SH::threads), smem,
+                        c.stream, a));
     c.launches++;
-    BMG_CUDA(cudaGetLastError());
     return BMG_OK;
 }
 
@@ -843,8 +984,8 @@ bmg_status hs3_up(Ctx& c, int l, const T* f, T* x, const T* xc) {
     const Level& K = c.lev[l + 1];
     T* xcor = (T*)F.r;
     prof_begin(c, BMG_PROF_PROLONG, l);
-    k_prolong3d_to<T><<<g3(K.n - 1, K.n - 1, K.n - 1), 64, 0, c.stream>>>(F.n, F.ld, x, xcor, P_of<T>(F), K.n, K.ld,
-                                                                           K.plane, xc);
+    BMG_CUDA(launch_pdl(k_prolong3d_to<T>, g3(K.n - 1, K.n - 1, K.n - 1), dim3(64), 0, c.stream, F.n, F.ld, x, xcor,
+                        P_of<T>(F), K.n, K.ld, K.plane, xc));
     prof_end(c, BMG_PROF_PROLONG, l, (2.0 + c.np / 8.0 + 0.125) * sizeof(T) * dofs3(c, l));
     c.launches += 1;
     BMG_TRY((hsweep3d<T, 2, false>(c, l, f, xcor, xcor, x, 1)));
@@ -873,11 +1014,12 @@ bmg_status vcycle3d_impl(Ctx& c, const T* b0, T* x0, T* xout) {
             for (int col = 0; col < 8; col++) BMG_TRY(colour_sweep<T>(c, l, v, bl(l), xl(l), col, h));
         }
         prof_begin(c, BMG_PROF_RESIDUAL, l);
-        k_residual3d_sweep<T><<<g3((F.n - 1) / 2, F.n - 2, F.n - 2), 64, 0, s>>>(v, xl(l), (T*)F.r);
+        BMG_CUDA(launch_pdl(k_residual3d_sweep<T>, g3((F.n - 1) / 2, F.n - 2, F.n - 2), dim3(64), 0, s, v, xl(l),
+                            (T*)F.r));
         prof_end(c, BMG_PROF_RESIDUAL, l, (c.ns + 3) * sz * N);
         prof_begin(c, BMG_PROF_RESTRICT, l);
-        k_restrict3d<T><<<g3(K.n, K.n, K.n), 64, 0, s>>>(F.n, F.ld, (const T*)F.r, P_of<T>(F), K.n, K.ld, K.plane,
-                                                        (T*)K.b);
+        BMG_CUDA(launch_pdl(k_restrict3d<T>, g3(K.n, K.n, K.n), dim3(64), 0, s, F.n, F.ld, (const T*)F.r, P_of<T>(F),
+                            K.n, K.ld, K.plane, (T*)K.b));
         prof_end(c, BMG_PROF_RESTRICT, l, (1.0 + c.np / 8.0 + 0.125) * sz * N);
         c.launches += 2;   // residual, restriction (the colours count themselves)
     }
@@ -896,7 +1038,7 @@ bmg_status vcycle3d_impl(Ctx& c, const T* b0, T* x0, T* xout) {
         a.st = c.st;
         const size_t smem = a.pack_bytes + sizeof(T) * tail3_vec_elems(c);
         BMG_CUDA(cudaFuncSetAttribute(k_vtail3d<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-        k_vtail3d<T><<<1, kTail3Threads, smem, s>>>(a);
+        BMG_CUDA(launch_pdl(k_vtail3d<T>, dim3(1), dim3(kTail3Threads), smem, s, a));
         c.launches++;
     }
     for (int l = t - 1; l >= 0; l--) {
