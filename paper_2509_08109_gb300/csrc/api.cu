@@ -179,8 +179,13 @@ bmg_status enqueue_iteration(Ctx& c, int parity) {
     } else {
         double* zn = c.z[parity];
         double* zo = c.z[parity ^ 1];
-        BMG_TRY(vcycle(c, c.r, zn));
-        BMG_TRY(k_rz_beta(c, zn, zo, c.opts.outer == BMG_OUTER_FLEXIBLE_CG));
+        const bool flexible = c.opts.outer == BMG_OUTER_FLEXIBLE_CG;
+        if (vcycle_forms_beta(c)) {
+            BMG_TRY(vcycle(c, c.r, zn, zo, flexible ? 2 : 1));   // the finest up kernel also forms beta
+        } else {
+            BMG_TRY(vcycle(c, c.r, zn));
+            BMG_TRY(k_rz_beta(c, zn, zo, flexible));
+        }
         BMG_TRY(k_p_update(c, zn));
         BMG_TRY(k_spmv_pq(c, c.p, c.q));
         BMG_TRY(k_update_xr(c));

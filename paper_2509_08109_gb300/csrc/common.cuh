@@ -355,15 +355,17 @@ bmg_status batch_solve(Batch& B, int nrhs, const double* const* b, double* const
 void batch_destroy(Batch* B);
 size_t batch_single_bytes(Ctx& c);
 bmg_status batch_single_create(Ctx& c, Batch** out);
-// vcycle.cu: z = M r on the finest level (FP64 in/out, internal layout)
-bmg_status vcycle(Ctx& c, const double* r, double* z);
+// vcycle.cu: z = M r on the finest level (FP64 in/out, internal layout); dots
+// (only where vcycle_forms_beta): the finest up kernel also forms beta from
+// r.z (1) or r.z - r.zold (2)
+bmg_status vcycle(Ctx& c, const double* r, double* z, const double* zold = nullptr, int dots = 0);
 // fused2d.cu / tmaps.cu
 int fused_rows_per_step(bool f32);
 int fused_down_smem(bool f32, bool f64in, int wc);
 int fused_up_smem(bool f32, bool f64in, int wc);
 bmg_status fused_occupancy(bool f32, bool f64in, int wc, int* down_blocks, int* up_blocks);
 bmg_status fused_down(Ctx& c, int l, bool ir = false);
-bmg_status fused_up(Ctx& c, int l, void* out, bool ir = false, const float* zold = nullptr);
+bmg_status fused_up(Ctx& c, int l, void* out, bool ir = false, const void* zold = nullptr, int dots = 0);
 bmg_status vcycle_f32(Ctx& c, float* z32, const float* zold = nullptr);
 // batched streaming kernels (fused2d.cu): FP32, kBatchR right-hand sides, strip width 16 or 32
 int batch_down_smem(int wc);
@@ -410,8 +412,8 @@ bmg_status tail_pack(Ctx& c);                     // fills c.tail_pack (bmg_setu
 bmg_status tail_vcycle(Ctx& c, int t);
 size_t tail3_pack_bytes(const Ctx& c);            // the same for the 3-D tail (vcycle3d.cu)
 bmg_status tail3_pack(Ctx& c);
-// z32 = M r32 (FP32 in and out); with zold and the streaming kernels the
-// finest up kernel also forms r.z, r.z_old and the flexible-CG beta
+// whether the streaming kernels' finest up kernel can form beta (its tiles'
+// sums fit the partials)
 bool vcycle_forms_beta(const Ctx& c);
 template <typename T>
 bmg_status vcycle3d_impl(Ctx& c, const T* b0, T* x0, T* xout);

@@ -356,23 +356,32 @@ __global__ void __launch_bounds__((WC + 8) * K, sizeof(T) == 4 ? 3 : 1)
     rg.q0 = J0 - 2;
     rg.qb = qb;
     const int npairs = p.hc + 2;
-    auto issue = [&](int q) {
+    auto issue_op = [&](int q) {    // the operator's rows, which no kernel of the iteration writes
         const int s = (int)((qb + (unsigned)q) % (unsigned)RP), Jp = rg.q0 + q;
         uint64_t* bar = rg.bars + s;
         mbar::expect_tx(bar, txb);
-        if constexpr (BATCH) {
-            // vector maps group 8 nodes x NR values into their innermost
-            // dimension (x0 is a multiple of 8)
+        if constexpr (BATCH)
             tma4d(rg.pA + s * L.sA, &tmA, bar, x0, 2 * Jp + 1, 0, mi);
-            tma4d(rg.pF + s * L.sF, &tmF, bar, 0, x0 / 8, 2 * Jp + 1, mi);
-        } else {
+        else
             tma3d(rg.pA + s * L.sA, &tmA, bar, x0, 2 * Jp + 1, 0);
+    };
+    auto issue_vec = [&](int q) {
+        const int s = (int)((qb + (unsigned)q) % (unsigned)RP), Jp = rg.q0 + q;
+        uint64_t* bar = rg.bars + s;
+        // batched vector maps group 8 nodes x NR values into their innermost
+        // dimension (x0 is a multiple of 8)
+        if constexpr (BATCH)
+            tma4d(rg.pF + s * L.sF, &tmF, bar, 0, x0 / 8, 2 * Jp + 1, mi);
+        else
             tma2d(rg.pF + s * L.sF, &tmF, bar, x0, 2 * Jp + 1);
-        }
+    };
+    auto issue = [&](int q) {
+        issue_op(q);
+        issue_vec(q);
     };
     int issued = npairs < RP ? npairs : RP, waited = 0;
     if (lead)
-        for (int q = 0; q < issued; q++) issue(q);
+        for (int q = 0; q < issued; q++) issue_op(q);
 
     // per-thread columns: the even/odd pair (2 tx, 2 tx + 1) of the window
     const int ce = 2 * tx, co = ce + 1;
@@ -439,6 +448,26 @@ __global__ void __launch_bounds__((WC + 8) * K, sizeof(T) == 4 ? 3 : 1)
         }
     };
 
+    // interpolation weights of the thread's coarse node for the restriction,
+    // loaded one step ahead.  After colour 3 the odd-odd fine points have
+    // zero residual, so their four weights are not needed.
+    T w[4];
+    auto load_w = [&](int Jp) {
+        const bool d = vres && Jp <= nc - 2;
+        const long long o = (long long)Jp * p.ldc + I;
+        w[0] = d ? Pg[PXR * p.plc + o - 1] : (T)0;
+        w[1] = d ? Pg[PXL * p.plc + o] : (T)0;
+        w[2] = d ? Pg[PYN * p.plc + o - p.ldc] : (T)0;
+        w[3] = d ? Pg[PYS * p.plc + o] : (T)0;
+    };
+    load_w(J0 + ty);
+    if (!BATCH) {
+        pdl_wait();
+        pdl_trigger();
+    }
+    if (lead)
+        for (int q = 0; q < issued; q++) issue_vec(q);
+
     bool ok = wait_pairs<RP>(rg.bars, qb, qb + 2);
     waited = ok ? 2 : 0;
     if (ok) {   // pre-roll: rows 2J0-2 .. 2J0 final, residual of row 2J0-1
@@ -453,19 +482,6 @@ __global__ void __launch_bounds__((WC + 8) * K, sizeof(T) == 4 ? 3 : 1)
         if (ty == 0) resid(2 * J0 - 1);
         __syncthreads();
     }
-    // interpolation weights of the thread's coarse node for the restriction,
-    // loaded one step ahead.  After colour 3 the odd-odd fine points have
-    // zero residual, so their four weights are not needed.
-    T w[4];
-    auto load_w = [&](int Jp) {
-        const bool d = vres && Jp <= nc - 2;
-        const long long o = (long long)Jp * p.ldc + I;
-        w[0] = d ? Pg[PXR * p.plc + o - 1] : (T)0;
-        w[1] = d ? Pg[PXL * p.plc + o] : (T)0;
-        w[2] = d ? Pg[PYN * p.plc + o - p.ldc] : (T)0;
-        w[3] = d ? Pg[PYS * p.plc + o] : (T)0;
-    };
-    load_w(J0 + ty);
     for (int J = J0; ok && J < J0 + p.hc; J += K) {
         const int qa = J - rg.q0;
         ok = wait_pairs<RP>(rg.bars, qb + qa, qb + qa + K);
@@ -596,28 +612,38 @@ __global__ void __launch_bounds__((WC + 8) * K, sizeof(T) == 4 ? 3 : 1)
     rg.q0 = J0 - 2;
     rg.qb = qb;
     const int npairs = p.hc + 2;
-    auto issue = [&](int q) {
+    auto issue_op = [&](int q) {    // the operator's rows, which no kernel of the iteration writes
         const int s = (int)((qb + (unsigned)q) % (unsigned)RP), Jp = rg.q0 + q;
         uint64_t* bar = rg.bars + s;
         mbar::expect_tx(bar, txb);
+        if constexpr (BATCH)
+            tma4d(rg.pA + s * L.sA, &tmA, bar, x0, 2 * Jp + 1, 0, mi);
+        else
+            tma3d(rg.pA + s * L.sA, &tmA, bar, x0, 2 * Jp + 1, 0);
+    };
+    auto issue_vec = [&](int q) {
+        const int s = (int)((qb + (unsigned)q) % (unsigned)RP), Jp = rg.q0 + q;
+        uint64_t* bar = rg.bars + s;
         if constexpr (BATCH) {
             // vector maps group 8 nodes x NR values (fine rows; x0 is a
             // multiple of 8) or 4 nodes (the coarse row; xc0 a multiple of 4)
             // into their innermost dimension
-            tma4d(rg.pA + s * L.sA, &tmA, bar, x0, 2 * Jp + 1, 0, mi);
             tma4d(rg.pF + s * L.sF, &tmF, bar, 0, x0 / 8, 2 * Jp + 1, mi);
             tma4d(rg.pXp + s * L.sXp, &tmX, bar, 0, x0 / 8, 2 * Jp + 1, mi);
             tma4d(rg.pC + s * L.sC, &tmC, bar, 0, xc0 / 4, Jp + 1, cmi);
         } else {
-            tma3d(rg.pA + s * L.sA, &tmA, bar, x0, 2 * Jp + 1, 0);
             tma2d(rg.pF + s * L.sF, &tmF, bar, x0, 2 * Jp + 1);
             tma2d(rg.pXp + s * L.sXp, &tmX, bar, x0, 2 * Jp + 1);
             tma2d(rg.pC + s * L.sC, &tmC, bar, xc0, Jp + 1);
         }
     };
+    auto issue = [&](int q) {
+        issue_op(q);
+        issue_vec(q);
+    };
     int issued = npairs < RP ? npairs : RP, waited = 0;
     if (lead)
-        for (int q = 0; q < issued; q++) issue(q);
+        for (int q = 0; q < issued; q++) issue_op(q);
 
     const int ce = 2 * tx, co = ce + 1;
     const int ie = x0 + ce;
@@ -635,9 +661,15 @@ __global__ void __launch_bounds__((WC + 8) * K, sizeof(T) == 4 ? 3 : 1)
     };
     const T* Pg = BATCH ? (const T*)M->P : (const T*)p.P;
     VO* out = (VO*)(BATCH ? M->x[p.parity] : p.x);
-    // finest level of the refinement mode only
-    const VZ* zold = (const VZ*)(BATCH ? M->zold[p.parity] : p.zold);
+    // finest level of a Krylov iteration only: the sums' type follows the
+    // right-hand side's (FP32: compensated, FP64: plain)
+    constexpr bool D64 = sizeof(TF) == 8;
+    using VD = typename std::conditional<D64, double, VZ>::type;
+    const VD* zold = (const VD*)(BATCH ? M->zold[p.parity] : p.zold);
+    const bool dots = BATCH ? zold != nullptr : p.dots != 0;
+    const bool two = BATCH || p.dots == 2;
     AccN<NR> rz, rzo;
+    double rz64 = 0.0, rzo64 = 0.0;
     const V z0 = vzero<V>();
     auto pw = [&](int plane, int Jc) -> T {
         return (vI && Jc >= 0 && Jc <= nc - 1) ? Pg[plane * p.plc + (long long)Jc * p.ldc + I] : (T)0;
@@ -670,22 +702,6 @@ __global__ void __launch_bounds__((WC + 8) * K, sizeof(T) == 4 ? 3 : 1)
         X(j)[c] = divide(vcast<V>(rg.F(j)[c]) - r.offdiag(c), r.diag(c));
     };
 
-    bool ok = wait_pairs<RP>(rg.bars, qb, qb + 2);
-    waited = ok ? 2 : 0;
-    if (ok) {   // pre-roll: corrected rows 2J0-2 .. 2J0, odd row 2J0-1 smoothed
-        if (ty == 0) {
-            const int Jm = J0 - 1;
-            const T wy[6] = {pw(PYS, Jm), pw(PYN, Jm), pw(PSW, Jm), pw(PSE, Jm), pw(PNW, Jm), pw(PNE, Jm)};
-            corr_even(2 * J0 - 2, pw(PXL, Jm), pw(PXR, Jm));
-            corr_odd(2 * J0 - 1, wy);
-            corr_even(2 * J0, pw(PXL, J0), pw(PXR, J0));
-        }
-        __syncthreads();
-        if (ty == 0) gs(2 * J0 - 1, co, vo);     // colour 3
-        __syncthreads();
-        if (ty == 0) gs(2 * J0 - 1, ce, ve);     // colour 2
-        __syncthreads();
-    }
     // weights for the corrected values of this thread's rows, loaded one step ahead
     T wy[6], wxl, wxr;
     auto load_w = [&](int Jp) {
@@ -699,10 +715,46 @@ __global__ void __launch_bounds__((WC + 8) * K, sizeof(T) == 4 ? 3 : 1)
         wxr = pw(PXR, Jp + 1);
     };
     load_w(J0 + ty);
+    // the pre-roll's weights (rows of coarse rows J0 - 1 and J0)
+    T w0[10];
+    if (ty == 0) {
+        const int Jm = J0 - 1;
+        w0[0] = pw(PYS, Jm);
+        w0[1] = pw(PYN, Jm);
+        w0[2] = pw(PSW, Jm);
+        w0[3] = pw(PSE, Jm);
+        w0[4] = pw(PNW, Jm);
+        w0[5] = pw(PNE, Jm);
+        w0[6] = pw(PXL, Jm);
+        w0[7] = pw(PXR, Jm);
+        w0[8] = pw(PXL, J0);
+        w0[9] = pw(PXR, J0);
+    }
+    if (!BATCH) {
+        pdl_wait();
+        pdl_trigger();
+    }
+    if (lead)
+        for (int q = 0; q < issued; q++) issue_vec(q);
+
+    bool ok = wait_pairs<RP>(rg.bars, qb, qb + 2);
+    waited = ok ? 2 : 0;
+    if (ok) {   // pre-roll: corrected rows 2J0-2 .. 2J0, odd row 2J0-1 smoothed
+        if (ty == 0) {
+            corr_even(2 * J0 - 2, w0[6], w0[7]);
+            corr_odd(2 * J0 - 1, w0);
+            corr_even(2 * J0, w0[8], w0[9]);
+        }
+        __syncthreads();
+        if (ty == 0) gs(2 * J0 - 1, co, vo);     // colour 3
+        __syncthreads();
+        if (ty == 0) gs(2 * J0 - 1, ce, ve);     // colour 2
+        __syncthreads();
+    }
     // previous preconditioned residual at this thread's stored nodes of the
     // rows 2Jp-1, 2Jp, also loaded one step ahead (refinement mode only)
-    const VZ zz = vzero<VZ>();
-    VZ zo_nx[2][2] = {{zz, zz}, {zz, zz}};
+    const VD zz = vzero<VD>();
+    VD zo_nx[2][2] = {{zz, zz}, {zz, zz}};
     auto load_zo = [&](int Jp) {
         for (int rr = 0; rr < 2; rr++) {
             const int j = 2 * Jp - 1 + rr;
@@ -712,7 +764,7 @@ __global__ void __launch_bounds__((WC + 8) * K, sizeof(T) == 4 ? 3 : 1)
             zo_nx[rr][1] = (rj && own_o) ? zold[o + 1] : zz;
         }
     };
-    if (zold) load_zo(J0 + ty);
+    if (dots && two) load_zo(J0 + ty);
     for (int J = J0; ok && J < J0 + p.hc; J += K) {
         const int qa = J - rg.q0;
         const int Jp = J + ty, jm = 2 * Jp, jo = jm + 1, je = jm + 2;
@@ -729,8 +781,8 @@ __global__ void __launch_bounds__((WC + 8) * K, sizeof(T) == 4 ? 3 : 1)
         corr_odd(jo, wy);
         corr_even(je, wxl, wxr);
         load_w(Jp + K);
-        VZ zo_now[2][2] = {{zo_nx[0][0], zo_nx[0][1]}, {zo_nx[1][0], zo_nx[1][1]}};
-        if (zold) load_zo(Jp + K);
+        VD zo_now[2][2] = {{zo_nx[0][0], zo_nx[0][1]}, {zo_nx[1][0], zo_nx[1][1]}};
+        if (dots && two) load_zo(Jp + K);
         __syncthreads();
         gs(jo, co, vo);      // colour 3
         __syncthreads();
@@ -741,12 +793,12 @@ __global__ void __launch_bounds__((WC + 8) * K, sizeof(T) == 4 ? 3 : 1)
         gs(jm, ce, ve);      // colour 0
         // right-hand side of the stored rows, read while their ring slots
         // cannot yet be refilled (the next refill follows the next barrier)
-        VZ fr[2][2] = {{zz, zz}, {zz, zz}};
-        if (zold)
+        VD fr[2][2] = {{zz, zz}, {zz, zz}};
+        if (dots)
             for (int rr = 0; rr < 2; rr++) {
                 const RowV<const typename Ring<T, TF, K, true, NR>::VF> Fr = rg.F(jm - 1 + rr);
-                fr[rr][0] = vcast<VZ>(Fr[ce]);
-                fr[rr][1] = vcast<VZ>(Fr[co]);
+                fr[rr][0] = vcast<VD>(Fr[ce]);
+                fr[rr][1] = vcast<VD>(Fr[co]);
             }
         __syncthreads();
         for (int rr = 0; rr < 2; rr++) {
@@ -756,14 +808,23 @@ __global__ void __launch_bounds__((WC + 8) * K, sizeof(T) == 4 ? 3 : 1)
             const long long o = (long long)j * p.ldf + ie;
             if (own_e) out[o] = vcast<VO>(Xr[ce]);
             if (own_o) out[o + 1] = vcast<VO>(Xr[co]);
-            if (zold) {
-                if (own_e) {
-                    rz.add(fr[rr][0], vcast<VZ>(Xr[ce]));
-                    rzo.add(fr[rr][0], zo_now[rr][0]);
-                }
-                if (own_o) {
-                    rz.add(fr[rr][1], vcast<VZ>(Xr[co]));
-                    rzo.add(fr[rr][1], zo_now[rr][1]);
+            if (dots) {
+                if constexpr (D64) {
+                    if (own_e) rz64 += fr[rr][0] * (double)Xr[ce];
+                    if (own_o) rz64 += fr[rr][1] * (double)Xr[co];
+                    if (two) {
+                        if (own_e) rzo64 += fr[rr][0] * zo_now[rr][0];
+                        if (own_o) rzo64 += fr[rr][1] * zo_now[rr][1];
+                    }
+                } else {
+                    if (own_e) {
+                        rz.add(fr[rr][0], vcast<VZ>(Xr[ce]));
+                        rzo.add(fr[rr][0], zo_now[rr][0]);
+                    }
+                    if (own_o) {
+                        rz.add(fr[rr][1], vcast<VZ>(Xr[co]));
+                        rzo.add(fr[rr][1], zo_now[rr][1]);
+                    }
                 }
             }
         }
@@ -780,7 +841,7 @@ __global__ void __launch_bounds__((WC + 8) * K, sizeof(T) == 4 ? 3 : 1)
         return;
     }
     qb += (unsigned)npairs;
-    if (zold) {
+    if (dots) {
         // Deterministic reduction of (r.z, r.z_old) per right-hand side; the
         // last CTA (of the grid, or of the problem's tiles when batched)
         // forms the flexible-CG beta.  Every copy into the rings has
@@ -809,7 +870,10 @@ __global__ void __launch_bounds__((WC + 8) * K, sizeof(T) == 4 ? 3 : 1)
             }
         };
         double b1[NR], b2[NR];
-        for (int r = 0; r < NR; r++) block_sum2(rz.a[r].value(), rzo.a[r].value(), b1[r], b2[r]);
+        if constexpr (D64)
+            block_sum2(rz64, rzo64, b1[0], b2[0]);
+        else
+            for (int r = 0; r < NR; r++) block_sum2(rz.a[r].value(), rzo.a[r].value(), b1[r], b2[r]);
         if constexpr (!BATCH) {
             const int nb = gridDim.x * gridDim.y;
             if (tid == 0) {
@@ -835,8 +899,9 @@ __global__ void __launch_bounds__((WC + 8) * K, sizeof(T) == 4 ? 3 : 1)
                     if (st->first) {
                         st->beta = 0.0;
                         st->first = 0;
+                        st->rzn = t1;   // the run's first r.z, for the host's prediction
                     } else {
-                        st->beta = (t1 - t2) / st->rz;
+                        st->beta = (two ? t1 - t2 : t1) / st->rz;
                     }
                     st->rz = t1;
                 }
@@ -934,14 +999,17 @@ bmg_status launch_down(Ctx& c, const FusedLevel& F, cudaStream_t s) {
         const int smem = down_smem<T, TF>(F.wc);
         if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess)
             return BMG_ERR_DEVICE;
-        kern<<<dim3(F.tiles_x, F.tiles_y), dim3(F.wc + 8, k_of<T>()), smem, s>>>(F.mA, F.mF, F.down);
         c.launches++;
-        return cudaGetLastError() == cudaSuccess ? BMG_OK : BMG_ERR_DEVICE;
+        return launch_pdl(kern, dim3(F.tiles_x, F.tiles_y), dim3(F.wc + 8, k_of<T>()), smem, s, F.mA, F.mF, F.down) ==
+                       cudaSuccess
+                   ? BMG_OK
+                   : BMG_ERR_DEVICE;
     });
 }
 
 template <typename T, typename TF, typename TO>
-bmg_status launch_up(Ctx& c, const FusedLevel& F, cudaStream_t s, void* out, const void* zold = nullptr) {
+bmg_status launch_up(Ctx& c, const FusedLevel& F, cudaStream_t s, void* out, const void* zold = nullptr,
+                     int dots = 0) {
     return with_wc(F.wc, [&](auto W) {
         auto kern = k_vup2d<T, TF, TO, k_of<T>(), decltype(W)::value>;
         const int smem = up_smem<T, TF>(F.wc);
@@ -950,10 +1018,13 @@ bmg_status launch_up(Ctx& c, const FusedLevel& F, cudaStream_t s, void* out, con
         FusedArgs a = F.up;
         a.x = out;
         a.zold = zold;
-        a.partials = zold ? c.partials : nullptr;
-        kern<<<dim3(F.tiles_x, F.tiles_y_up), dim3(F.wc + 8, k_of<T>()), smem, s>>>(F.mA, F.mF, F.mXp, F.mXc, a);
+        a.dots = dots;
+        a.partials = dots ? c.partials : nullptr;
         c.launches++;
-        return cudaGetLastError() == cudaSuccess ? BMG_OK : BMG_ERR_DEVICE;
+        return launch_pdl(kern, dim3(F.tiles_x, F.tiles_y_up), dim3(F.wc + 8, k_of<T>()), smem, s, F.mA, F.mF, F.mXp,
+                          F.mXc, a) == cudaSuccess
+                   ? BMG_OK
+                   : BMG_ERR_DEVICE;
     });
 }
 
@@ -1057,12 +1128,14 @@ bmg_status fused_down(Ctx& c, int l, bool ir) {
     return launch_down<float, float>(c, F, c.stream);
 }
 
-bmg_status fused_up(Ctx& c, int l, void* out, bool ir, const float* zold) {
+// dots (level 0 only): see FusedArgs
+bmg_status fused_up(Ctx& c, int l, void* out, bool ir, const void* zold, int dots) {
     const FusedLevel& F = (ir && l == 0) ? c.fused_ir0 : c.fused[l];
     const bool f32 = c.opts.precision == BMG_PREC_FP32;
-    if (!f32) return launch_up<double, double, double>(c, F, c.stream, out);
-    if (l == 0 && !ir) return launch_up<float, double, double>(c, F, c.stream, out);
-    return launch_up<float, float, float>(c, F, c.stream, out, (ir && l == 0) ? zold : nullptr);
+    if (l != 0) dots = 0;
+    if (!f32) return launch_up<double, double, double>(c, F, c.stream, out, zold, dots);
+    if (l == 0 && !ir) return launch_up<float, double, double>(c, F, c.stream, out, zold, dots);
+    return launch_up<float, float, float>(c, F, c.stream, out, zold, dots);
 }
 
 }  // namespace bmg

@@ -33,11 +33,13 @@ struct FusedArgs {
     const void* P;   // interpolation planes (coarse grid)
     long long plc;   // plane stride of P
     KState* st;
-    // up kernel, finest level of the refinement mode: r.z and r.z_old of the
-    // owned nodes (r = this kernel's right-hand side, z = its output) reduced
-    // into the CG coefficient; null when not wanted
+    // up kernel, finest level of a Krylov iteration: r.z (dots >= 1) and r.z_old
+    // (dots == 2) of the owned nodes (r = this kernel's right-hand side, z = its
+    // output, both in the types of the right-hand side) reduced into the CG
+    // coefficient beta, r.z_old subtracted when it is formed
     const void* zold;
     double* partials;
+    int dots = 0;
     // batched kernels: a persistent grid walks the work-list of (member,
     // tile) items of one size class; members describe each (problem, level)
     const BatchMember* mem = nullptr;

@@ -209,7 +209,7 @@ bmg_status vcycle2d_impl(Ctx& c, const T* b0, T* x0) {
 // Streaming path: one down kernel and one up kernel per level pair above
 // the tail, and one single-CTA kernel for the tail levels.
 template <typename T>
-bmg_status vcycle2d_fused(Ctx& c, void* z, bool ir = false, const float* zold = nullptr) {
+bmg_status vcycle2d_fused(Ctx& c, void* z, bool ir = false, const void* zold = nullptr, int dots = 0) {
     const double sz = sizeof(T);
     // levels t.. (n <= kTailMaxN) run in one single-CTA launch
     const int t = tail_first_level(c);
@@ -228,8 +228,8 @@ bmg_status vcycle2d_fused(Ctx& c, void* z, bool ir = false, const float* zold = 
         const double szf = (l == 0 && !ir) ? 8.0 : sz;
         const double szo = (l == 0 && !ir) ? 8.0 : sz;
         prof_begin(c, BMG_PROF_VUP, l);
-        BMG_TRY(fused_up(c, l, l == 0 ? z : c.lev[l].r, ir, zold));
-        const double szz = (l == 0 && ir && zold) ? 4.0 : 0.0;   // z_old read for the fused beta
+        BMG_TRY(fused_up(c, l, l == 0 ? z : c.lev[l].r, ir, zold, dots));
+        const double szz = (l == 0 && dots == 2) ? szo : 0.0;   // z_old read for the fused beta
         prof_end(c, BMG_PROF_VUP, l, N * (c.ns * sz + szf + sz + c.np / 4.0 * sz + sz / 4 + szo + szz));
     }
     BMG_CUDA(cudaGetLastError());
@@ -271,16 +271,19 @@ bmg_status invert_diagonals(Ctx& c) {
     return BMG_OK;
 }
 
-bool vcycle_forms_beta(const Ctx& c) { return c.dim == 2 && c.use_fused && c.nlev >= 2; }
+bool vcycle_forms_beta(const Ctx& c) {
+    return c.dim == 2 && c.use_fused && c.nlev >= 2 &&
+           2LL * c.fused[0].tiles_x * c.fused[0].tiles_y_up <= kMaxBlocks;
+}
 
 bmg_status vcycle_f32(Ctx& c, float* z32, const float* zold) {
     if (c.opts.precision != BMG_PREC_FP32) return BMG_ERR_STATE;
     if (c.dim == 3) return vcycle3d_impl<float>(c, c.r32, z32, nullptr);
-    if (c.use_fused && c.nlev >= 2) return vcycle2d_fused<float>(c, z32, true, zold);
+    if (c.use_fused && c.nlev >= 2) return vcycle2d_fused<float>(c, z32, true, zold, zold ? 2 : 0);
     return vcycle2d_impl<float>(c, c.r32, z32);
 }
 
-bmg_status vcycle(Ctx& c, const double* r, double* z) {
+bmg_status vcycle(Ctx& c, const double* r, double* z, const double* zold, int dots) {
     if (c.dim == 3) {
         if (c.opts.precision == BMG_PREC_FP64) return vcycle3d_impl<double>(c, r, z, nullptr);
         Level& F = c.lev[0];
@@ -293,8 +296,8 @@ bmg_status vcycle(Ctx& c, const double* r, double* z) {
     }
     if (c.use_fused && c.nlev >= 2) {
         if (r != c.r) return BMG_ERR_ARG;   // the level-0 tensor map streams c.r
-        if (c.opts.precision == BMG_PREC_FP64) return vcycle2d_fused<double>(c, z);
-        return vcycle2d_fused<float>(c, z);
+        if (c.opts.precision == BMG_PREC_FP64) return vcycle2d_fused<double>(c, z, false, zold, dots);
+        return vcycle2d_fused<float>(c, z, false, zold, dots);
     }
     if (c.opts.precision == BMG_PREC_FP64) return vcycle2d_impl<double>(c, r, z);
     Level& F = c.lev[0];
