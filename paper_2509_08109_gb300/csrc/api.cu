@@ -295,6 +295,7 @@ bmg_status pcg_ir(Ctx& c, double tol, int maxit, bmg_info* info) {
                 mm = std::min(std::max(8, m / 4), std::min(kMaxInner - done, maxit - it));
             }
             m = done;
+            if ((it & 1) == 1) BMG_TRY(k_flush_dr32(c));   // the last iteration was even
             BMG_TRY(k_residual_to32(c));
             BMG_TRY(read_state(c, h));
             refinements++;

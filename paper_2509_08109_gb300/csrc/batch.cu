@@ -119,6 +119,7 @@ bmg_status advance(Job& j, double tol, int maxit) {
     for (int k = 0; k < m; k++) BMG_TRY(run_iteration(c, (j.it + k) & 1));
     j.it += m;
     j.m = m;
+    if (j.it & 1) BMG_TRY(k_flush_dr32(c));   // the last iteration was even
     BMG_TRY(k_residual_to32(c));
     BMG_TRY(post_state_copy(j));
     j.phase = 2;

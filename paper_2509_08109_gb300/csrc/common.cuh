@@ -49,10 +49,11 @@ struct KState {
     double bb;        // ||b||^2
     double rr;        // ||r||^2 (last reduction)
     double rz;        // r.z of the previous iteration
-    double rzn;       // r.z of this iteration
+    double rzn;       // r.z of the first iteration of the current inner run (refinement mode)
     double rzo;       // r.z_old (flexible CG)
     double pq;        // p.Aq
     double alpha, beta;
+    double alpha0;    // refinement mode: step of the last even iteration, not yet in x
     double dot;       // scratch result of a plain dot product
     int err;          // first device error (bmg_status), 0 = none
     int first;        // 1 on the first iteration (p = z, no beta)
@@ -67,6 +68,7 @@ struct SysState {
     double rz;        // r.z of the previous inner iteration
     double pq;        // p.Ap
     double alpha, beta;
+    double alpha0;    // step of the last even iteration, not yet in x
     double rz0;       // r.z of the first inner iteration of the current run
     double stop;      // the run ends for this system once r.z <= stop * rz0 (0: it takes its full count)
     int first;        // 1: the next inner iteration takes p = z
@@ -227,6 +229,34 @@ cudaError_t launch_pdl(void (*kern)(KA...), dim3 grid, dim3 block, size_t smem, 
     cfg.attrs = &at;
     cfg.numAttrs = 1;
     return cudaLaunchKernelEx(&cfg, kern, KA(args)...);
+}
+
+// The four floats as doubles, exactly, by moving the fields of their binary32
+// encoding (a normal number: exponent rebiased by 1023 - 127 = 0x380, fraction
+// left-aligned; a zero keeps its sign).  Subnormal numbers, infinities and NaN,
+// which are rare here, take the conversion instruction: it runs in the FP64
+// units, of which an SM has two lanes' worth, and a vector update of FP32
+// directions into an FP64 iterate spends half of its FP64 slots on it.
+__host__ __device__ inline bool plain_f32(unsigned u) {   // zero or normal
+    const unsigned t = u & 0x7fffffffu;
+    return t == 0u || t - 0x00800000u < 0x7f000000u;
+}
+__host__ __device__ inline unsigned widen_hi(unsigned u) {
+    const unsigned t = u & 0x7fffffffu;
+    return (u & 0x80000000u) | (t ? (t >> 3) + 0x38000000u : 0u);
+}
+__host__ __device__ inline unsigned widen_lo(unsigned u) { return u << 29; }
+__device__ __forceinline__ void widen4(float4 v, double* d) {
+    const unsigned u[4] = {__float_as_uint(v.x), __float_as_uint(v.y), __float_as_uint(v.z), __float_as_uint(v.w)};
+    if (plain_f32(u[0]) && plain_f32(u[1]) && plain_f32(u[2]) && plain_f32(u[3])) {
+#pragma unroll
+        for (int q = 0; q < 4; q++) d[q] = __hiloint2double((int)widen_hi(u[q]), (int)widen_lo(u[q]));
+    } else {
+        d[0] = (double)v.x;
+        d[1] = (double)v.y;
+        d[2] = (double)v.z;
+        d[3] = (double)v.w;
+    }
 }
 
 inline int cdiv(long long a, long long b) { return (int)((a + b - 1) / b); }
@@ -435,7 +465,8 @@ bmg_status k_p_update(Ctx& c, const double* z);                   // p = z + bet
 bmg_status k_row_sums32(Ctx& c);                // rs32 = row sums of A (computed in FP64)
 bmg_status k_residual_to32(Ctx& c);             // r32 = (float)(b - A x); rr; resets the inner CG state
 bmg_status k_rz_beta32(Ctx& c, const float* z, const float* zo);
-bmg_status k_update_dr32(Ctx& c, int parity);    // x (FP64) += alpha p; r32 -= alpha q
+bmg_status k_update_dr32(Ctx& c, int parity);    // r32 -= alpha q; odd parity: x (FP64) += both iterations' alpha p
+bmg_status k_flush_dr32(Ctx& c);                 // x += the step an even last iteration left
 bmg_status node_tiles_prepare(Ctx& c);           // tile shape of the FP64 products and residuals
 bmg_status pspmv_prepare(Ctx& c);                // tile shape of the 2-D operator product
 bmg_status k_pspmv32(Ctx& c, const float* z, int parity);   // p = z + beta p_old; q = A p; alpha

@@ -29,7 +29,7 @@ __device__ __forceinline__ long long d3(int t, int ld, int n) {
 
 // sum_j a_ij x_j of row o (symmetric-half storage)
 template <int DIM, typename T>
-__device__ __forceinline__ T apply_row(const T* __restrict__ A, long long pl, int ld, int n, const T* __restrict__ x,
+__device__ __forceinline__ T apply_row(const T* __restrict__ A, long long pl, int ld, int n, const T* x,
                                        long long o) {
     if (DIM == 2) {
         T s = A[C2 * pl + o] * x[o];
@@ -58,7 +58,7 @@ __device__ __forceinline__ T apply_row(const T* __restrict__ A, long long pl, in
 // (A x)_o is zero and the FP64 products can be skipped, e.g. for a zero
 // initial guess, where the residual is b itself.
 template <int DIM, typename T>
-__device__ __forceinline__ bool row_x_zero(const T* __restrict__ x, int ld, int n, long long o) {
+__device__ __forceinline__ bool row_x_zero(const T* x, int ld, int n, long long o) {
     auto bits = [](T v) -> unsigned long long {
         return sizeof(T) == 8 ? (unsigned long long)__double_as_longlong((double)v) << 1
                               : (unsigned long long)__float_as_uint((float)v) << 1;
@@ -81,7 +81,7 @@ __device__ __forceinline__ bool row_x_zero(const T* __restrict__ x, int ld, int 
 // differences keep FP32 relative accuracy on every mode.
 template <int DIM>
 __device__ __forceinline__ float apply_row_diff(const float* __restrict__ A, const float* __restrict__ rs, long long pl,
-                                                int ld, int n, const float* __restrict__ x, long long o) {
+                                                int ld, int n, const float* x, long long o) {
     const float xo = x[o];
     float s = rs[o] * xo;
     if (DIM == 2) {
@@ -126,36 +126,104 @@ struct Acc32 {
     __device__ __forceinline__ double value() const { return (double)s + (double)c; }
 };
 
+// alpha = r.z / p.Ap once p.Ap is known (one thread), and the pending step
+__device__ __forceinline__ void set_alpha32(KState* st, double pq, int parity) {
+    st->pq = pq;
+    if (!(pq > 0.0)) {
+        set_err(st, BMG_ERR_NOT_SPD);
+        st->alpha = 0.0;
+    } else {
+        st->alpha = st->rz / pq;
+    }
+    if (parity == 0) st->alpha0 = st->alpha;
+}
+
 #define FOR_ROWS(g)                                                       \
     for (int r_ = blockIdx.x; r_ < (g).rows(); r_ += gridDim.x)           \
         for (int i_ = threadIdx.x; i_ < (g).ld; i_ += blockDim.x)
 
-// Interior nodes in tiles of 32 columns x 8 rows, H steps of a tile per CTA
-// (2-D: the next 8 rows; 3-D: the next plane).  A row-strided loop left up to
-// 40% of the FP64 lanes idle (127 interior columns on 160 padded ones and 256
-// threads), and FP64 lanes are what bounds the products below.  Boundary and
-// padding entries are zero in every array and stay as they are.
+// FP64 products with the operator over the interior nodes: f(k, (A x)_k) for
+// every node k.  With SKIP, rows whose x neighbourhood is +-0 (bit test, no
+// FP64 operation) give zero without the products, e.g. for a zero initial
+// guess.  FP64 lanes bound these kernels (a row-strided loop left up to 40% of
+// them idle on 127 interior columns of 160 padded ones), then the loads:
+//   2-D: tiles of 32 columns x 8 rows, H groups of 8 rows per CTA, a thread
+//     per node;
+//   3-D: tiles of 64 columns x 8 rows, H planes per CTA, a thread per column
+//     pair (i, i + 1), i even, so that the loads are two wide and the zero
+//     test reads nothing of its own.
+// Boundary and padding entries are zero in every array and stay as they are.
 template <int DIM>
 struct NodeTiles {
+    static constexpr int cols = DIM == 2 ? 32 : 64;
     int n, ld, H, ti, tj;
-    template <class F>
-    __device__ __forceinline__ void each(F&& f) const {
-        const int t = (int)blockIdx.x;
-        const int i = 1 + 32 * (t % ti) + (int)(threadIdx.x & 31);
-        const int ty = (int)(threadIdx.x >> 5);
-        if (i > n - 2) return;
-        if (DIM == 2) {
-            const int j0 = 1 + 8 * H * (t / ti) + ty;
+    template <bool SKIP, class F>
+    __device__ __forceinline__ void products(const double* __restrict__ A, long long pl, const double* x,
+                                             F&& f) const {
+        const int t = (int)blockIdx.x, lane = (int)(threadIdx.x & 31), row = (int)(threadIdx.x >> 5);
+        if constexpr (DIM == 2) {
+            const int i = 1 + 32 * (t % ti) + lane;
+            if (i > n - 2) return;
+            const int j0 = 1 + 8 * H * (t / ti) + row;
             for (int s = 0; s < H; s++) {
                 const int j = j0 + 8 * s;
                 if (j > n - 2) break;
-                f((long long)j * ld + i);
+                const long long k = (long long)j * ld + i;
+                f(k, SKIP && row_x_zero<2, double>(x, ld, n, k) ? 0.0 : apply_row<2, double>(A, pl, ld, n, x, k));
             }
         } else {
-            const int j = 1 + 8 * (t / ti % tj) + ty;
-            if (j > n - 2) return;
+            const int i = 64 * (t % ti) + 2 * lane, j = 1 + 8 * (t / ti % tj) + row;
+            if (i + 1 > n - 2 || j > n - 2) return;
             const int k0 = 1 + H * (t / (ti * tj));
-            for (int k = k0; k < k0 + H && k <= n - 2; k++) f((long long)i + (long long)ld * (j + (long long)n * k));
+            for (int k = k0; k < k0 + H && k <= n - 2; k++) {
+                const long long o = (long long)i + (long long)ld * (j + (long long)n * k);
+                double s0, s1;
+                apply_pair<SKIP>(A, pl, x, i, o, s0, s1);
+                if (i > 0) f(o, s0);
+                f(o + 1, s1);
+            }
+        }
+    }
+    // rows o and o + 1 of A x (3-D), in the order of apply_row
+    template <bool SKIP>
+    __device__ __forceinline__ void apply_pair(const double* __restrict__ A, long long pl, const double* x,
+                                               int i, long long o, double& s0, double& s1) const {
+        const long long sy = ld, sz = (long long)ld * n;
+        double X[3][3][4];      // [dz + 1][dy + 1]: columns i - 1 .. i + 2
+        unsigned long long m = 0;
+#pragma unroll
+        for (int z = 0; z < 3; z++)
+#pragma unroll
+            for (int y = 0; y < 3; y++) {
+                const double* q = x + o + (y - 1) * sy + (z - 1) * sz;
+                const double2 v = *reinterpret_cast<const double2*>(q);
+                X[z][y][0] = i > 0 ? q[-1] : 0.0;
+                X[z][y][1] = v.x;
+                X[z][y][2] = v.y;
+                X[z][y][3] = q[2];
+                if (SKIP)
+#pragma unroll
+                    for (int c = 0; c < 4; c++) m |= (unsigned long long)__double_as_longlong(X[z][y][c]) << 1;
+            }
+        s0 = s1 = 0.0;
+        if (SKIP && m == 0) return;
+        {
+            const double2 d = *reinterpret_cast<const double2*>(A + 13 * pl + o);
+            s0 = d.x * X[1][1][1];
+            s1 = d.y * X[1][1][2];
+        }
+#pragma unroll
+        for (int t = 0; t < 13; t++) {
+            const int dx = t % 3 - 1, dy = (t / 3) % 3 - 1, dz = t / 9 - 1;
+            const double2 own = *reinterpret_cast<const double2*>(A + t * pl + o);
+            const double* b = A + t * pl + o - dy * sy - dz * sz;   // the mirrors, stored at the node - d
+            const double2 mr = *reinterpret_cast<const double2*>(b);
+            const double m0 = dx == 0 ? mr.x : dx < 0 ? mr.y : i > 0 ? b[-1] : 0.0;
+            const double m1 = dx == 0 ? mr.y : dx < 0 ? b[2] : mr.x;
+            s0 += own.x * X[dz + 1][dy + 1][1 + dx];
+            s0 += m0 * X[1 - dz][1 - dy][1 - dx];
+            s1 += own.y * X[dz + 1][dy + 1][2 + dx];
+            s1 += m1 * X[1 - dz][1 - dy][2 - dx];
         }
     }
 };
@@ -182,12 +250,13 @@ __global__ void k_unpack_t(int n, int ld, const double* __restrict__ src, double
 // r = b - A x ; st.rr = ||r||^2 (rows with a zero x neighbourhood: r = b)
 template <int DIM>
 __global__ void __launch_bounds__(kThreads) k_residual64(NodeTiles<DIM> g, const double* __restrict__ A, long long pl,
-                                                         const double* __restrict__ b, const double* __restrict__ x,
+                                                         const double* b, const double* x,
                                                          double* __restrict__ r, double* partials, KState* st) {
+    pdl_wait();
+    pdl_trigger();
     double acc = 0.0;
-    g.each([&](long long k) {
-        const double v =
-            row_x_zero<DIM, double>(x, g.ld, g.n, k) ? b[k] : b[k] - apply_row<DIM, double>(A, pl, g.ld, g.n, x, k);
+    g.template products<true>(A, pl, x, [&](long long k, double ax) {
+        const double v = b[k] - ax;
         r[k] = v;
         acc += v * v;
     });
@@ -217,11 +286,12 @@ __global__ void __launch_bounds__(kThreads) k_dot64(long long pairs, const doubl
 // q = A p; st.pq = p.q; alpha = rz / pq
 template <int DIM>
 __global__ void __launch_bounds__(kThreads) k_spmv_pq64(NodeTiles<DIM> g, const double* __restrict__ A, long long pl,
-                                                        const double* __restrict__ p, double* __restrict__ q,
+                                                        const double* p, double* __restrict__ q,
                                                         double* partials, KState* st) {
+    pdl_wait();
+    pdl_trigger();
     double acc = 0.0;
-    g.each([&](long long k) {
-        const double v = apply_row<DIM, double>(A, pl, g.ld, g.n, p, k);
+    g.template products<false>(A, pl, p, [&](long long k, double v) {
         q[k] = v;
         acc += p[k] * v;
     });
@@ -239,9 +309,11 @@ __global__ void __launch_bounds__(kThreads) k_spmv_pq64(NodeTiles<DIM> g, const 
 
 // x += alpha p; r -= alpha q; st.rr = ||r||^2
 __global__ void __launch_bounds__(kThreads) k_update_xr64(long long pairs, double2* __restrict__ x,
-                                                          double2* __restrict__ r, const double2* __restrict__ p,
-                                                          const double2* __restrict__ q, double* partials,
+                                                          double2* __restrict__ r, const double2* p,
+                                                          const double2* q, double* partials,
                                                           KState* st) {
+    pdl_wait();
+    pdl_trigger();
     const double alpha = st->alpha;
     double acc = 0.0;
     for (long long k = blockIdx.x * (long long)blockDim.x + threadIdx.x; k < pairs;
@@ -264,10 +336,12 @@ __global__ void __launch_bounds__(kThreads) k_update_xr64(long long pairs, doubl
 // r.z and (flexible) r.z_old in one pass, then beta in the last block; the
 // first iteration has no beta.
 template <bool FLEX>
-__global__ void __launch_bounds__(kThreads) k_rz_beta64(long long pairs, const double2* __restrict__ r,
-                                                        const double2* __restrict__ z,
-                                                        const double2* __restrict__ zo, double* partials,
+__global__ void __launch_bounds__(kThreads) k_rz_beta64(long long pairs, const double2* r,
+                                                        const double2* z,
+                                                        const double2* zo, double* partials,
                                                         KState* st) {
+    pdl_wait();
+    pdl_trigger();
     double a1 = 0.0, a2 = 0.0;
     for (long long k = blockIdx.x * (long long)blockDim.x + threadIdx.x; k < pairs;
          k += (long long)gridDim.x * blockDim.x) {
@@ -295,8 +369,10 @@ __global__ void __launch_bounds__(kThreads) k_rz_beta64(long long pairs, const d
 }
 
 // p = z + beta p
-__global__ void __launch_bounds__(kThreads) k_p_update64(long long pairs, const double2* __restrict__ z,
+__global__ void __launch_bounds__(kThreads) k_p_update64(long long pairs, const double2* z,
                                                          double2* __restrict__ p, KState* st) {
+    pdl_wait();
+    pdl_trigger();
     const double beta = st->beta;
     for (long long k = blockIdx.x * (long long)blockDim.x + threadIdx.x; k < pairs;
          k += (long long)gridDim.x * blockDim.x) {
@@ -314,13 +390,14 @@ __global__ void __launch_bounds__(kThreads) k_p_update64(long long pairs, const 
 // (the FP64 rate, not HBM, bounds this kernel otherwise).
 template <int DIM>
 __global__ void __launch_bounds__(kThreads) k_residual_to32_t(NodeTiles<DIM> g, const double* __restrict__ A,
-                                                              long long pl, const double* __restrict__ b,
-                                                              const double* __restrict__ x, float* __restrict__ r32,
+                                                              long long pl, const double* b,
+                                                              const double* x, float* __restrict__ r32,
                                                               double* partials, KState* st) {
+    pdl_wait();
+    pdl_trigger();
     double acc = 0.0;
-    g.each([&](long long k) {
-        const double v =
-            row_x_zero<DIM, double>(x, g.ld, g.n, k) ? b[k] : b[k] - apply_row<DIM, double>(A, pl, g.ld, g.n, x, k);
+    g.template products<true>(A, pl, x, [&](long long k, double ax) {
+        const double v = b[k] - ax;
         r32[k] = (float)v;
         acc += v * v;
     });
@@ -328,6 +405,7 @@ __global__ void __launch_bounds__(kThreads) k_residual_to32_t(NodeTiles<DIM> g, 
     if (grid_sum(acc, partials, &st->counter[0], &t)) {
         st->rr = t;
         st->first = 1;
+        st->alpha0 = 0.0;
     }
 }
 
@@ -346,8 +424,10 @@ __global__ void k_row_sums32_t(RowGrid<DIM> g, const double* __restrict__ A, lon
 // p_old, so p is written to a second buffer (p_old is still being read).
 template <int DIM>
 __global__ void k_pspmv32_t(RowGrid<DIM> g, const float* __restrict__ A, const float* __restrict__ rs, long long pl,
-                            const float* __restrict__ z, const float* __restrict__ pold, float* __restrict__ p,
-                            float* __restrict__ q, double* partials, KState* st) {
+                            const float* z, const float* pold, float* __restrict__ p,
+                            float* __restrict__ q, double* partials, KState* st, int parity) {
+    pdl_wait();
+    pdl_trigger();
     const float beta = (float)st->beta;
     Acc32 acc;
     FOR_ROWS(g) {
@@ -383,49 +463,81 @@ __global__ void k_pspmv32_t(RowGrid<DIM> g, const float* __restrict__ A, const f
     }
     double t;
     if (grid_sum(acc.value(), partials, &st->counter[2], &t)) {
-        st->pq = t;
-        if (!(t > 0.0)) {
-            set_err(st, BMG_ERR_NOT_SPD);
-            st->alpha = 0.0;
-        } else {
-            st->alpha = st->rz / t;
-        }
+        set_alpha32(st, t, parity);
     }
 }
 
 // x += alpha p straight into the FP64 iterate (an FP32 correction would cap
 // the true residual near eps_32 ||A|| ||d|| / ||A d||, far above 1e-10 for a
-// smooth correction d); r -= alpha q in FP32.
+// smooth correction d); r -= alpha q in FP32.  The FP64 iterate is touched
+// every other iteration: an even one (PARITY 0) updates r alone and leaves its
+// alpha in alpha0 (the product kernel puts it there), the odd one adds both
+// steps, and k_flush_x32 adds what an odd count leaves.  24 instead of 32 bytes
+// a node and iteration.  4097^2: 114 us a pair of iterations, 2 x 88 with x in
+// every iteration; 157 with the conversion instruction in place of widen4,
+// whose slots in the FP64 units then bound the odd iterations.
+__device__ __forceinline__ void add_step(double2& x0, double2& x1, double alpha, float4 p) {
+    double d[4];
+    widen4(p, d);
+    x0.x += alpha * d[0];
+    x0.y += alpha * d[1];
+    x1.x += alpha * d[2];
+    x1.y += alpha * d[3];
+}
+
+template <int PARITY>
 __global__ void __launch_bounds__(kThreads) k_update_xr32(long long quads, double2* __restrict__ x,
-                                                          float4* __restrict__ r, const float4* __restrict__ p,
-                                                          const float4* __restrict__ q, const KState* st) {
-    const double alpha = st->alpha;
+                                                          float4* __restrict__ r, const float4* p0,
+                                                          const float4* p1,
+                                                          const float4* q, const KState* st) {
+    pdl_wait();
+    pdl_trigger();
+    const double alpha = st->alpha, alpha0 = st->alpha0;
     const float a32 = (float)alpha;
     for (long long k = blockIdx.x * (long long)blockDim.x + threadIdx.x; k < quads;
          k += (long long)gridDim.x * blockDim.x) {
-        const float4 pv = p[k], qv = q[k];
+        const float4 qv = q[k];
         float4 rv = r[k];
-        double2 x0 = x[2 * k], x1 = x[2 * k + 1];
-        x0.x += alpha * (double)pv.x;
-        x0.y += alpha * (double)pv.y;
-        x1.x += alpha * (double)pv.z;
-        x1.y += alpha * (double)pv.w;
+        if (PARITY) {
+            const float4 pv = p1[k];
+            double2 x0 = x[2 * k], x1 = x[2 * k + 1];
+            if (alpha0 != 0.0) add_step(x0, x1, alpha0, p0[k]);
+            add_step(x0, x1, alpha, pv);
+            x[2 * k] = x0;
+            x[2 * k + 1] = x1;
+        }
         rv.x -= a32 * qv.x;
         rv.y -= a32 * qv.y;
         rv.z -= a32 * qv.z;
         rv.w -= a32 * qv.w;
+        r[k] = rv;
+    }
+}
+
+// x += alpha0 p0: the step an even iteration left at the end of a run
+__global__ void __launch_bounds__(kThreads) k_flush_x32(long long quads, double2* __restrict__ x,
+                                                        const float4* p0, const KState* st) {
+    pdl_wait();
+    pdl_trigger();
+    const double alpha0 = st->alpha0;
+    if (alpha0 == 0.0) return;
+    for (long long k = blockIdx.x * (long long)blockDim.x + threadIdx.x; k < quads;
+         k += (long long)gridDim.x * blockDim.x) {
+        double2 x0 = x[2 * k], x1 = x[2 * k + 1];
+        add_step(x0, x1, alpha0, p0[k]);
         x[2 * k] = x0;
         x[2 * k + 1] = x1;
-        r[k] = rv;
     }
 }
 
 // r.z and r.z_old in one pass; the last block forms the flexible-CG beta.
 // Four values a load, two CTAs per SM (as the FP64 vector kernels).
-__global__ void __launch_bounds__(kThreads) k_rz_beta32_t(long long quads, const float4* __restrict__ r,
-                                                          const float4* __restrict__ z,
-                                                          const float4* __restrict__ zo, double* partials,
+__global__ void __launch_bounds__(kThreads) k_rz_beta32_t(long long quads, const float4* r,
+                                                          const float4* z,
+                                                          const float4* zo, double* partials,
                                                           KState* st) {
+    pdl_wait();
+    pdl_trigger();
     Acc32 a1, a2;
     for (long long k = blockIdx.x * (long long)blockDim.x + threadIdx.x; k < quads;
          k += (long long)gridDim.x * blockDim.x) {
@@ -444,6 +556,7 @@ __global__ void __launch_bounds__(kThreads) k_rz_beta32_t(long long quads, const
         if (st->first) {
             st->beta = 0.0;
             st->first = 0;
+            st->rzn = t1;   // the run's first r.z, for the host's prediction
         } else {
             st->beta = (t1 - t2) / st->rz;
         }
@@ -471,11 +584,11 @@ inline double dofs0(const Ctx& c) {
     do {                                                                                                   \
         const Level& L_ = (c).lev[0];                                                                      \
         if ((c).dim == 2)                                                                                  \
-            KERNEL<2><<<(c).nt_tiles, kThreads, 0, (c).stream>>>(                                          \
-                NodeTiles<2>{L_.n, L_.ld, (c).nt_h, (c).nt_i, (c).nt_j}, __VA_ARGS__);                     \
+            BMG_CUDA(launch_pdl(KERNEL<2>, dim3((c).nt_tiles), dim3(kThreads), 0, (c).stream,              \
+                                NodeTiles<2>{L_.n, L_.ld, (c).nt_h, (c).nt_i, (c).nt_j}, __VA_ARGS__));    \
         else                                                                                               \
-            KERNEL<3><<<(c).nt_tiles, kThreads, 0, (c).stream>>>(                                          \
-                NodeTiles<3>{L_.n, L_.ld, (c).nt_h, (c).nt_i, (c).nt_j}, __VA_ARGS__);                     \
+            BMG_CUDA(launch_pdl(KERNEL<3>, dim3((c).nt_tiles), dim3(kThreads), 0, (c).stream,              \
+                                NodeTiles<3>{L_.n, L_.ld, (c).nt_h, (c).nt_i, (c).nt_j}, __VA_ARGS__));    \
         (c).launches++;                                                                                    \
     } while (0)
 
@@ -494,7 +607,8 @@ inline int vec_blocks(const Ctx& c) {
 bmg_status node_tiles_prepare(Ctx& c) {
     BMG_CUDA(cudaDeviceGetAttribute(&c.sms, cudaDevAttrMultiProcessorCount, c.device));
     const int m = c.lev[0].n - 2;
-    const int ti = cdiv(m, 32), tj = cdiv(m, 8), steps = c.dim == 2 ? tj : m;
+    const int ti = c.dim == 2 ? cdiv(m, NodeTiles<2>::cols) : cdiv(m + 1, NodeTiles<3>::cols);   // 3-D from column 0
+    const int tj = cdiv(m, 8), steps = c.dim == 2 ? tj : m;
     const long long cols = c.dim == 2 ? ti : (long long)ti * tj;
     long long best = -1;
     for (int h = 1; h <= steps; h++) {
@@ -562,9 +676,8 @@ bmg_status k_spmv_pq(Ctx& c, const double* p, double* q) {
 bmg_status k_update_xr(Ctx& c) {
     const Level& L = c.lev[0];
     prof_begin(c, BMG_PROF_UPDATE, 0);
-    k_update_xr64<<<vec_blocks(c), kThreads, 0, c.stream>>>(L.plane / 2, (double2*)c.x, (double2*)c.r,
-                                                            (const double2*)c.p, (const double2*)c.q, c.partials,
-                                                            c.st);
+    BMG_CUDA(launch_pdl(k_update_xr64, dim3(vec_blocks(c)), dim3(kThreads), 0, c.stream, L.plane / 2, (double2*)c.x,
+                        (double2*)c.r, (const double2*)c.p, (const double2*)c.q, c.partials, c.st));
     prof_end(c, BMG_PROF_UPDATE, 0, 6 * 8.0 * dofs0(c));
     c.launches++;
     BMG_CUDA(cudaGetLastError());
@@ -575,9 +688,11 @@ bmg_status k_rz_beta(Ctx& c, const double* z, const double* zold, bool flexible)
     const Level& L = c.lev[0];
     const double2 *r2 = (const double2*)c.r, *z2 = (const double2*)z, *o2 = (const double2*)zold;
     if (flexible)
-        k_rz_beta64<true><<<vec_blocks(c), kThreads, 0, c.stream>>>(L.plane / 2, r2, z2, o2, c.partials, c.st);
+        BMG_CUDA(launch_pdl(k_rz_beta64<true>, dim3(vec_blocks(c)), dim3(kThreads), 0, c.stream, L.plane / 2, r2, z2, o2,
+                            c.partials, c.st));
     else
-        k_rz_beta64<false><<<vec_blocks(c), kThreads, 0, c.stream>>>(L.plane / 2, r2, z2, o2, c.partials, c.st);
+        BMG_CUDA(launch_pdl(k_rz_beta64<false>, dim3(vec_blocks(c)), dim3(kThreads), 0, c.stream, L.plane / 2, r2, z2,
+                            o2, c.partials, c.st));
     c.launches++;
     BMG_CUDA(cudaGetLastError());
     return BMG_OK;
@@ -586,8 +701,8 @@ bmg_status k_rz_beta(Ctx& c, const double* z, const double* zold, bool flexible)
 bmg_status k_p_update(Ctx& c, const double* z) {
     const Level& L = c.lev[0];
     const int blocks = cdiv(L.plane / 2, 2 * kThreads);
-    k_p_update64<<<blocks < c.red_blocks ? blocks : c.red_blocks, kThreads, 0, c.stream>>>(
-        L.plane / 2, (const double2*)z, (double2*)c.p, c.st);
+    BMG_CUDA(launch_pdl(k_p_update64, dim3(blocks < c.red_blocks ? blocks : c.red_blocks), dim3(kThreads), 0, c.stream,
+                        L.plane / 2, (const double2*)z, (double2*)c.p, c.st));
     c.launches++;
     BMG_CUDA(cudaGetLastError());
     return BMG_OK;
@@ -600,120 +715,142 @@ bmg_status k_residual_to32(Ctx& c) {
     return BMG_OK;
 }
 
-// 2-D form of k_pspmv32_t: one CTA per tile of kThreads interior columns x H
-// rows, marching up the rows.  Every value of z, p_old and of the stored
-// planes is loaded once (plus a one-column, two-row halo) into a four-row
-// ring in shared memory; the loads of row j+2 are in flight while row j is
-// formed, with one barrier per row.  Same arithmetic, in the same order, as
-// k_pspmv32_t<2>.
-__global__ void __launch_bounds__(kThreads) k_pspmv2d_tiled(int n, int ld, long long pl, int H, int tiles_x,
-                                                            const float* __restrict__ A,
-                                                            const float* __restrict__ rs,
-                                                            const float* __restrict__ z,
-                                                            const float* __restrict__ pold, float* __restrict__ p,
-                                                            float* __restrict__ q, double* partials, KState* st) {
-    constexpr int TW = kThreads;
-    __shared__ float sP[4][TW + 2];    // p at columns i0-1 .. i0+TW
-    __shared__ float sW[4][TW + 1];    // stored planes at columns i0 .. i0+TW
-    __shared__ float sSW[4][TW + 1];
-    __shared__ float sNW[4][TW + 1];
+// 2-D form of k_pspmv32_t: a warp owns a strip of 64 columns and a band of H
+// rows and marches up the rows on its own, without barriers.  A lane holds the
+// column pair (i, i + 1), i even, of the three rows in play in registers (p and
+// the planes' values, loaded two wide); its neighbours' columns come by
+// shuffle, and lanes 0 and 31 load the strip's edge columns.  The next row's
+// raw values (z, p_old, planes) are in flight while a row is formed.  HBM
+// bounds the kernel on large grids (36 bytes a node), the chain of row loads
+// on small ones.  4097^2: 120 us, 65^2: 6.8 us, against 129 and 8.1 us for a
+// thread per column, a block barrier per row and the planes in shared memory.
+// Same arithmetic, in the same order, as k_pspmv32_t<2>.
+__global__ void __launch_bounds__(kThreads) k_pspmv2d_strips(int n, int ld, long long pl, int H, int strips, int bands,
+                                                             const float* __restrict__ A,
+                                                             const float* __restrict__ rs, const float* z,
+                                                             const float* pold, float* __restrict__ p,
+                                                             float* __restrict__ q, double* partials, KState* st,
+                                                             int parity) {
+    pdl_wait();
+    pdl_trigger();
     const float beta = (float)st->beta;
-    const int t = threadIdx.x;
-    const int i0 = 1 + (int)(blockIdx.x % tiles_x) * TW;
-    const int j0 = 1 + (int)(blockIdx.x / tiles_x) * H;
-    const int j1 = min(j0 + H, n - 1);
-    const int i = i0 + t;
-    const bool act = i <= n - 2;
-    const int il = i0 - 1, ir = i0 + TW;    // halo columns (thread 0: left, thread 1: right)
-    // raw loads only: p = z + beta p_old is formed when the row is stored,
-    // a step later, so no instruction waits on these loads before the
-    // current row has been computed
-    struct Row {
-        float z, po, w, sw, nw, s, r, hz, hpo, hw, hsw, hnw;
-    };
-    auto load = [&](int j, Row& v) {
-        v = Row{0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-        if (j < 1 || j > n - 2) return;
-        const long long kr = (long long)j * ld;
-        if (act) {
-            const long long k = kr + i;
-            v.z = z[k];
-            v.po = pold[k];
-            v.w = A[W2 * pl + k];
-            v.sw = A[SW2 * pl + k];
-            v.nw = A[NW2 * pl + k];
-            v.s = A[S2 * pl + k];
-            v.r = rs[k];
-        }
-        if (t == 0 && il >= 1) {
-            v.hz = z[kr + il];
-            v.hpo = pold[kr + il];
-        }
-        if (t == 1 && ir <= n - 2) {
-            const long long k = kr + ir;
-            v.hz = z[k];
-            v.hpo = pold[k];
-            v.hw = A[W2 * pl + k];
-            v.hsw = A[SW2 * pl + k];
-            v.hnw = A[NW2 * pl + k];
-        }
-    };
-    auto put = [&](int j, const Row& v) {
-        const int sl = j & 3;
-        sP[sl][t + 1] = v.z + beta * v.po;
-        sW[sl][t] = v.w;
-        sSW[sl][t] = v.sw;
-        sNW[sl][t] = v.nw;
-        if (t == 0) sP[sl][0] = v.hz + beta * v.hpo;
-        if (t == 1) {
-            sP[sl][TW + 1] = v.hz + beta * v.hpo;
-            sW[sl][TW] = v.hw;
-            sSW[sl][TW] = v.hsw;
-            sNW[sl][TW] = v.hnw;
-        }
-    };
-    Row nx;
-    load(j0 - 1, nx);
-    put(j0 - 1, nx);
-    load(j0, nx);
-    put(j0, nx);
-    float rs_j = nx.r, s_j = nx.s;
-    load(j0 + 1, nx);
+    const int lane = threadIdx.x & 31;
+    const int g = blockIdx.x * (kThreads / 32) + (threadIdx.x >> 5);
+    const int strip = g % strips, band = g / strips;
     Acc32 acc;
-    for (int j = j0; j < j1; j++) {
-        put(j + 1, nx);
-        const float s_n = nx.s, rs_n = nx.r;
-        load(j + 2, nx);
-        __syncthreads();
-        if (act) {
-            const int sm = (j - 1) & 3, s0 = j & 3, sp = (j + 1) & 3;
-            const float pv = sP[s0][t + 1];
-            float v = rs_j * pv;
-            v += sW[s0][t] * (sP[s0][t] - pv);
-            v += sW[s0][t + 1] * (sP[s0][t + 2] - pv);
-            v += s_j * (sP[sm][t + 1] - pv);
-            v += s_n * (sP[sp][t + 1] - pv);
-            v += sSW[s0][t] * (sP[sm][t] - pv);
-            v += sSW[sp][t + 1] * (sP[sp][t + 2] - pv);
-            v += sNW[s0][t] * (sP[sp][t] - pv);
-            v += sNW[sm][t + 1] * (sP[sm][t + 2] - pv);
+    if (band < bands) {
+        const int j0 = 1 + band * H, j1 = min(j0 + H, n - 1);
+        const int i = 64 * strip + 2 * lane;
+        const bool act0 = i >= 1 && i <= n - 2, act1 = i + 1 <= n - 2;   // act0 implies act1 (n is odd)
+        // raw values of a row: the pair's, and the edge column of lane 0 (left)
+        // or lane 31 (right)
+        struct Raw {
+            float2 z, po, w, s, sw, nw, r;
+            float ez, ep, ew, esw, enw;
+        };
+        const int ie = lane == 0 ? i - 1 : i + 2;
+        const bool edge = lane == 0 ? i >= 2 : lane == 31 && ie <= n - 2;
+        auto load = [&](int j, Raw& v) {
+            v = Raw{};
+            if (j < 1 || j > n - 2) return;
+            const long long kr = (long long)j * ld;
+            if (act1) {
+                const long long k = kr + i;
+                v.z = *reinterpret_cast<const float2*>(z + k);
+                v.po = *reinterpret_cast<const float2*>(pold + k);
+                v.w = *reinterpret_cast<const float2*>(A + W2 * pl + k);
+                v.s = *reinterpret_cast<const float2*>(A + S2 * pl + k);
+                v.sw = *reinterpret_cast<const float2*>(A + SW2 * pl + k);
+                v.nw = *reinterpret_cast<const float2*>(A + NW2 * pl + k);
+                v.r = *reinterpret_cast<const float2*>(rs + k);
+            }
+            if (edge) {
+                const long long k = kr + ie;
+                v.ez = z[k];
+                v.ep = pold[k];
+                if (lane == 31) {
+                    v.ew = A[W2 * pl + k];
+                    v.esw = A[SW2 * pl + k];
+                    v.enw = A[NW2 * pl + k];
+                }
+            }
+        };
+        // p at columns i-1 .. i+2, W, SW, NW at i .. i+2, S and row sums at i, i+1
+        struct Row {
+            float pl, p0, p1, pr, w0, w1, w2, sw0, sw1, sw2, nw0, nw1, nw2, s0, s1, r0, r1;
+        };
+        auto form = [&](const Raw& v) {
+            Row r;
+            r.p0 = v.z.x + beta * v.po.x;
+            r.p1 = v.z.y + beta * v.po.y;
+            const float e = v.ez + beta * v.ep;
+            r.pl = __shfl_up_sync(0xffffffffu, r.p1, 1);
+            r.pr = __shfl_down_sync(0xffffffffu, r.p0, 1);
+            r.w2 = __shfl_down_sync(0xffffffffu, v.w.x, 1);
+            r.sw2 = __shfl_down_sync(0xffffffffu, v.sw.x, 1);
+            r.nw2 = __shfl_down_sync(0xffffffffu, v.nw.x, 1);
+            if (lane == 0) r.pl = e;
+            if (lane == 31) {
+                r.pr = e;
+                r.w2 = v.ew;
+                r.sw2 = v.esw;
+                r.nw2 = v.enw;
+            }
+            r.w0 = v.w.x;
+            r.w1 = v.w.y;
+            r.sw0 = v.sw.x;
+            r.sw1 = v.sw.y;
+            r.nw0 = v.nw.x;
+            r.nw1 = v.nw.y;
+            r.s0 = v.s.x;
+            r.s1 = v.s.y;
+            r.r0 = v.r.x;
+            r.r1 = v.r.y;
+            return r;
+        };
+        Raw va, vb, vc;
+        load(j0 - 1, va);
+        load(j0, vb);
+        load(j0 + 1, vc);
+        Row rm = form(va), r0 = form(vb);
+        for (int j = j0; j < j1; j++) {
+            const Row rp = form(vc);
+            load(j + 2, vc);
+            float u = r0.r0 * r0.p0, v = r0.r1 * r0.p1;
+            u += r0.w0 * (r0.pl - r0.p0);
+            v += r0.w1 * (r0.p0 - r0.p1);
+            u += r0.w1 * (r0.p1 - r0.p0);
+            v += r0.w2 * (r0.pr - r0.p1);
+            u += r0.s0 * (rm.p0 - r0.p0);
+            v += r0.s1 * (rm.p1 - r0.p1);
+            u += rp.s0 * (rp.p0 - r0.p0);
+            v += rp.s1 * (rp.p1 - r0.p1);
+            u += r0.sw0 * (rm.pl - r0.p0);
+            v += r0.sw1 * (rm.p0 - r0.p1);
+            u += rp.sw1 * (rp.p1 - r0.p0);
+            v += rp.sw2 * (rp.pr - r0.p1);
+            u += r0.nw0 * (rp.pl - r0.p0);
+            v += r0.nw1 * (rp.p0 - r0.p1);
+            u += rm.nw1 * (rm.p1 - r0.p0);
+            v += rm.nw2 * (rm.pr - r0.p1);
             const long long k = (long long)j * ld + i;
-            p[k] = pv;
-            q[k] = v;
-            acc.add(pv * v);
+            if (act0) {
+                *reinterpret_cast<float2*>(p + k) = make_float2(r0.p0, r0.p1);
+                *reinterpret_cast<float2*>(q + k) = make_float2(u, v);
+                acc.add(r0.p0 * u);
+                acc.add(r0.p1 * v);
+            } else if (act1) {      // the boundary column and the first interior one
+                p[k + 1] = r0.p1;
+                q[k + 1] = v;
+                acc.add(r0.p1 * v);
+            }
+            rm = r0;
+            r0 = rp;
         }
-        rs_j = rs_n;
-        s_j = s_n;
     }
     double tot;
     if (grid_sum(acc.value(), partials, &st->counter[2], &tot)) {
-        st->pq = tot;
-        if (!(tot > 0.0)) {
-            set_err(st, BMG_ERR_NOT_SPD);
-            st->alpha = 0.0;
-        } else {
-            st->alpha = st->rz / tot;
-        }
+        set_alpha32(st, tot, parity);
     }
 }
 
@@ -726,70 +863,73 @@ bmg_status k_row_sums32(Ctx& c) {
 
 bmg_status k_rz_beta32(Ctx& c, const float* z, const float* zo) {
     const Level& L = c.lev[0];
-    k_rz_beta32_t<<<vec_blocks(c), kThreads, 0, c.stream>>>(L.plane / 4, (const float4*)c.r32, (const float4*)z,
-                                                            (const float4*)zo, c.partials, c.st);
+    BMG_CUDA(launch_pdl(k_rz_beta32_t, dim3(vec_blocks(c)), dim3(kThreads), 0, c.stream, L.plane / 4,
+                        (const float4*)c.r32, (const float4*)z, (const float4*)zo, c.partials, c.st));
     c.launches++;
     BMG_CUDA(cudaGetLastError());
     return BMG_OK;
 }
 
-// 3-D form of k_pspmv32_t: one CTA per tile of 32 x 8 (i, j) interior nodes
-// and a band of k-planes, marching up k; p of the next k-plane, with a
-// one-node halo in i and j, goes from registers (loaded a step ahead) into a
-// shared ring of 4 slots, so one barrier per plane suffices.
-constexpr int kP3I = 32, kP3J = 8;
-constexpr int kP3W = kP3I + 2, kP3H = kP3J + 2, kP3A = kP3W * kP3H;   // halo tile
-constexpr int kP3Per = (kP3A + kThreads - 1) / kThreads;              // halo positions per thread
+// 3-D form of k_pspmv32_t: one CTA per tile of 64 columns x 8 rows and a band
+// of k-planes, marching up k; p of the next plane, with a halo of one row and
+// one column pair, goes from registers (loaded a step ahead) into a shared
+// ring of 4 slots, so one barrier per plane suffices.
+//
+// A thread forms the column pair (i, i + 1), i even: its two nodes' 13 stored
+// planes and 13 mirrors a(-d) (stored at the node - d) are two-wide loads
+// straight from global memory, issued before the step's barrier so that they
+// overlap the wait; the mirrors are other threads' own values, served by L1
+// and L2.  HBM bounds the kernel (72 bytes a node).  257^3: 214 us, against
+// 252 us with a thread per node and one-wide loads.  Same products in the same
+// order as k_pspmv32_t<3>.
+constexpr int kP3I = 64, kP3J = 8;
+constexpr int kP3Pairs = kP3I / 2 + 2, kP3W = 2 * kP3Pairs, kP3H = kP3J + 2;   // halo tile: pairs a row, columns, rows
+constexpr int kP3A = kP3W * kP3H;
+constexpr int kP3Per = (kP3Pairs * kP3H + kThreads - 1) / kThreads;           // halo pairs per thread
 
-// The stencil is read straight from global memory: each thread loads its
-// node's 13 stored planes and the 13 mirrors a(-d) (stored at the node - d)
-// into registers before the step's barrier, so the loads overlap the wait;
-// the mirrors of the CTA's interior are its own threads' loads of a
-// neighbouring row or of the next plane, served by L1 and L2.  Only p lives
-// in shared memory, so the CTA's footprint is a few KB and occupancy is set
-// by registers (64 per thread, 4 CTAs per SM).  A version that staged the 13
-// planes in shared rings as well (58 KB per CTA, 3 CTAs per SM) took 349
-// instead of 253 us per 257^3 product.  Same products in the same order as
-// k_pspmv32_t<3>.
 __global__ void __launch_bounds__(kThreads) k_pspmv3d_direct(int n, int ld, long long pl, int H, int tiles_i,
                                                              int tiles_j, const float* __restrict__ A,
                                                              const float* __restrict__ rs,
-                                                             const float* __restrict__ z,
-                                                             const float* __restrict__ pold, float* __restrict__ p,
-                                                             float* __restrict__ q, double* partials, KState* st) {
-    __shared__ float sP[4][kP3A];
+                                                             const float* z,
+                                                             const float* pold, float* __restrict__ p,
+                                                             float* __restrict__ q, double* partials, KState* st,
+                                                             int parity) {
+    __shared__ __align__(8) float sP[4][kP3A];
+    pdl_wait();
+    pdl_trigger();
     const float beta = (float)st->beta;
     const int tid = threadIdx.x;
     const int tile = blockIdx.x;
     const int ti = tile % tiles_i, tj = (tile / tiles_i) % tiles_j, tk = tile / (tiles_i * tiles_j);
-    const int i0 = 1 + ti * kP3I, j0 = 1 + tj * kP3J, k0 = 1 + tk * H;
+    const int i0 = ti * kP3I, j0 = 1 + tj * kP3J, k0 = 1 + tk * H;
     const int k1 = min(k0 + H, n - 1);
-    const long long sz = (long long)ld * n;
-    float rz[kP3Per], rpo[kP3Per];
+    const long long sy = ld, sz = (long long)ld * n;
+    // halo pair u of the thread: columns i0 - 2 + 2 hp, row j0 - 1 + hj
+    float2 rz[kP3Per], rpo[kP3Per];
     auto load = [&](int k) {
 #pragma unroll
         for (int u = 0; u < kP3Per; u++) {
             const int h = tid + u * kThreads;
-            const int hi = h % kP3W, hj = h / kP3W;
-            const int i = i0 - 1 + hi, j = j0 - 1 + hj;
-            const bool in = h < kP3A && i <= n - 1 && j <= n - 1 && k >= 0 && k <= n - 1;
-            const long long o = in ? (long long)i + (long long)ld * j + sz * k : 0;
-            rz[u] = in ? z[o] : 0.f;
-            rpo[u] = in ? pold[o] : 0.f;
+            const int hp = h % kP3Pairs, hj = h / kP3Pairs;
+            const int i = i0 - 2 + 2 * hp, j = j0 - 1 + hj;
+            const bool in = hj < kP3H && i >= 0 && i + 1 < ld && j <= n - 1 && k <= n - 1;
+            const long long o = in ? (long long)i + sy * j + sz * k : 0;
+            rz[u] = in ? *reinterpret_cast<const float2*>(z + o) : make_float2(0.f, 0.f);
+            rpo[u] = in ? *reinterpret_cast<const float2*>(pold + o) : make_float2(0.f, 0.f);
         }
     };
     auto put = [&](int k) {
-        float* pp = sP[k & 3];
+        float2* pp = reinterpret_cast<float2*>(sP[k & 3]);
 #pragma unroll
         for (int u = 0; u < kP3Per; u++) {
             const int h = tid + u * kThreads;
-            if (h < kP3A) pp[h] = rz[u] + beta * rpo[u];
+            if (h < kP3Pairs * kP3H) pp[h] = make_float2(rz[u].x + beta * rpo[u].x, rz[u].y + beta * rpo[u].y);
         }
     };
-    const int ti_ = tid % kP3I, tj_ = tid / kP3I;
-    const int i = i0 + ti_, j = j0 + tj_;
-    const bool act = i <= n - 2 && j <= n - 2;
-    const int hc = (tj_ + 1) * kP3W + (ti_ + 1);
+    const int lane = tid & 31, row = tid >> 5;
+    const int i = i0 + 2 * lane, j = j0 + row;
+    const bool act0 = i >= 1 && i <= n - 2 && j <= n - 2, act1 = i + 1 <= n - 2 && j <= n - 2;
+    const int hc = (row + 1) * kP3W + 2 * (lane + 1);
     load(k0 - 1);
     put(k0 - 1);
     load(k0);
@@ -799,52 +939,60 @@ __global__ void __launch_bounds__(kThreads) k_pspmv3d_direct(int n, int ld, long
     for (int k = k0; k < k1; k++) {
         put(k + 1);
         load(k + 2);
-        const long long o = (long long)i + (long long)ld * j + sz * k;
-        float a0[13], am[13], rsv = 0.f;
-        if (act) {
+        const long long o = (long long)i + sy * j + sz * k;
+        float2 a0[13], am[13];
+        float as[13];
+        float2 rsv = make_float2(0.f, 0.f);
+        if (act1) {
 #pragma unroll
             for (int t = 0; t < 13; t++) {
-                const long long d = (t % 3 - 1) + (long long)ld * ((t / 3) % 3 - 1) + sz * (t / 9 - 1);
-                a0[t] = __ldg(A + t * pl + o);
-                am[t] = __ldg(A + t * pl + o - d);
+                const int dx = t % 3 - 1;
+                a0[t] = __ldg(reinterpret_cast<const float2*>(A + t * pl + o));
+                const float* b = A + t * pl + o - sy * ((t / 3) % 3 - 1) - sz * (t / 9 - 1);
+                am[t] = __ldg(reinterpret_cast<const float2*>(b));
+                as[t] = dx < 0 ? __ldg(b + 2) : dx > 0 && i > 0 ? __ldg(b - 1) : 0.f;
             }
-            rsv = __ldg(rs + o);
+            rsv = __ldg(reinterpret_cast<const float2*>(rs + o));
         }
         __syncthreads();
-        if (act) {
+        if (act1) {
             const float* pm = sP[(k + 3) & 3];   // p at k-1
             const float* p0 = sP[k & 3];         // p at k
             const float* pp = sP[(k + 1) & 3];   // p at k+1
-            const float pv = p0[hc];
-            float s = rsv * pv;
+            const float2 pv = *reinterpret_cast<const float2*>(p0 + hc);
+            float s0 = rsv.x * pv.x, s1 = rsv.y * pv.y;
 #pragma unroll
             for (int t = 0; t < 13; t++) {
                 const int dx = t % 3 - 1, dy = (t / 3) % 3 - 1, dz = t / 9 - 1;
                 const int dh = dx + dy * kP3W;
                 const float* pn = dz < 0 ? pm : p0;
                 const float* pr = dz < 0 ? pp : p0;
-                s += a0[t] * (pn[hc + dh] - pv);
-                s += am[t] * (pr[hc - dh] - pv);
+                // the pair's mirrors sit at columns i - dx and i + 1 - dx
+                const float m0 = dx == 0 ? am[t].x : dx < 0 ? am[t].y : as[t];
+                const float m1 = dx == 0 ? am[t].y : dx < 0 ? as[t] : am[t].x;
+                s0 += a0[t].x * (pn[hc + dh] - pv.x);
+                s0 += m0 * (pr[hc - dh] - pv.x);
+                s1 += a0[t].y * (pn[hc + 1 + dh] - pv.y);
+                s1 += m1 * (pr[hc + 1 - dh] - pv.y);
             }
-            p[o] = pv;
-            q[o] = s;
-            acc.add(pv * s);
+            if (act0) {
+                p[o] = pv.x;
+                q[o] = s0;
+                acc.add(pv.x * s0);
+            }
+            p[o + 1] = pv.y;
+            q[o + 1] = s1;
+            acc.add(pv.y * s1);
         }
     }
     double tot;
     if (grid_sum(acc.value(), partials, &st->counter[2], &tot)) {
-        st->pq = tot;
-        if (!(tot > 0.0)) {
-            set_err(st, BMG_ERR_NOT_SPD);
-            st->alpha = 0.0;
-        } else {
-            st->alpha = st->rz / tot;
-        }
+        set_alpha32(st, tot, parity);
     }
 }
 
-// Rows per tile of k_pspmv2d_tiled: minimise waves x (rows + 2 halo rows)
-// at the kernel's occupancy, with at most kMaxBlocks tiles.
+// Rows per band of k_pspmv2d_strips (planes per band in 3-D): minimise waves x
+// (rows + 2 halo rows) at the kernel's occupancy, with at most kMaxBlocks tiles.
 bmg_status pspmv_prepare(Ctx& c) {
     if (!c.rs32) return BMG_OK;
     if (c.dim == 3) {
@@ -854,7 +1002,7 @@ bmg_status pspmv_prepare(Ctx& c) {
         BMG_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_pspmv3d_direct, kThreads, 0));
         if (occ < 1) return BMG_ERR_DEVICE;
         const int m = c.lev[0].n - 2;
-        const int ti = cdiv(m, kP3I), tj = cdiv(m, kP3J);
+        const int ti = cdiv(m + 1, kP3I), tj = cdiv(m, kP3J);   // columns 0 .. n-2
         const long long slots = (long long)sms * occ;
         long long best = -1;
         for (int h = 1; h <= m; h++) {
@@ -872,21 +1020,21 @@ bmg_status pspmv_prepare(Ctx& c) {
     }
     int sms = 0, occ = 0;
     BMG_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, c.device));
-    BMG_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_pspmv2d_tiled, kThreads, 0));
+    BMG_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_pspmv2d_strips, kThreads, 0));
     if (occ < 1) return BMG_ERR_DEVICE;
     const int m = c.lev[0].n - 2;
-    const int tx = cdiv(m, kThreads);
+    const int strips = cdiv(m + 1, 64);    // columns 0 .. n-2
     const long long slots = (long long)sms * occ;
     long long best = -1;
     for (int h = 1; h <= m; h++) {
-        const long long tiles = (long long)tx * cdiv(m, h);
-        if (tiles > kMaxBlocks) continue;
-        const long long cost = cdiv(tiles, slots) * (h + 2LL);
+        const long long ctas = cdiv((long long)strips * cdiv(m, h), kThreads / 32);
+        if (ctas > kMaxBlocks) continue;
+        const long long cost = cdiv(ctas, slots) * (h + 2LL);
         if (best < 0 || cost < best) {
             best = cost;
             c.spmv_h = h;
-            c.spmv_tiles_x = tx;
-            c.spmv_tiles = (int)tiles;
+            c.spmv_tiles_x = strips;
+            c.spmv_tiles = (int)ctas;
         }
     }
     return best < 0 ? BMG_ERR_SHAPE : BMG_OK;
@@ -896,19 +1044,19 @@ bmg_status k_pspmv32(Ctx& c, const float* z, int parity) {
     const Level& L = c.lev[0];
     prof_begin(c, BMG_PROF_SPMV, 0);
     if (c.dim == 2 && c.spmv_h > 0) {
-        k_pspmv2d_tiled<<<c.spmv_tiles, kThreads, 0, c.stream>>>(L.n, L.ld, L.plane, c.spmv_h, c.spmv_tiles_x,
-                                                                 L.A32, c.rs32, z, c.p32s[parity ^ 1],
-                                                                 c.p32s[parity], c.q32, c.partials, c.st);
+        BMG_CUDA(launch_pdl(k_pspmv2d_strips, dim3(c.spmv_tiles), dim3(kThreads), 0, c.stream, L.n, L.ld, L.plane,
+                            c.spmv_h, c.spmv_tiles_x, cdiv(L.n - 2, c.spmv_h), L.A32, c.rs32, z, c.p32s[parity ^ 1],
+                            c.p32s[parity], c.q32, c.partials, c.st, parity));
         c.launches++;
     } else if (c.dim == 3 && c.spmv_h > 0) {
         const int tj = cdiv(L.n - 2, kP3J);
-        k_pspmv3d_direct<<<c.spmv_tiles, kThreads, 0, c.stream>>>(L.n, L.ld, L.plane, c.spmv_h, c.spmv_tiles_x, tj,
-                                                                 L.A32, c.rs32, z, c.p32s[parity ^ 1],
-                                                                 c.p32s[parity], c.q32, c.partials, c.st);
+        BMG_CUDA(launch_pdl(k_pspmv3d_direct, dim3(c.spmv_tiles), dim3(kThreads), 0, c.stream, L.n, L.ld, L.plane,
+                            c.spmv_h, c.spmv_tiles_x, tj, L.A32, c.rs32, z, c.p32s[parity ^ 1], c.p32s[parity], c.q32,
+                            c.partials, c.st, parity));
         c.launches++;
     } else {
         DISPATCH_DIM(c, k_pspmv32_t, L.A32, c.rs32, L.plane, z, c.p32s[parity ^ 1], c.p32s[parity], c.q32,
-                     c.partials, c.st);
+                     c.partials, c.st, parity);
     }
     prof_end(c, BMG_PROF_SPMV, 0, (c.ns + 4) * 4.0 * dofs0(c));
     BMG_CUDA(cudaGetLastError());
@@ -917,13 +1065,23 @@ bmg_status k_pspmv32(Ctx& c, const float* z, int parity) {
 
 bmg_status k_update_dr32(Ctx& c, int parity) {
     const Level& L = c.lev[0];
+    const int want = cdiv(L.plane / 4, kThreads), blocks = want < 8 * c.sms ? want : 8 * c.sms;
     prof_begin(c, BMG_PROF_UPDATE, 0);
-    const int blocks = cdiv(L.plane / 4, kThreads);
-    k_update_xr32<<<blocks < 8 * c.sms ? blocks : 8 * c.sms, kThreads, 0, c.stream>>>(
-        L.plane / 4, (double2*)c.x, (float4*)c.r32, (const float4*)c.p32s[parity], (const float4*)c.q32, c.st);
-    prof_end(c, BMG_PROF_UPDATE, 0, (4 * 4.0 + 2 * 8.0) * dofs0(c));
+    auto kern = parity ? k_update_xr32<1> : k_update_xr32<0>;
+    BMG_CUDA(launch_pdl(kern, dim3(blocks), dim3(kThreads), 0, c.stream, L.plane / 4, (double2*)c.x, (float4*)c.r32,
+                        (const float4*)c.p32s[0], (const float4*)c.p32s[1], (const float4*)c.q32, c.st));
+    // r, q in and r out; the odd iteration also both steps and x
+    prof_end(c, BMG_PROF_UPDATE, 0, (parity ? 3 * 4.0 + 2 * 4.0 + 2 * 8.0 : 3 * 4.0) * dofs0(c));
     c.launches++;
-    BMG_CUDA(cudaGetLastError());
+    return BMG_OK;
+}
+
+bmg_status k_flush_dr32(Ctx& c) {
+    const Level& L = c.lev[0];
+    const int want = cdiv(L.plane / 4, kThreads), blocks = want < 8 * c.sms ? want : 8 * c.sms;
+    BMG_CUDA(launch_pdl(k_flush_x32, dim3(blocks), dim3(kThreads), 0, c.stream, L.plane / 4, (double2*)c.x,
+                        (const float4*)c.p32s[0], c.st));
+    c.launches++;
     return BMG_OK;
 }
 
