@@ -232,6 +232,38 @@ bmg_status run_iteration(Ctx& c, int parity) {
     return BMG_OK;
 }
 
+// Length of an inner run that aims at the reduction want: as many iterations
+// as the contraction per iteration seen so far (rho) needs.  The first run has
+// seen none, so it is read after four iterations and then goes on by
+// refine_next.
+int refine_start(double want, double rho, int refinements, int left) {
+    int m = (int)ceil(log(want) / log(rho)) + 1;
+    if (m < 2) m = 2;
+    if (refinements == 0) m = std::min(m, 4);
+    return std::min(m, std::min(kMaxInner, left));
+}
+
+// Iterations the first run goes on for after `done` (at most `left`), from its
+// own r.z (the run's first value is kept in rzn); 0 once the reduction is
+// reached.  Far from it only half the predicted way is taken, since the
+// contraction of the first iterations is no guide to the later ones.
+int refine_next(const KState& h, double want, double rho, int done, int left) {
+    if (h.err || left < 1) return 0;
+    const double at = sqrt(h.rz / h.rzn);   // at the start of the last iteration
+    const double g = done > 1 ? pow(at, 1.0 / (done - 1)) : rho;
+    if (!(at * g > 2.0 * want)) return 0;
+    const double more = g < 1.0 ? ceil(log(want / (at * g)) / log(g)) : 8.0;
+    const int m = more > 16.0 ? (int)std::min(more / 2, 64.0) : std::max(1, (int)more);
+    return std::min(m, left);
+}
+
+// Contraction per iteration after a run of m that reduced the residual by red.
+double refine_rho(double rho, double red, int m) {
+    if (!(red > 0 && red < 1)) return rho;
+    const double r1 = pow(red, 1.0 / m);
+    return r1 < 0.999 ? std::max(r1, 0.02) : rho;
+}
+
 bmg_status stage_in_async(Ctx& c, const double* src, double* dst);
 bmg_status stage_out_async(Ctx& c, const double* src, double* dst);
 void fill_complexity_info(const Ctx& c, bmg_info* info);
@@ -246,12 +278,7 @@ namespace {
 // on A d = r for m iterations whose updates go straight into the FP64 iterate
 // x; m is chosen from the contraction seen
 // so far so that one inner solve aims at the remaining reduction (bounded
-// below by what FP32 can deliver).  The first run, whose prediction has no
-// contraction to go by, goes on in steps of max(8, m/4) instead of
-// restarting while its r.z is still more than 100 times above its goal
-// (want^2 times its first r.z): on the 257^3 shell the solve took 520 inner
-// iterations instead of 604 (532 when every run could go on).  maxit caps
-// the total inner iterations.
+// below by what FP32 can deliver).  maxit caps the total inner iterations.
 bmg_status pcg_ir(Ctx& c, double tol, int maxit, bmg_info* info) {
     KState h;
     BMG_TRY(reset_state(c));
@@ -264,35 +291,23 @@ bmg_status pcg_ir(Ctx& c, double tol, int maxit, bmg_info* info) {
     int it = 0, refinements = 0;
     bmg_status status = BMG_OK;
     double rho = 0.3;                 // contraction per inner iteration, updated as we go
-    const double floor_red = 1e-6;    // reduction one FP32 inner solve can deliver
     if (bb == 0.0) {
         BMG_CUDA(cudaMemsetAsync(c.x, 0, sizeof(double) * c.lev[0].plane, c.stream));
         rr = 0.0;
     } else {
         const double lim = tol > 0 ? tol * tol * bb : -1.0;
         while (!(rr <= lim) && it < maxit) {
-            double want = tol > 0 ? sqrt(lim / rr) : floor_red;
-            if (want < floor_red) want = floor_red;
-            int m = (int)ceil(log(want) / log(rho)) + 1;
-            if (m < 2) m = 2;
-            if (m > kMaxInner) m = kMaxInner;
-            if (m > maxit - it) m = maxit - it;
-            // the predicted run.  The first run has no contraction to go by:
-            // while its r.z stays far above the run's goal (more than 100x
-            // want^2 times its first value, kept on the device in rzn) it
-            // goes on instead of restarting
-            BMG_TRY(run_iteration(c, it & 1));
-            it++;
-            BMG_CUDA(cudaMemcpyAsync(&c.st->rzn, &c.st->rz, sizeof(double), cudaMemcpyDeviceToDevice, c.stream));
-            int done = 1, mm = m - 1;
+            double want = tol > 0 ? sqrt(lim / rr) : kRefineFloor;
+            if (want < kRefineFloor) want = kRefineFloor;
+            int m, done = 0, mm = refine_start(want, rho, refinements, maxit - it);
             for (;;) {
                 for (int k = 0; k < mm; k++) BMG_TRY(run_iteration(c, (it + k) & 1));
                 it += mm;
                 done += mm;
                 if (done >= kMaxInner || it >= maxit || refinements > 0) break;
                 BMG_TRY(read_state(c, h));
-                if (h.err || !(h.rz > 100.0 * want * want * h.rzn)) break;
-                mm = std::min(std::max(8, m / 4), std::min(kMaxInner - done, maxit - it));
+                mm = refine_next(h, want, rho, done, std::min(kMaxInner - done, maxit - it));
+                if (mm == 0) break;
             }
             m = done;
             if ((it & 1) == 1) BMG_TRY(k_flush_dr32(c));   // the last iteration was even
@@ -303,11 +318,7 @@ bmg_status pcg_ir(Ctx& c, double tol, int maxit, bmg_info* info) {
                 status = (bmg_status)h.err;
                 break;
             }
-            const double red = sqrt(h.rr / rr);
-            if (red > 0 && red < 1) {
-                const double r1 = pow(red, 1.0 / m);
-                if (r1 > 0.02 && r1 < 0.999) rho = r1;
-            }
+            rho = refine_rho(rho, sqrt(h.rr / rr), m);
             rr = h.rr;
         }
         if (status == BMG_OK && tol > 0 && !(rr <= lim)) status = BMG_ERR_NOT_CONVERGED;

@@ -8,6 +8,7 @@
 #include <math.h>
 #include <string.h>
 
+#include <algorithm>
 #include <vector>
 
 #include "common.cuh"
@@ -29,9 +30,10 @@ struct Job {
     double* const* x = nullptr;
     bmg_info* info = nullptr;
     cudaEvent_t ev = nullptr;
-    int phase = 0;           // 0: idle, 1: waiting for the initial residual, 2: waiting for a refinement
-    int it = 0, refinements = 0, m = 0;
-    double bb = 0, rr = 0, rr0 = 0, rho = 0.3;
+    // 0: idle, 1: waiting for the initial residual, 2: for a refinement's, 3: for the first run's r.z
+    int phase = 0;
+    int it = 0, refinements = 0, m = 0;      // m: iterations of the current run so far
+    double bb = 0, rr = 0, rr0 = 0, rho = 0.3, want = 0;
     bool done = false;
     bmg_status status = BMG_OK;
 };
@@ -79,6 +81,24 @@ bmg_status finish_rhs(Job& j, double tol) {
     return BMG_OK;
 }
 
+// mm more iterations of the current run, then the read that follows them: the
+// run's r.z while the first run may go on (the single-problem rule), else the
+// FP64 residual.
+bmg_status go_on(Job& j, int mm, int maxit) {
+    Ctx& c = *j.c;
+    for (int k = 0; k < mm; k++) BMG_TRY(run_iteration(c, (j.it + k) & 1));
+    j.it += mm;
+    j.m += mm;
+    if (mm > 0 && j.refinements == 0 && j.m < kMaxInner && j.it < maxit) {
+        j.phase = 3;
+        return post_state_copy(j);
+    }
+    if (j.it & 1) BMG_TRY(k_flush_dr32(c));   // the last iteration was even
+    BMG_TRY(k_residual_to32(c));
+    j.phase = 2;
+    return post_state_copy(j);
+}
+
 // Called when the job's event has completed: decide and enqueue the next step.
 bmg_status advance(Job& j, double tol, int maxit) {
     Ctx& c = *j.c;
@@ -87,6 +107,8 @@ bmg_status advance(Job& j, double tol, int maxit) {
         j.status = (bmg_status)h.err;
         return finish_rhs(j, tol);
     }
+    if (j.phase == 3)
+        return go_on(j, refine_next(h, j.want, j.rho, j.m, std::min(kMaxInner - j.m, maxit - j.it)), maxit);
     if (j.phase == 1) {
         j.bb = h.bb;
         j.rr = j.rr0 = h.rr;
@@ -96,11 +118,7 @@ bmg_status advance(Job& j, double tol, int maxit) {
             return finish_rhs(j, tol);
         }
     } else {
-        const double red = sqrt(h.rr / j.rr);
-        if (red > 0 && red < 1) {
-            const double r1 = pow(red, 1.0 / j.m);
-            if (r1 > 0.02 && r1 < 0.999) j.rho = r1;
-        }
+        j.rho = refine_rho(j.rho, sqrt(h.rr / j.rr), j.m);
         j.rr = h.rr;
         j.refinements++;
     }
@@ -110,20 +128,9 @@ bmg_status advance(Job& j, double tol, int maxit) {
         j.status = BMG_ERR_NOT_CONVERGED;
         return finish_rhs(j, tol);
     }
-    double want = sqrt(lim / j.rr);
-    if (want < 1e-6) want = 1e-6;
-    int m = (int)ceil(log(want) / log(j.rho)) + 1;
-    if (m < 2) m = 2;
-    if (m > kMaxInner) m = kMaxInner;
-    if (m > maxit - j.it) m = maxit - j.it;
-    for (int k = 0; k < m; k++) BMG_TRY(run_iteration(c, (j.it + k) & 1));
-    j.it += m;
-    j.m = m;
-    if (j.it & 1) BMG_TRY(k_flush_dr32(c));   // the last iteration was even
-    BMG_TRY(k_residual_to32(c));
-    BMG_TRY(post_state_copy(j));
-    j.phase = 2;
-    return BMG_OK;
+    j.want = std::max(sqrt(lim / j.rr), kRefineFloor);
+    j.m = 0;
+    return go_on(j, refine_start(j.want, j.rho, j.refinements, maxit - j.it), maxit);
 }
 
 }  // namespace

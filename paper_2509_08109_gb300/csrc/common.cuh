@@ -466,6 +466,11 @@ bmg_status k_row_sums32(Ctx& c);                // rs32 = row sums of A (compute
 bmg_status k_residual_to32(Ctx& c);             // r32 = (float)(b - A x); rr; resets the inner CG state
 bmg_status k_rz_beta32(Ctx& c, const float* z, const float* zo);
 bmg_status k_update_dr32(Ctx& c, int parity);    // r32 -= alpha q; odd parity: x (FP64) += both iterations' alpha p
+// run lengths of the refinement mode (api.cu)
+constexpr double kRefineFloor = 1e-6;   // reduction one FP32 inner solve can deliver
+int refine_start(double want, double rho, int refinements, int left);
+int refine_next(const KState& h, double want, double rho, int done, int left);
+double refine_rho(double rho, double red, int m);
 bmg_status k_flush_dr32(Ctx& c);                 // x += the step an even last iteration left
 bmg_status node_tiles_prepare(Ctx& c);           // tile shape of the FP64 products and residuals
 bmg_status pspmv_prepare(Ctx& c);                // tile shape of the 2-D operator product
