@@ -20,8 +20,10 @@
 // is one thread's chain of shared-memory reads and products (about 550 cycles
 // at every level with a thread per point), so two lanes share a point: lane 0
 // takes the couplings stored at the point (W, S, SW, NW), lane 1 their mirrors
-// (E, N, NE, SE), and a shuffle adds the two sums.  Per V-cycle, FP32: 17.7 -> 16.9 us, FP64:
-// 32.9 -> 32.1 us.  Each launch then
+// (E, N, NE, SE), and a shuffle adds the two sums; with one right-hand side a phase is one round
+// and the warps beyond a small level's points go straight to the barrier.  Per
+// V-cycle, FP32: 17.7 -> 15.4 us, FP64: 32.9 -> 27 us, 16 problems of four
+// right-hand sides: 25.6 -> 19.5 us.  Each launch then
 // stages it with a few bulk asynchronous copies completed on one mbarrier
 // (bounded wait), while the threads clear the vectors and load the
 // right-hand side.
@@ -137,11 +139,28 @@ __global__ void __launch_bounds__(kTailThreads) k_vtail2d(TailArgs a0, const Tai
     }
     __syncthreads();
     {
+        // a warp a row, every load before the first store (the last column is
+        // boundary, so a row of 33 nodes takes one load per right-hand side)
+        constexpr int kW = kTailThreads / 32, kPass = (kTailMaxN + kW - 1) / kW;
+        static_assert(kTailMaxN == 33, "columns 0 .. 31 and the boundary");
         const int m = s_n[0];
         T* b = base + s_oB[0];
         const T* bg = (const T*)a.b0;
-        for (int j = tid >> 5; j < m; j += nth >> 5)
-            for (int c = tid & 31; c < m * NR; c += 32) b[j * m * NR + c] = bg[(long long)j * a.ld0 * NR + c];
+        T v[kPass][NR];
+#pragma unroll
+        for (int u = 0; u < kPass; u++)
+#pragma unroll
+            for (int q = 0; q < NR; q++) {
+                const int j = (tid >> 5) + u * kW, c = (tid & 31) + 32 * q;
+                v[u][q] = j < m && c < (m - 1) * NR ? bg[(long long)j * a.ld0 * NR + c] : (T)0;
+            }
+#pragma unroll
+        for (int u = 0; u < kPass; u++)
+#pragma unroll
+            for (int q = 0; q < NR; q++) {
+                const int j = (tid >> 5) + u * kW, c = (tid & 31) + 32 * q;
+                if (j < m && c < (m - 1) * NR) b[j * m * NR + c] = v[u][q];
+            }
     }
     const bool staged = mbar::wait(&bar, 0);
     if (!staged) {
@@ -170,6 +189,18 @@ __global__ void __launch_bounds__(kTailThreads) k_vtail2d(TailArgs a0, const Tai
         return s;
     };
     auto join = [](T s) { return s + __shfl_xor_sync(0xffffffffu, s, 1); };
+    // the update (f - s) / a_c; FP64 as f d - s d, one step less in the chain
+    auto update = [](T fv, T dg, T s) { return sizeof(T) == 8 ? fv * dg - s * dg : (fv - s) * dg; };
+    // body(kk) for the pairs of lanes over cnt items; one right-hand side: at
+    // most 16^2 items, one round, and warps beyond them go on
+    auto each = [&](int cnt, auto body) {
+        if constexpr (NR == 1) {
+            static_assert(kTailThreads >= 2 * ((kTailMaxN - 1) / 2) * ((kTailMaxN - 1) / 2));
+            if ((tid & ~31) >> 1 < cnt) body(tid >> 1);
+        } else {
+            for (int k0 = 0; k0 < cnt; k0 += nth >> 1) body(k0 + (tid >> 1));
+        }
+    };
     // every interior node of colour c of level l
     // (m = 2^k + 1, so nb = (m-1)/2 is a power of two and positions are shifts
     // and masks)
@@ -180,14 +211,14 @@ __global__ void __launch_bounds__(kTailThreads) k_vtail2d(TailArgs a0, const Tai
         // index of that parity i0, j0, and nb or nb - 1 such nodes a side
         const int i0 = 1 + ((c & 1) ^ 1), j0 = 1 + (((c >> 1) & 1) ^ 1);
         const int nb = (m - 1) >> 1, lg = log2nb(nb);
-        for (int k0 = 0; k0 < nb * nb * NR; k0 += nth >> 1) {
-            const int kk = k0 + (tid >> 1), k = kk / NR, rh = kk - k * NR;
+        each(nb * nb * NR, [&](int kk) {
+            const int k = kk / NR, rh = kk - k * NR;
             const int i = i0 + 2 * (k & (nb - 1)), j = j0 + 2 * (k >> lg);
             const bool on = k < nb * nb && i <= m - 2 && j <= m - 2;
             const int o = j * m + i;
             const T sum = join(on ? half(A, m, m2, x, o, rh) : (T)0);
-            if (on && h == 0) x[o * NR + rh] = (f[o * NR + rh] - sum) * A[C2 * m2 + o];
-        }
+            if (on && h == 0) x[o * NR + rh] = update(f[o * NR + rh], A[C2 * m2 + o], sum);
+        });
     };
 
     // Fine points are grouped in 2x2 blocks {2I, 2I+1} x {2J, 2J+1} around
@@ -216,7 +247,7 @@ __global__ void __launch_bounds__(kTailThreads) k_vtail2d(TailArgs a0, const Tai
             T sum = A[W2 * m2 + o] * xl;
             sum += A[W2 * m2 + o + 1] * xr;
             if (I >= 1) x[(o - 1) * NR + rh] = xl;
-            x[o * NR + rh] = (f[o * NR + rh] - sum) * A[C2 * m2 + o];
+            x[o * NR + rh] = update(f[o * NR + rh], A[C2 * m2 + o], sum);
         }
         __syncthreads();
         // colours 2 and 3, one thread per colour-3 point: the colour-2 row
@@ -230,10 +261,10 @@ __global__ void __launch_bounds__(kTailThreads) k_vtail2d(TailArgs a0, const Tai
             sum += A[SW2 * m2 + o + m + 1] * X(o + m + 1);
             sum += A[NW2 * m2 + o] * X(o + m - 1);
             sum += A[NW2 * m2 + o - m + 1] * X(o - m + 1);
-            return (f[o * NR + rh] - sum) * A[C2 * m2 + o];
+            return update(f[o * NR + rh], A[C2 * m2 + o], sum);
         };
-        for (int k0 = 0; k0 < nb * nb * NR; k0 += nth >> 1) {
-            const int kk = k0 + (tid >> 1), k = kk / NR, rh = kk - k * NR;
+        each(nb * nb * NR, [&](int kk) {
+            const int k = kk / NR, rh = kk - k * NR;
             const int J = k >> lg, I = k & (nb - 1);
             const int o = (2 * J + 1) * m + 2 * I + 1;
             const bool on = k < nb * nb;
@@ -252,9 +283,9 @@ __global__ void __launch_bounds__(kTailThreads) k_vtail2d(TailArgs a0, const Tai
             sum = join(sum);
             if (on && h == 0) {
                 if (I >= 1) x[(o - 1) * NR + rh] = xn;
-                x[o * NR + rh] = (f[o * NR + rh] - sum) * A[C2 * m2 + o];
+                x[o * NR + rh] = update(f[o * NR + rh], A[C2 * m2 + o], sum);
             }
-        }
+        });
         __syncthreads();
         // residual and restriction, two lanes per interior coarse node, each with
         // half of the centre's couplings and the neighbours on one side.
@@ -278,8 +309,8 @@ __global__ void __launch_bounds__(kTailThreads) k_vtail2d(TailArgs a0, const Tai
         auto r2 = [&](int o, int rh) {   // colour 2 (even i, odd j)
             return -(A[W2 * m2 + o] * x[(o - 1) * NR + rh] + A[W2 * m2 + o + 1] * x[(o + 1) * NR + rh]);
         };
-        for (int k0 = 0; k0 < nb * nb * NR; k0 += nth >> 1) {   // mc - 2 = nb - 1 interior coarse nodes a side
-            const int kk = k0 + (tid >> 1), k = kk / NR, rh = kk - k * NR;
+        each(nb * nb * NR, [&](int kk) {   // mc - 2 = nb - 1 interior coarse nodes a side
+            const int k = kk / NR, rh = kk - k * NR;
             const int J = k >> lg, I = k & (nb - 1);
             const int O = J * mc + I, o = 2 * J * m + 2 * I;
             const bool on = k < nb * nb && I > 0 && J > 0;
@@ -291,7 +322,7 @@ __global__ void __launch_bounds__(kTailThreads) k_vtail2d(TailArgs a0, const Tai
             }
             b = join(b);
             if (on && h == 0) bc[O * NR + rh] = b;
-        }
+        });
         __syncthreads();
     }
     // ---- coarsest: one unknown, in FP64
@@ -325,8 +356,8 @@ __global__ void __launch_bounds__(kTailThreads) k_vtail2d(TailArgs a0, const Tai
         // correction and colour 3, two lanes per colour-3 point: four of its
         // eight corrected neighbours each in registers; lane 0 stores the
         // corrected points of its block and the new value
-        for (int k0 = 0; k0 < nb * nb * NR; k0 += nth >> 1) {
-            const int kk = k0 + (tid >> 1), k = kk / NR, rh = kk - k * NR;
+        each(nb * nb * NR, [&](int kk) {
+            const int k = kk / NR, rh = kk - k * NR;
             const int J = k >> lg, I = k & (nb - 1);
             const int sg = h ? -1 : 1;
             const int i = 2 * I + 1, j = 2 * J + 1, o = j * m + i;
@@ -347,9 +378,9 @@ __global__ void __launch_bounds__(kTailThreads) k_vtail2d(TailArgs a0, const Tai
                 if (I >= 1 && J >= 1) x[(o - m - 1) * NR + rh] = sw;
                 if (J >= 1) x[(o - m) * NR + rh] = so;
                 if (I >= 1) x[(o - 1) * NR + rh] = w;
-                x[o * NR + rh] = (f[o * NR + rh] - sum) * A[C2 * m2 + o];
+                x[o * NR + rh] = update(f[o * NR + rh], A[C2 * m2 + o], sum);
             }
-        }
+        });
         __syncthreads();
         for (int c = 2; c >= 0; c--) {
             colour(A, m, x, f, c);

@@ -305,8 +305,11 @@ inline dim3 g3(int ni, int nj, int nk) { return dim3(cdiv(ni, 64), nj, nk); }
 //     busy: two lanes, the stored couplings and the mirrors);
 //   - eight lanes share a coarse node of the restriction, and prolongation
 //     runs one thread per fine point, all of one parity class in a warp.
-// Measured per V-cycle: FP64 206 -> 54 us (it started at 17^3, in global
-// memory), FP32 42 -> 25.5 us.
+//   - what a thread does in a level's colour phases is formed once per level,
+//     and arrays are offsets from the shared image (pointers kept in a structure
+//     became generic addresses).
+// Measured per V-cycle: FP64 41 us (54 before the last two points; 206 when it
+// started at 17^3, in global memory), FP32 19.7 us (25.5; 42 in its first form).
 constexpr int kTail3Threads = 512;
 constexpr int kTail3MaxN = 9;    // first tail level: n <= this
 constexpr int kTail3Lev = 3;     // levels of a tail: 9, 5, 3 at most
@@ -315,7 +318,7 @@ constexpr unsigned kTail3Chunk = 16384;   // bytes per bulk copy
 template <typename T>
 struct Tail3Args {
     int nlev;
-    int n[kTail3Lev];      // nodes per side
+    int n;                 // nodes per side of the first
     const void* pack;      // packed operators and weights (shared-memory image)
     unsigned pack_bytes;   // its size, a multiple of 16
     const T* b;            // right-hand side of the first tail level
@@ -345,26 +348,40 @@ size_t tail3_vec_elems(const Ctx& c) {
     return e;
 }
 
-// A level in shared memory: n^3 arrays.
-template <typename T>
+// A level in shared memory: n^3 arrays, as element offsets from the image's
+// start (stored pointers would lose their address space).
 struct T3 {
     int n, nc;           // nodes per side, of the next level
-    T *A, *P, *b, *x, *r;
+    int A, P, b, x, r;
 };
 
 // lanes per point of a colour phase
 template <typename T>
 __device__ __forceinline__ int tail3_lanes(int n) { return sizeof(T) == 8 && n > 5 ? 2 : 8; }
 
-// this thread's share of a point's couplings with eight lanes: offsets
-// lane and lane + 8 (none where that is not below 13)
+// What a thread does in every colour phase of a level, formed once per level:
+// its point, lane and share of the point's couplings (eight lanes: offsets lane
+// and lane + 8).  n = 2^k + 1, and a colour's points are walked 2^(k-1) a side,
+// leaving out the even coordinates' last one; all fit in one round (64 points
+// of eight lanes at 9^3).
 struct T3Lane {
+    bool any;             // the warp has points
+    int lane, lanes;
+    int o, last;          // the all-even colour's point; bit d: it lies inside in direction d
     int da, db, pa, pb;   // index distance and plane offset
     int ma, mb;           // parity masks; 0: no offset
 };
+template <typename T>
 __device__ __forceinline__ T3Lane tail3_lane(int n, int tid) {
-    const int a = tid & 7, b = a + 8, n3 = n * n * n;
     T3Lane q;
+    q.lanes = tail3_lanes<T>(n);
+    const int lgl = q.lanes == 8 ? 3 : 1, lg = 31 - __clz(n - 1) - 1, m = 1 << lg, n3 = n * n * n;
+    q.lane = tid & (q.lanes - 1);
+    const int t = tid >> lgl, I = t & (m - 1), J = (t >> lg) & (m - 1), K = t >> (2 * lg);
+    q.any = (tid & ~31) >> lgl < m * m * m;
+    q.o = 2 * (1 + I + n * (1 + J + n * (1 + K)));
+    q.last = K < m ? (I < m - 1) | ((J < m - 1) << 1) | ((K < m - 1) << 2) : -8;
+    const int a = tid & 7, b = a + 8;
     q.da = off_x(a) + n * (off_y(a) + n * off_z(a));
     q.db = off_x(b) + n * (off_y(b) + n * off_z(b));
     q.pa = a * n3;
@@ -380,64 +397,63 @@ __device__ __forceinline__ T3Lane tail3_lane(int n, int tid) {
 // colour is a run-time value, uniform over the CTA: unrolled per colour the
 // code outran the instruction cache (FP32 tail 72 us instead of 42).
 template <typename T>
-__device__ __forceinline__ void tail3_colour(const T3<T>& v, const T3Lane& ln, int col, int sel, int tid) {
+__device__ __forceinline__ void tail3_colour(T* sm, const T3& v, const T3Lane& ln, int col, int sel) {
+    if (!ln.any) return;
     const int n = v.n, n3 = n * n * n;
-    const int pi = col & 1, pj = (col >> 1) & 1, pk = col >> 2;
-    // n = 2^k + 1: walk 2^(k-1) points a side and leave out the even
-    // coordinates' last one, so that positions are shifts and masks
-    const int lg = 31 - __clz(n - 1) - 1, m = 1 << lg;
-    const int lanes = tail3_lanes<T>(n), lgl = lanes == 8 ? 3 : 1;
-    const int h = tid & (lanes - 1);
-    for (int t0 = 0; t0 < m * m * m; t0 += kTail3Threads >> lgl) {
-        const int t = t0 + (tid >> lgl);
-        const int I = t & (m - 1), J = (t >> lg) & (m - 1), K = t >> (2 * lg);
-        const int i = 2 - pi + 2 * I, j = 2 - pj + 2 * J, k = 2 - pk + 2 * K;
-        const bool on = i < n - 1 && j < n - 1 && k < n - 1;
-        const int o = i + n * (j + n * k);
-        T s = 0;
-        if (lanes == 8) {
-            const bool ua = sel == 0 || ((col ^ ln.ma) > col) == (sel > 0);
-            const bool ub = ln.mb && (sel == 0 || ((col ^ ln.mb) > col) == (sel > 0));
-            if (on && ua) {
-                s = v.A[ln.pa + o] * v.x[o + ln.da];
-                s += v.A[ln.pa + o - ln.da] * v.x[o - ln.da];
-            }
-            if (on && ub) {
-                s += v.A[ln.pb + o] * v.x[o + ln.db];
-                s += v.A[ln.pb + o - ln.db] * v.x[o - ln.db];
-            }
-            s += __shfl_xor_sync(0xffffffffu, s, 4);
-            s += __shfl_xor_sync(0xffffffffu, s, 2);
-        } else if (on) {
-            T s1 = 0;   // two chains
+    const T* A = sm + v.A;
+    const T* x = sm + v.x;
+    const int o = ln.o - ((col & 1) + n * (((col >> 1) & 1) + n * (col >> 2)));
+    const bool on = ln.last >= 0 && ((ln.last | col) & 7) == 7;
+    T s = 0, f = 0, dg = 0;
+    if (on && sel <= 0) {
+        f = sm[v.b + o];
+        dg = A[13 * n3 + o];
+    }
+    if (ln.lanes == 8) {
+        const bool ua = sel == 0 || ((col ^ ln.ma) > col) == (sel > 0);
+        const bool ub = ln.mb && (sel == 0 || ((col ^ ln.mb) > col) == (sel > 0));
+        T s1 = 0;
+        if (on && ua) {
+            s = A[ln.pa + o] * x[o + ln.da];
+            s += A[ln.pa + o - ln.da] * x[o - ln.da];
+        }
+        if (on && ub) {
+            s1 = A[ln.pb + o] * x[o + ln.db];
+            s1 += A[ln.pb + o - ln.db] * x[o - ln.db];
+        }
+        s += s1;
+        s += __shfl_xor_sync(0xffffffffu, s, 4);
+        s += __shfl_xor_sync(0xffffffffu, s, 2);
+    } else if (on) {
+        const int h = ln.lane;
+        T s1 = 0;   // two chains
 #pragma unroll
-            for (int q = 0; q < 13; q++) {
-                const int c = col ^ off_mask(q);
-                if (sel == 0 || (c > col) == (sel > 0)) {
-                    const int d = off_x(q) + n * (off_y(q) + n * off_z(q));
-                    const T a = v.A[q * n3 + (h ? o - d : o)], y = v.x[h ? o - d : o + d];
-                    if (q & 1)
-                        s1 += a * y;
-                    else
-                        s += a * y;
-                }
+        for (int q = 0; q < 13; q++) {
+            const int c = col ^ off_mask(q);
+            if (sel == 0 || (c > col) == (sel > 0)) {
+                const int d = off_x(q) + n * (off_y(q) + n * off_z(q));
+                const T a = A[q * n3 + (h ? o - d : o)], y = x[h ? o - d : o + d];
+                if (q & 1)
+                    s1 += a * y;
+                else
+                    s += a * y;
             }
-            s += s1;
         }
-        s += __shfl_xor_sync(0xffffffffu, s, 1);
-        if (on && h == 0) {
-            if (sel > 0)
-                v.r[o] = -s;
-            else
-                v.x[o] = (v.b[o] - s) * v.A[13 * n3 + o];
-        }
+        s += s1;
+    }
+    s += __shfl_xor_sync(0xffffffffu, s, 1);
+    if (on && ln.lane == 0) {
+        if (sel > 0)
+            sm[v.r + o] = -s;
+        else   // FP64: f d - s d, one step less in the chain
+            sm[v.x + o] = sizeof(T) == 8 ? f * dg - s * dg : (f - s) * dg;
     }
 }
 
 template <typename T>
 __global__ void __launch_bounds__(kTail3Threads) k_vtail3d(Tail3Args<T> a) {
     extern __shared__ __align__(16) unsigned char t3_raw[];
-    __shared__ T3<T> lv[kTail3Lev];
+    __shared__ T3 lv[kTail3Lev];
     __shared__ uint64_t bar;
     __shared__ int s_rw[27];   // restriction: weight plane (31: none) and, from bit 8, the owner's offset bits
     const int tid = threadIdx.x, nth = kTail3Threads;
@@ -452,12 +468,12 @@ __global__ void __launch_bounds__(kTail3Threads) k_vtail3d(Tail3Args<T> a) {
             const unsigned len = a.pack_bytes - off < kTail3Chunk ? a.pack_bytes - off : kTail3Chunk;
             mbar::bulk_g2s(t3_raw + off, (const unsigned char*)a.pack + off, len, &bar);
         }
-        T* sp = base;
-        T* vp = base + a.pack_bytes / sizeof(T);
-        for (int q = 0; q < L; q++) {
-            T3<T>& v = lv[q];
-            const int n = v.n = a.n[q], n3 = n * n * n;
-            v.nc = q + 1 < L ? a.n[q + 1] : 0;
+        int sp = 0, vp = (int)(a.pack_bytes / sizeof(T));
+        for (int q = 0, n = a.n; q < L; q++, n = (n + 1) / 2) {
+            T3& v = lv[q];
+            const int n3 = n * n * n;
+            v.n = n;
+            v.nc = q + 1 < L ? (n + 1) / 2 : 0;
             v.A = sp;
             v.P = v.A + NS3 * n3;
             sp = v.P + NP3 * v.nc * v.nc * v.nc;
@@ -478,18 +494,27 @@ __global__ void __launch_bounds__(kTail3Threads) k_vtail3d(Tail3Args<T> a) {
     __syncthreads();
     // meanwhile: zero vectors, then the first level's right-hand side
     {
-        T* v0 = lv[0].b;
-        const int nv = (int)(lv[L - 1].r - v0) + lv[L - 1].n * lv[L - 1].n * lv[L - 1].n;
-        for (int u = tid; u < nv; u += nth) v0[u] = (T)0;
+        const int nv = lv[L - 1].r + lv[L - 1].n * lv[L - 1].n * lv[L - 1].n;
+        for (int u = lv[0].b + tid; u < nv; u += nth) base[u] = (T)0;
     }
     pdl_wait();
     pdl_trigger();
     __syncthreads();
     {
-        const int n = lv[0].n;   // at most 16: half a warp a row
-        T* b = lv[0].b;
-        for (int row = tid >> 4; row < n * n; row += nth >> 4)
-            if ((tid & 15) < n) b[row * n + (tid & 15)] = a.b[(long long)a.ld * row + (tid & 15)];
+        // half a warp a row, every load before the first store
+        constexpr int kPass = (kTail3MaxN * kTail3MaxN + kTail3Threads / 16 - 1) / (kTail3Threads / 16);
+        const int n = lv[0].n, i = tid & 15, rows = i < n ? n * n : 0;
+        T v[kPass];
+#pragma unroll
+        for (int q = 0; q < kPass; q++) {
+            const int row = (tid >> 4) + q * (kTail3Threads / 16);
+            v[q] = row < rows ? a.b[(long long)a.ld * row + i] : (T)0;
+        }
+#pragma unroll
+        for (int q = 0; q < kPass; q++) {
+            const int row = (tid >> 4) + q * (kTail3Threads / 16);
+            if (row < rows) base[lv[0].b + row * n + i] = v[q];
+        }
     }
     if (!__syncthreads_and(mbar::wait(&bar, 0))) {
         // record the expiry, give the copies in flight one more bounded wait
@@ -499,11 +524,11 @@ __global__ void __launch_bounds__(kTail3Threads) k_vtail3d(Tail3Args<T> a) {
         return;
     }
     for (int l = 0; l + 1 < L; l++) {
-        const T3<T> v = lv[l], w = lv[l + 1];
-        const T3Lane ln = tail3_lane(v.n, tid);
+        const T3 v = lv[l], w = lv[l + 1];
+        const T3Lane ln = tail3_lane<T>(v.n, tid);
 #pragma unroll 1
         for (int ph = 0; ph < 15; ph++) {      // colours 0..7 forward, residuals of colours 0..6
-            tail3_colour<T>(v, ln, ph & 7, ph < 8 ? -1 : 1, tid);
+            tail3_colour<T>(base, v, ln, ph & 7, ph < 8 ? -1 : 1);
             if (ph < 8 || ph == 14) __syncthreads();
         }
         // restriction: the 27 fine neighbours of a coarse node over eight lanes
@@ -517,25 +542,25 @@ __global__ void __launch_bounds__(kTail3Threads) k_vtail3d(Tail3Args<T> a) {
             if (on)
                 for (int o = tid & 7; o < 27; o += 8) {
                     const int pw = s_rw[o], sb = pw >> 8;
-                    const T rv = v.r[of + off_x(o) + n * (off_y(o) + n * off_z(o))];
+                    const T rv = base[v.r + of + off_x(o) + n * (off_y(o) + n * off_z(o))];
                     const int own = oc - (sb & 1) - nc * (((sb >> 1) & 1) + nc * (sb >> 2));
-                    s += (pw & 31) == 31 ? rv : v.P[(pw & 31) * nc3 + own] * rv;
+                    s += (pw & 31) == 31 ? rv : base[v.P + (pw & 31) * nc3 + own] * rv;
                 }
             s += __shfl_xor_sync(0xffffffffu, s, 4);
             s += __shfl_xor_sync(0xffffffffu, s, 2);
             s += __shfl_xor_sync(0xffffffffu, s, 1);
-            if (on && (tid & 7) == 0) w.b[oc] = s;
+            if (on && (tid & 7) == 0) base[w.b + oc] = s;
         }
         __syncthreads();
     }
     if (tid == 0) {   // coarsest: one unknown, in FP64
-        const T3<T> v = lv[L - 1];
+        const T3 v = lv[L - 1];
         const int o = 1 + v.n * (1 + v.n);
-        v.x[o] = (T)((double)v.b[o] * ainv);
+        base[v.x + o] = (T)((double)base[v.b + o] * ainv);
     }
     __syncthreads();
     for (int l = L - 2; l >= 0; l--) {
-        const T3<T> v = lv[l], w = lv[l + 1];
+        const T3 v = lv[l], w = lv[l + 1];
         const int n = v.n, nc = w.n, lg = 31 - __clz(nc - 1), mc = 1 << lg, nc3 = nc * nc * nc;
         // cell (I, J, K) of the coarse level owns the fine points 2 (I, J, K) + b
         for (int t = tid; t < 8 * mc * mc * mc; t += nth) {
@@ -545,30 +570,30 @@ __global__ void __launch_bounds__(kTail3Threads) k_vtail3d(Tail3Args<T> a) {
             const int oc = I + nc * (J + nc * K);
             T s = 0;
             if (b == 0) {
-                s = w.x[oc];
+                s = base[w.x + oc];
             } else {
-                const T* P = v.P + kPBase(b) * nc3 + oc;
+                const T* P = base + v.P + kPBase(b) * nc3 + oc;
 #pragma unroll
                 for (int c = 0; c < 8; c++)
                     if ((c & ~b) == 0) {
-                        s += *P * w.x[oc + (c & 1) + nc * (((c >> 1) & 1) + nc * (c >> 2))];
+                        s += *P * base[w.x + oc + (c & 1) + nc * (((c >> 1) & 1) + nc * (c >> 2))];
                         P += nc3;
                     }
             }
-            v.x[i + n * (j + n * k)] += s;
+            base[v.x + i + n * (j + n * k)] += s;
         }
         __syncthreads();
-        const T3Lane ln = tail3_lane(n, tid);
+        const T3Lane ln = tail3_lane<T>(n, tid);
 #pragma unroll 1
         for (int col = 7; col >= 0; col--) {
-            tail3_colour<T>(v, ln, col, 0, tid);
+            tail3_colour<T>(base, v, ln, col, 0);
             __syncthreads();
         }
     }
     {   // the first level's iterate to its array
         const int n = lv[0].n;
         for (int row = tid >> 4; row < n * n; row += nth >> 4)
-            if ((tid & 15) < n) a.x[(long long)a.ld * row + (tid & 15)] = lv[0].x[row * n + (tid & 15)];
+            if ((tid & 15) < n) a.x[(long long)a.ld * row + (tid & 15)] = base[lv[0].x + row * n + (tid & 15)];
     }
 }
 
@@ -1027,7 +1052,7 @@ bmg_status vcycle3d_impl(Ctx& c, const T* b0, T* x0, T* xout) {
         Tail3Args<T> a{};
         a.nlev = L - t;
         if (a.nlev > kTail3Lev) return BMG_ERR_STATE;   // n <= 9 has at most kTail3Lev levels
-        for (int q = 0; q < a.nlev; q++) a.n[q] = c.lev[t + q].n;
+        a.n = c.lev[t].n;
         a.pack = c.tail_pack;
         a.pack_bytes = (unsigned)tail3_pack_bytes(c);
         a.b = bl(t);
