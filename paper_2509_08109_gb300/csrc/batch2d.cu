@@ -246,10 +246,11 @@ __global__ void k_bunpack_all(const BProbDev* __restrict__ probs, const PackEnt*
 // A block takes kResRows rows, so a problem has blocks in proportion to its
 // rows (the grid's width is the largest problem's count, the blocks past a
 // problem's own leave at once): FP64 arithmetic, 12 operations a value, bounds
-// the kernel, and with a fixed 32 blocks for every problem the largest ones
-// ran on a fraction of the SMs (16 problems of 65..1025 x 4: mean of a
-// solve's four calls 1.12 ms, now 0.63 ms).
-constexpr int kResRows = 8;
+// the kernel, so a block holds its share of an SM's FP64 units for as long as
+// its rows take, and few long blocks leave the last ones running alone (16
+// problems of 65..1025 x 4, a solve's full calls: 0.76 ms with eight rows a
+// block, 0.64 with four, 0.62 with two, 0.555 with one).
+constexpr int kResRows = 1;
 __host__ __device__ inline int res_blocks(int n) { return (n - 2 + kResRows - 1) / kResRows; }
 
 __global__ void __launch_bounds__(kBThreads) k_bresidual(const BProbDev* __restrict__ probs, SysState* sys,
