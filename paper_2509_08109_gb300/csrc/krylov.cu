@@ -722,10 +722,11 @@ bmg_status k_residual_to32(Ctx& c) {
 // shuffle, and lanes 0 and 31 load the strip's edge columns.  The next row's
 // raw values (z, p_old, planes) are in flight while a row is formed.  HBM
 // bounds the kernel on large grids (36 bytes a node), the chain of row loads
-// on small ones.  4097^2: 120 us, 65^2: 6.8 us, against 129 and 8.1 us for a
-// thread per column, a block barrier per row and the planes in shared memory.
+// on small ones.  4097^2: 103 us, 65^2: 7 us, against 129 and 8.1 us for a
+// thread per column, a block barrier per row and the planes in shared memory;
+// with two CTAs an SM instead of three (92 registers a thread for 80) 120 us.
 // Same arithmetic, in the same order, as k_pspmv32_t<2>.
-__global__ void __launch_bounds__(kThreads) k_pspmv2d_strips(int n, int ld, long long pl, int H, int strips, int bands,
+__global__ void __launch_bounds__(kThreads, 3) k_pspmv2d_strips(int n, int ld, long long pl, int H, int strips, int bands,
                                                              const float* __restrict__ A,
                                                              const float* __restrict__ rs, const float* z,
                                                              const float* pold, float* __restrict__ p,
