@@ -503,10 +503,10 @@ def run_own(args):
 # FP64 floating-point operations per interior node of one launch of each
 # finest-level class of the plain FP64 solve, counted by ncu
 # (smsp__sass_thread_inst_executed_op_{dfma,dmul,dadd}_pred_on, an FMA as two)
-# on the 2049^2 annulus: profiles/vdown64_annulus2049_fp64.md.  The FP64
+# on the 2049^2 annulus: profiles/fp64_vcycle_annulus2049.md.  The FP64
 # kernels of this path are bound by the FP64 rate rather than by HBM; their
 # roofline is the FP64 peak.
-FP64_FLOPS_PER_NODE = {"vdown": 36.81, "vup": 39.28, "spmv": 19.45, "update": 6.52}
+FP64_FLOPS_PER_NODE = {"vdown": 20.97, "vup": 25.75, "spmv": 19.04, "update": 6.16}
 # GB300 FP64 (non-tensor) peak, nominal: 1.25 TFLOP/s
 FP64_PEAK_GFLOPS = 1250.0
 
