@@ -658,7 +658,12 @@ __global__ void k_tail3_pack(const T* __restrict__ A, int n, int ld, long long p
 // a row takes four warps, so either the rows' halo grows (four slots) or the
 // CTA does: 257 us against 196 for the 58-column tiles (169 since their
 // accesses are pairs and the first rows' stencils are fetched while the
-// iterates are staged).  The halo row that no owned row needs is left out: a
+// iterates are staged).  The levels up to 65 take the slots that leave the
+// fewest row slots on the fullest of the 152 SMs (CTAs an SM, rounded up, times
+// S): at 65 five (eight tiles in 32 planes, two CTAs an SM), at 33 and below
+// three.  FP64, a reverse half sweep: 65^3 22.0 -> 16.3 us with five slots for
+// eight, 33^3 13.2 -> 11.1 and 17^3 12.9 -> 10.6 with three; 129^3 CG solve 6.48
+// -> 6.24 ms.  The halo row that no owned row needs is left out: a
 // seventh of the FP64 arithmetic of the four-slot tiles (129^3 FP64, reverse
 // 100 -> 92 us, forward 79 -> 69 us).
 template <int W_, int S_, bool FULL_>
@@ -986,8 +991,10 @@ bmg_status hsweep3d(Ctx& c, int l, const T* f, const T* xcur, const T* xz, T* xo
     const HS3Args<T> a{A_of<T>(F), F.n, F.ld, F.plane, f, xcur, xz, xout, parity};
     prof_begin(c, BMG_PROF_SMOOTH, l);
     bmg_status st;
-    if (F.n <= 65)
-        st = launch_hsweep3d<T, HsShape<1, 8, true>, MODE, FWD>(c, a, planes);
+    if (F.n <= 33)
+        st = launch_hsweep3d<T, HsShape<1, 3, true>, MODE, FWD>(c, a, planes);
+    else if (F.n <= 65)
+        st = launch_hsweep3d<T, HsShape<1, 5, true>, MODE, FWD>(c, a, planes);
     else if (F.n <= 129)
         st = launch_hsweep3d<T, HsShape<2, 4, true>, MODE, FWD>(c, a, planes);
     else
