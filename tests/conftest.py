@@ -1,3 +1,4 @@
+import gc
 import os
 import sys
 
@@ -21,3 +22,12 @@ def pytest_collection_modifyitems(config, items):
     for item in items:
         if "gpu" in item.keywords:
             item.add_marker(skip)
+
+
+def pytest_runtest_setup(item):
+    # The allocation-free entry point's test compares the allocator's state
+    # around a call.  An exception that a test before it caught keeps its
+    # frame's tensors alive in a reference cycle, and the collector may free
+    # them between the two readings: collect them first.
+    if item.path.name == "test_zz_no_alloc.py":
+        gc.collect()
