@@ -233,20 +233,19 @@ bmg_status run_iteration(Ctx& c, int parity) {
 }
 
 // Length of an inner run that aims at the reduction want: as many iterations
-// as the contraction per iteration seen so far (rho) needs.  The first run has
-// seen none, so it is read after four iterations and then goes on by
-// refine_next.
-int refine_start(double want, double rho, int refinements, int left) {
+// as the contraction per iteration seen so far (rho; 0.3 before the first run)
+// needs.
+int refine_start(double want, double rho, int left) {
     int m = (int)ceil(log(want) / log(rho)) + 1;
     if (m < 2) m = 2;
-    if (refinements == 0) m = std::min(m, 4);
     return std::min(m, std::min(kMaxInner, left));
 }
 
-// Iterations the first run goes on for after `done` (at most `left`), from its
-// own r.z (the run's first value is kept in rzn); 0 once the reduction is
-// reached.  Far from it only half the predicted way is taken, since the
-// contraction of the first iterations is no guide to the later ones.
+// Iterations the first run, whose count rests on a guess, goes on for after
+// `done` (at most `left`), from its own r.z (the run's first value is kept in
+// rzn); 0 once the reduction is reached.  Far from it only half the predicted
+// way is taken, since the contraction of the first iterations is no guide to
+// the later ones.
 int refine_next(const KState& h, double want, double rho, int done, int left) {
     if (h.err || left < 1) return 0;
     const double at = sqrt(h.rz / h.rzn);   // at the start of the last iteration
@@ -257,11 +256,12 @@ int refine_next(const KState& h, double want, double rho, int done, int left) {
     return std::min(m, left);
 }
 
-// Contraction per iteration after a run of m that reduced the residual by red.
+// Contraction per iteration after a run of m that reduced the residual by red
+// (one below 0.02 is no rate to go by: the run was short).
 double refine_rho(double rho, double red, int m) {
     if (!(red > 0 && red < 1)) return rho;
     const double r1 = pow(red, 1.0 / m);
-    return r1 < 0.999 ? std::max(r1, 0.02) : rho;
+    return r1 > 0.02 && r1 < 0.999 ? r1 : rho;
 }
 
 bmg_status stage_in_async(Ctx& c, const double* src, double* dst);
@@ -299,7 +299,7 @@ bmg_status pcg_ir(Ctx& c, double tol, int maxit, bmg_info* info) {
         while (!(rr <= lim) && it < maxit) {
             double want = tol > 0 ? sqrt(lim / rr) : kRefineFloor;
             if (want < kRefineFloor) want = kRefineFloor;
-            int m, done = 0, mm = refine_start(want, rho, refinements, maxit - it);
+            int m, done = 0, mm = refine_start(want, rho, maxit - it);
             for (;;) {
                 for (int k = 0; k < mm; k++) BMG_TRY(run_iteration(c, (it + k) & 1));
                 it += mm;

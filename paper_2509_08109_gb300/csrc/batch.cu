@@ -130,7 +130,7 @@ bmg_status advance(Job& j, double tol, int maxit) {
     }
     j.want = std::max(sqrt(lim / j.rr), kRefineFloor);
     j.m = 0;
-    return go_on(j, refine_start(j.want, j.rho, j.refinements, maxit - j.it), maxit);
+    return go_on(j, refine_start(j.want, j.rho, maxit - j.it), maxit);
 }
 
 }  // namespace

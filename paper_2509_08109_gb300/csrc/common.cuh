@@ -468,7 +468,7 @@ bmg_status k_rz_beta32(Ctx& c, const float* z, const float* zo);
 bmg_status k_update_dr32(Ctx& c, int parity);    // r32 -= alpha q; odd parity: x (FP64) += both iterations' alpha p
 // run lengths of the refinement mode (api.cu)
 constexpr double kRefineFloor = 1e-6;   // reduction one FP32 inner solve can deliver
-int refine_start(double want, double rho, int refinements, int left);
+int refine_start(double want, double rho, int left);
 int refine_next(const KState& h, double want, double rho, int done, int left);
 double refine_rho(double rho, double red, int m);
 bmg_status k_flush_dr32(Ctx& c);                 // x += the step an even last iteration left
