@@ -316,6 +316,7 @@ bmg_status pcg_ir(Ctx& c, double tol, int maxit, bmg_info* info) {
             refinements++;
             if (h.err) {
                 status = (bmg_status)h.err;
+                rr = h.rr;   // the residual of the iterate that is returned
                 break;
             }
             rho = refine_rho(rho, sqrt(h.rr / rr), m);

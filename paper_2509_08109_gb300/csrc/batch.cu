@@ -103,11 +103,12 @@ bmg_status go_on(Job& j, int mm, int maxit) {
 bmg_status advance(Job& j, double tol, int maxit) {
     Ctx& c = *j.c;
     const KState& h = *c.st_host;
-    if (h.err) {
+    if (h.err && j.phase != 3) {
         j.status = (bmg_status)h.err;
+        if (j.phase == 2) j.rr = h.rr;   // the residual of the iterate that is returned
         return finish_rhs(j, tol);
     }
-    if (j.phase == 3)
+    if (j.phase == 3)   // after an error too: the pending step and the residual (refine_next gives 0)
         return go_on(j, refine_next(h, j.want, j.rho, j.m, std::min(kMaxInner - j.m, maxit - j.it)), maxit);
     if (j.phase == 1) {
         j.bb = h.bb;

@@ -1343,10 +1343,6 @@ bmg_status batch_solve(Batch& B, int nrhs, const double* const* b, double* const
         if (global_it & 1) BMG_TRY(launch_update(B, 2));   // the last iteration was even
         BMG_TRY(residual(B, false));
         BMG_TRY(read_sys(B));
-        if (B.st_h->err) {
-            first_err = (bmg_status)B.st_h->err;
-            break;
-        }
         for (int s = 0; s < S; s++) {
             if (!act[s]) continue;
             const int m = B.sys_h[s].taken;
@@ -1360,6 +1356,10 @@ bmg_status batch_solve(Batch& B, int nrhs, const double* const* b, double* const
             }
             rr[s] = nr;
             lastm[s] = m;
+        }
+        if (B.st_h->err) {   // counts and residuals are those of the iterates returned
+            first_err = (bmg_status)B.st_h->err;
+            break;
         }
     }
     // solutions back to the caller
