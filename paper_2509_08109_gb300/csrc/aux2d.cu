@@ -237,7 +237,7 @@ __global__ void k_inv(int nr, double* __restrict__ v) {
 // with the fused conversions and the dependent launches below.
 template <typename V, typename X, typename F>
 __device__ __forceinline__ V sell_sum(int b, int e, int step, const int* __restrict__ ci, const V* __restrict__ va,
-                                      const X* __restrict__ x, F&& term, V s = 0) {
+                                      const X* x, F&& term, V s = 0) {
     for (int k = b; k < e; k += 8 * step) {
         int c[8];
         V v[8];
@@ -259,7 +259,7 @@ __device__ __forceinline__ V sell_sum(int b, int e, int step, const int* __restr
 }
 
 __device__ __forceinline__ double csr_row(const int* __restrict__ so, const int* __restrict__ ci,
-                                          const double* __restrict__ va, const double* __restrict__ x, int i) {
+                                          const double* __restrict__ va, const double* x, int i) {
     const int sl = i >> 5;
     return sell_sum(so[sl] + (i & 31), so[sl + 1], 32, ci, va, x, [](double v, double g) { return v * g; });
 }
@@ -340,7 +340,7 @@ __global__ void k_restrict_ct(int nq, const int* __restrict__ rp, const int* __r
 // with u: u[i] += gamma * out[i] instead
 __global__ void k_prolong_c(int nr, const int* __restrict__ rp, const int* __restrict__ ci,
                             const double* __restrict__ va, const double* z, const double* __restrict__ w,
-                            double* __restrict__ out, double* __restrict__ u, double gamma) {
+                            double* out, double* u, double gamma) {
     pdl_wait();
     pdl_trigger();
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
@@ -427,7 +427,7 @@ __global__ void k_spmv_dot(int nr, const int* __restrict__ rp, const int* __rest
 }
 
 // u += alpha p; r -= alpha q; ||r||^2 (alpha from the device state)
-__global__ void k_update_ur(int nr, double* __restrict__ u, double* __restrict__ r, const double* p,
+__global__ void k_update_ur(int nr, double* u, double* r, const double* p,
                             const double* q, const AuxState* stc, double* partials, unsigned int* counter,
                             double* slot) {
     pdl_wait();
@@ -463,7 +463,7 @@ __global__ void k_dot2_aux(int nr, const double* r, const double* z,
     }
 }
 
-__global__ void k_p_update_aux(int nr, double* __restrict__ p, const double* z, const AuxState* st) {
+__global__ void k_p_update_aux(int nr, double* p, const double* z, const AuxState* st) {
     pdl_wait();
     pdl_trigger();
     const double beta = st->beta_o;
@@ -477,7 +477,7 @@ __global__ void k_p_update_aux(int nr, double* __restrict__ p, const double* z, 
 // lose A u to cancellation (the diagonal entry contributes a_ii * 0).
 __device__ __forceinline__ float sell_diff32(const int* __restrict__ so, const int* __restrict__ ci,
                                             const float* __restrict__ va, const float* __restrict__ rs,
-                                            const float* __restrict__ x, int i) {
+                                            const float* x, int i) {
     const int sl = i >> 5;
     const float xi = x[i];
     return sell_sum(so[sl] + (i & 31), so[sl + 1], 32, ci, va, x, [xi](float v, float g) { return v * (g - xi); },
@@ -547,7 +547,7 @@ __global__ void __launch_bounds__(32 * kCtWarps) k_restrict_ct32(int nq, const i
 // u += gamma w (C z), z the coarse correction (FP64, padded layout)
 __global__ void k_prolong_c32(int nr, const int* __restrict__ so, const int* __restrict__ ci,
                               const float* __restrict__ va, const double* z, const float* __restrict__ w,
-                              float* __restrict__ u, float gamma) {
+                              float* u, float gamma) {
     pdl_wait();
     pdl_trigger();
     const int i = blockIdx.x * blockDim.x + threadIdx.x;

@@ -205,7 +205,11 @@ inline void prof_end(Ctx& c, int kind, int level, double bytes) {
 // kernel of the iteration writes (operators, weights) while the last CTAs of
 // the one before still run.  pdl_wait() returns once every earlier kernel has
 // finished and its writes are visible, so it stands before the first access to
-// a vector or scalar.  Without a trigger the next kernel comes up as this one's
+// a vector or scalar.  __restrict__ would let the compiler take the wait for
+// one that does not concern an array and move a load of it above; so in a
+// waiting kernel, and in what it calls, only arrays that no kernel of the
+// iteration writes (operators, weights, index lists) and arrays that this one
+// writes and does not read carry it.  Without a trigger the next kernel comes up as this one's
 // CTAs leave; pdl_trigger(), after the wait, calls it earlier, which pays only
 // where this grid leaves SMs idle: a large one's CTAs lose their places to
 // CTAs that wait (4097^2 solve 14.62 ms without triggers, 14.76 with; 65^2 1.00

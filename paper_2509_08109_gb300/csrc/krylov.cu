@@ -308,8 +308,8 @@ __global__ void __launch_bounds__(kThreads) k_spmv_pq64(NodeTiles<DIM> g, const 
 }
 
 // x += alpha p; r -= alpha q; st.rr = ||r||^2
-__global__ void __launch_bounds__(kThreads) k_update_xr64(long long pairs, double2* __restrict__ x,
-                                                          double2* __restrict__ r, const double2* p,
+__global__ void __launch_bounds__(kThreads) k_update_xr64(long long pairs, double2* x,
+                                                          double2* r, const double2* p,
                                                           const double2* q, double* partials,
                                                           KState* st) {
     pdl_wait();
@@ -370,7 +370,7 @@ __global__ void __launch_bounds__(kThreads) k_rz_beta64(long long pairs, const d
 
 // p = z + beta p
 __global__ void __launch_bounds__(kThreads) k_p_update64(long long pairs, const double2* z,
-                                                         double2* __restrict__ p, KState* st) {
+                                                         double2* p, KState* st) {
     pdl_wait();
     pdl_trigger();
     const double beta = st->beta;
@@ -486,8 +486,8 @@ __device__ __forceinline__ void add_step(double2& x0, double2& x1, double alpha,
 }
 
 template <int PARITY>
-__global__ void __launch_bounds__(kThreads) k_update_xr32(long long quads, double2* __restrict__ x,
-                                                          float4* __restrict__ r, const float4* p0,
+__global__ void __launch_bounds__(kThreads) k_update_xr32(long long quads, double2* x,
+                                                          float4* r, const float4* p0,
                                                           const float4* p1,
                                                           const float4* q, const KState* st) {
     pdl_wait();
@@ -515,7 +515,7 @@ __global__ void __launch_bounds__(kThreads) k_update_xr32(long long quads, doubl
 }
 
 // x += alpha0 p0: the step an even iteration left at the end of a run
-__global__ void __launch_bounds__(kThreads) k_flush_x32(long long quads, double2* __restrict__ x,
+__global__ void __launch_bounds__(kThreads) k_flush_x32(long long quads, double2* x,
                                                         const float4* p0, const KState* st) {
     pdl_wait();
     pdl_trigger();
