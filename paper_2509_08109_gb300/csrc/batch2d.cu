@@ -122,9 +122,11 @@ struct BProbDev {
     float* q;              // FP32 A p
     int sp_tiles_x, sp_tiles;   // tiles of the operator product
     long long sp_part;     // first partial of the operator product
+    long long res_part;    // first partial of the residual (a block an interior row)
 };
 
-// Item of the batched operator product: one tile of one problem.
+// Work item: one tile (operator product) or interior row (residual, from 0) of
+// one problem.
 struct SpItem {
     int prob, tile;
 };
@@ -243,60 +245,57 @@ __global__ void k_bunpack_all(const BProbDev* __restrict__ probs, const PackEnt*
 // ||r||^2 (and, with bb, ||b||^2) per system; the last block of the problem
 // stores them and restarts the inner CG of its active systems.  Rows whose x
 // neighbourhood is zero take r = b without the FP64 products.
-// A block takes kResRows rows, so a problem has blocks in proportion to its
-// rows (the grid's width is the largest problem's count, the blocks past a
-// problem's own leave at once): FP64 arithmetic, 12 operations a value, bounds
-// the kernel, so a block holds its share of an SM's FP64 units for as long as
-// its rows take, and few long blocks leave the last ones running alone (16
-// problems of 65..1025 x 4, a solve's full calls: 0.76 ms with eight rows a
-// block, 0.64 with four, 0.62 with two, 0.555 with one).
-constexpr int kResRows = 1;
-__host__ __device__ inline int res_blocks(int n) { return (n - 2 + kResRows - 1) / kResRows; }
-
-__global__ void __launch_bounds__(kBThreads) k_bresidual(const BProbDev* __restrict__ probs, SysState* sys,
+// A block takes one row from a work-list of every problem's rows: FP64
+// arithmetic, 12 operations a value, bounds the kernel, so a block holds its
+// share of an SM's FP64 units for as long as its rows take, and few long blocks
+// leave the last ones running alone (16 problems of 65..1025 x 4, a solve's full
+// calls: 0.76 ms with eight rows a block, 0.64 with four, 0.62 with two, 0.555
+// with one).  A grid of the largest problem's rows for every problem, with
+// partials to match, costs an uneven batch blocks that only leave: one of 4097^2
+// beside 511 of 65^2 took 46.3 ms a solve and 132 MB more instead of 43.0.
+__global__ void __launch_bounds__(kBThreads) k_bresidual(const BProbDev* __restrict__ probs,
+                                                         const SpItem* __restrict__ items, SysState* sys,
                                                          double* partials, unsigned* counters, int bb) {
     __shared__ double red[kBThreads];
     __shared__ bool last;
-    const int pi = blockIdx.y;
+    const SpItem it = items[blockIdx.x];
+    const int pi = it.prob;
     const BProbDev P = probs[pi];
-    const int n = P.n, ld = P.ld, nb = res_blocks(n);
-    if ((int)blockIdx.x >= nb) return;
+    const int n = P.n, ld = P.ld, nb = n - 2;
     const int rh = threadIdx.x % R, col = threadIdx.x / R;
     const long long pl = P.plane;
     double acc = 0.0, accb = 0.0;
-    const int j1 = min(1 + ((int)blockIdx.x + 1) * kResRows, n - 1);
-    for (int j = 1 + (int)blockIdx.x * kResRows; j < j1; j++) {
-        for (int i = 1 + col; i <= n - 2; i += kBCols) {
-            const long long o = (long long)j * ld + i;
-            const double* A = P.A64;
-            auto X = [&](long long q) { return P.x[q * R + rh]; };
-            auto bits = [](double v) { return (unsigned long long)__double_as_longlong(v) << 1; };
-            const unsigned long long zx = bits(X(o)) | bits(X(o - 1)) | bits(X(o + 1)) | bits(X(o - ld)) |
-                                          bits(X(o + ld)) | bits(X(o - ld - 1)) | bits(X(o + ld + 1)) |
-                                          bits(X(o + ld - 1)) | bits(X(o - ld + 1));
-            const double bv = P.b[o * R + rh];
-            double v = bv;
-            if (zx != 0) {
-                double s = A[C2 * pl + o] * X(o);
-                s += A[W2 * pl + o] * X(o - 1);
-                s += A[W2 * pl + o + 1] * X(o + 1);
-                s += A[S2 * pl + o] * X(o - ld);
-                s += A[S2 * pl + o + ld] * X(o + ld);
-                s += A[SW2 * pl + o] * X(o - ld - 1);
-                s += A[SW2 * pl + o + ld + 1] * X(o + ld + 1);
-                s += A[NW2 * pl + o] * X(o + ld - 1);
-                s += A[NW2 * pl + o - ld + 1] * X(o - ld + 1);
-                v = bv - s;
-            }
-            P.r[o * R + rh] = (float)v;
-            acc += v * v;
-            if (bb) accb += bv * bv;
+    const int j = 1 + it.tile;
+    for (int i = 1 + col; i <= n - 2; i += kBCols) {
+        const long long o = (long long)j * ld + i;
+        const double* A = P.A64;
+        auto X = [&](long long q) { return P.x[q * R + rh]; };
+        auto bits = [](double v) { return (unsigned long long)__double_as_longlong(v) << 1; };
+        const unsigned long long zx = bits(X(o)) | bits(X(o - 1)) | bits(X(o + 1)) | bits(X(o - ld)) |
+                                      bits(X(o + ld)) | bits(X(o - ld - 1)) | bits(X(o + ld + 1)) |
+                                      bits(X(o + ld - 1)) | bits(X(o - ld + 1));
+        const double bv = P.b[o * R + rh];
+        double v = bv;
+        if (zx != 0) {
+            double s = A[C2 * pl + o] * X(o);
+            s += A[W2 * pl + o] * X(o - 1);
+            s += A[W2 * pl + o + 1] * X(o + 1);
+            s += A[S2 * pl + o] * X(o - ld);
+            s += A[S2 * pl + o + ld] * X(o + ld);
+            s += A[SW2 * pl + o] * X(o - ld - 1);
+            s += A[SW2 * pl + o + ld + 1] * X(o + ld + 1);
+            s += A[NW2 * pl + o] * X(o + ld - 1);
+            s += A[NW2 * pl + o - ld + 1] * X(o - ld + 1);
+            v = bv - s;
         }
+        P.r[o * R + rh] = (float)v;
+        acc += v * v;
+        if (bb) accb += bv * bv;
     }
     const double t1 = block_sum_r(acc, red);
     const double t2 = bb ? block_sum_r(accb, red) : 0.0;
-    double* base = partials + (long long)pi * gridDim.x * 2 * R;
-    double* part = base + (long long)blockIdx.x * 2 * R;
+    double* base = partials + P.res_part * 2 * R;
+    double* part = base + (long long)it.tile * 2 * R;
     if (threadIdx.x < R) {
         part[2 * threadIdx.x] = t1;
         part[2 * threadIdx.x + 1] = t2;
@@ -606,6 +605,8 @@ struct Batch {
     std::vector<SpItem> sp_h;
     SpItem* sp_d = nullptr;
     int sp_h_rows = 0;
+    std::vector<SpItem> row_h;
+    SpItem* row_d = nullptr;
     TailArgs* targs = nullptr;
     size_t tail_smem = 0;
     SysState* sys = nullptr;            // device, count * R
@@ -615,7 +616,7 @@ struct Batch {
     unsigned* counters = nullptr;       // count (finest up) + count (product) + count (residual)
     double* part_up = nullptr;          // finest up kernel partials
     double* part_sp = nullptr;          // operator product partials
-    double* part_res = nullptr;         // residual partials (count * the largest problem's blocks * 2R)
+    double* part_res = nullptr;         // residual partials (2R a row)
     double* stage = nullptr;            // host staging (largest n^2 * R doubles)
     PackEnt* ptab = nullptr;            // device: 3 * count pack/unpack entries
     PackEnt* ptab_h = nullptr;          // pinned mirror
@@ -629,12 +630,6 @@ struct Batch {
 };
 
 namespace {
-
-int max_res_blocks(const Batch& B) {
-    int m = 1;
-    for (const BProbDev& P : B.prob_h) m = std::max(m, res_blocks(P.n));
-    return m;
-}
 
 // Walks the workspace layout; with base == nullptr it only measures.
 size_t carve_batch(Batch& B, char* base) {
@@ -682,13 +677,14 @@ size_t carve_batch(Batch& B, char* base) {
     }
     B.prob_d = (BProbDev*)take(sizeof(BProbDev) * B.count);
     B.sp_d = (SpItem*)take(sizeof(SpItem) * B.sp_h.size());
+    B.row_d = (SpItem*)take(sizeof(SpItem) * B.row_h.size());
     B.targs = (TailArgs*)take(sizeof(TailArgs) * B.count);
     B.sys = (SysState*)take(sizeof(SysState) * B.count * R);
     B.st = (KState*)take(sizeof(KState));
     B.counters = (unsigned*)take(sizeof(unsigned) * 3 * B.count);
     B.part_up = (double*)take(sizeof(double) * 2 * R * (parts_up > 0 ? parts_up : 1));
     B.part_sp = (double*)take(sizeof(double) * R * (parts_sp > 0 ? parts_sp : 1));
-    B.part_res = (double*)take(sizeof(double) * 2 * R * max_res_blocks(B) * B.count);
+    B.part_res = (double*)take(sizeof(double) * 2 * R * B.row_h.size());
     B.stage = (double*)take(sizeof(double) * B.stage_elems);
     B.ptab = (PackEnt*)take(sizeof(PackEnt) * 3 * B.count);
     return a256(off);
@@ -889,8 +885,8 @@ bmg_status run_iteration(Batch& B, int parity) {
 }
 
 bmg_status residual(Batch& B, bool bb) {
-    k_bresidual<<<dim3(max_res_blocks(B), B.count), kBThreads, 0, B.stream>>>(B.prob_d, B.sys, B.part_res,
-                                                                       B.counters + 2 * B.count, bb ? 1 : 0);
+    k_bresidual<<<(int)B.row_h.size(), kBThreads, 0, B.stream>>>(B.prob_d, B.row_d, B.sys, B.part_res,
+                                                                 B.counters + 2 * B.count, bb ? 1 : 0);
     B.launches++;
     BMG_CUDA(cudaGetLastError());
     return BMG_OK;
@@ -990,7 +986,7 @@ bmg_status batch_build(int count, Ctx* const* ctxs, int flags, bool sizing, bool
         }
         K.tiles_x = cdiv(K.nc - 1, K.wc);   // rows per tile are modelled at attach
     }
-    // per problem: the operator-product tiles and the staging size
+    // per problem: the operator-product tiles, the residual's rows and the staging size
     int H = 32;
     B->sp_h_rows = H;
     for (int p = 0; p < count; p++) {
@@ -1004,6 +1000,8 @@ bmg_status batch_build(int count, Ctx* const* ctxs, int flags, bool sizing, bool
         P.sp_tiles_x = cdiv(m, kBThreads);
         P.sp_tiles = P.sp_tiles_x * cdiv(m, H);
         for (int t = 0; t < P.sp_tiles; t++) B->sp_h.push_back(SpItem{p, t});
+        P.res_part = (long long)B->row_h.size();
+        for (int t = 0; t < m; t++) B->row_h.push_back(SpItem{p, t});
         B->stage_elems = std::max<long long>(B->stage_elems, (long long)P.n * P.n * R);
     }
     B->ws_need = carve_batch(*B, nullptr);
@@ -1082,6 +1080,8 @@ bmg_status batch_attach(Batch& B, void* ws, size_t bytes, void* stream) {
     BMG_CUDA(cudaMemcpyAsync(B.prob_d, B.prob_h.data(), sizeof(BProbDev) * B.count, cudaMemcpyHostToDevice,
                              B.stream));
     BMG_CUDA(cudaMemcpyAsync(B.sp_d, B.sp_h.data(), sizeof(SpItem) * B.sp_h.size(), cudaMemcpyHostToDevice,
+                             B.stream));
+    BMG_CUDA(cudaMemcpyAsync(B.row_d, B.row_h.data(), sizeof(SpItem) * B.row_h.size(), cudaMemcpyHostToDevice,
                              B.stream));
     // tails: each problem's tail reads the tail class's right-hand side and
     // writes its final iterate there (the up kernels of n = 65 read it)
