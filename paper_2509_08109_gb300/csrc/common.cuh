@@ -50,7 +50,6 @@ struct KState {
     double rr;        // ||r||^2 (last reduction)
     double rz;        // r.z of the previous iteration
     double rzn;       // r.z of the first iteration of the current inner run (refinement mode)
-    double rzo;       // r.z_old (flexible CG)
     double pq;        // p.Aq
     double alpha, beta;
     double alpha0;    // refinement mode: step of the last even iteration, not yet in x
@@ -450,7 +449,7 @@ bmg_status tail3_pack(Ctx& c);
 // sums fit the partials)
 bool vcycle_forms_beta(const Ctx& c);
 template <typename T>
-bmg_status vcycle3d_impl(Ctx& c, const T* b0, T* x0, T* xout);
+bmg_status vcycle3d_impl(Ctx& c, const T* b0, T* x0);
 bmg_status fused_prepare(Ctx& c);
 bmg_status fused_configure(Ctx& c, int l, int wc, int hc, int hc_up);
 bmg_status fused_autotune(Ctx& c, int reps, double* best_ms_total);

@@ -27,81 +27,35 @@ __device__ __forceinline__ long long d3(int t, int ld, int n) {
     return (long long)(t % 3 - 1) + (long long)ld * (((t / 3) % 3 - 1) + (long long)n * (t / 9 - 1));
 }
 
-// sum_j a_ij x_j of row o (symmetric-half storage)
-template <int DIM, typename T>
-__device__ __forceinline__ T apply_row(const T* __restrict__ A, long long pl, int ld, int n, const T* x,
-                                       long long o) {
-    if (DIM == 2) {
-        T s = A[C2 * pl + o] * x[o];
-        s += A[W2 * pl + o] * x[o - 1];
-        s += A[W2 * pl + o + 1] * x[o + 1];
-        s += A[S2 * pl + o] * x[o - ld];
-        s += A[S2 * pl + o + ld] * x[o + ld];
-        s += A[SW2 * pl + o] * x[o - ld - 1];
-        s += A[SW2 * pl + o + ld + 1] * x[o + ld + 1];
-        s += A[NW2 * pl + o] * x[o + ld - 1];
-        s += A[NW2 * pl + o - ld + 1] * x[o - ld + 1];
-        return s;
-    } else {
-        T s = A[13 * pl + o] * x[o];
-#pragma unroll
-        for (int t = 0; t < 13; t++) {
-            const long long d = d3(t, ld, n);
-            s += A[(long long)t * pl + o] * x[o + d];
-            s += A[(long long)t * pl + o - d] * x[o - d];
-        }
-        return s;
-    }
+// sum_j a_ij x_j of row o (2-D, symmetric-half storage)
+__device__ __forceinline__ double apply_row(const double* __restrict__ A, long long pl, int ld, const double* x,
+                                            long long o) {
+    double s = A[C2 * pl + o] * x[o];
+    s += A[W2 * pl + o] * x[o - 1];
+    s += A[W2 * pl + o + 1] * x[o + 1];
+    s += A[S2 * pl + o] * x[o - ld];
+    s += A[S2 * pl + o + ld] * x[o + ld];
+    s += A[SW2 * pl + o] * x[o - ld - 1];
+    s += A[SW2 * pl + o + ld + 1] * x[o + ld + 1];
+    s += A[NW2 * pl + o] * x[o + ld - 1];
+    s += A[NW2 * pl + o - ld + 1] * x[o - ld + 1];
+    return s;
 }
 
-// True when every x_j row o couples to is +-0 (bit test, no FP64 op): then
-// (A x)_o is zero and the FP64 products can be skipped, e.g. for a zero
+// True when every x_j row o (2-D) couples to is +-0 (bit test, no FP64 op):
+// then (A x)_o is zero and the FP64 products can be skipped, e.g. for a zero
 // initial guess, where the residual is b itself.
-template <int DIM, typename T>
-__device__ __forceinline__ bool row_x_zero(const T* x, int ld, int n, long long o) {
-    auto bits = [](T v) -> unsigned long long {
-        return sizeof(T) == 8 ? (unsigned long long)__double_as_longlong((double)v) << 1
-                              : (unsigned long long)__float_as_uint((float)v) << 1;
-    };
+__device__ __forceinline__ bool row_x_zero(const double* x, int ld, long long o) {
+    auto bits = [](double v) { return (unsigned long long)__double_as_longlong(v) << 1; };
     unsigned long long m = 0;
     // row by row and not unrolled: holding the neighbourhood in registers for
     // the products that follow costs more occupancy than reading it again
-    const int rows = DIM == 2 ? 3 : 9;
 #pragma unroll 1
-    for (int q = 0; q < rows && m == 0; q++) {
-        const T* r = x + o + (long long)ld * ((q % 3 - 1) + (DIM == 2 ? 0LL : (long long)n * (q / 3 - 1)));
+    for (int q = -1; q <= 1 && m == 0; q++) {
+        const double* r = x + o + (long long)ld * q;
         m = bits(r[-1]) | bits(r[0]) | bits(r[1]);
     }
     return m == 0;
-}
-
-// (A x)_i in difference form: s_i x_i + sum_{j != i} a_ij (x_j - x_i), with
-// the row sums s_i computed in FP64.  The operator's rows nearly sum to zero,
-// so the plain FP32 product loses the smooth part of A x to cancellation; the
-// differences keep FP32 relative accuracy on every mode.
-template <int DIM>
-__device__ __forceinline__ float apply_row_diff(const float* __restrict__ A, const float* __restrict__ rs, long long pl,
-                                                int ld, int n, const float* x, long long o) {
-    const float xo = x[o];
-    float s = rs[o] * xo;
-    if (DIM == 2) {
-        s += A[W2 * pl + o] * (x[o - 1] - xo);
-        s += A[W2 * pl + o + 1] * (x[o + 1] - xo);
-        s += A[S2 * pl + o] * (x[o - ld] - xo);
-        s += A[S2 * pl + o + ld] * (x[o + ld] - xo);
-        s += A[SW2 * pl + o] * (x[o - ld - 1] - xo);
-        s += A[SW2 * pl + o + ld + 1] * (x[o + ld + 1] - xo);
-        s += A[NW2 * pl + o] * (x[o + ld - 1] - xo);
-        s += A[NW2 * pl + o - ld + 1] * (x[o - ld + 1] - xo);
-    } else {
-#pragma unroll
-        for (int t = 0; t < 13; t++) {
-            const long long d = d3(t, ld, n);
-            s += A[(long long)t * pl + o] * (x[o + d] - xo);
-            s += A[(long long)t * pl + o - d] * (x[o - d] - xo);
-        }
-    }
-    return s;
 }
 
 // Row sums s_i = sum_j a_ij of the FP64 operator (all stored couplings).
@@ -169,7 +123,7 @@ struct NodeTiles {
                 const int j = j0 + 8 * s;
                 if (j > n - 2) break;
                 const long long k = (long long)j * ld + i;
-                f(k, SKIP && row_x_zero<2, double>(x, ld, n, k) ? 0.0 : apply_row<2, double>(A, pl, ld, n, x, k));
+                f(k, SKIP && row_x_zero(x, ld, k) ? 0.0 : apply_row(A, pl, ld, x, k));
             }
         } else {
             const int i = 64 * (t % ti) + 2 * lane, j = 1 + 8 * (t / ti % tj) + row;
@@ -184,7 +138,7 @@ struct NodeTiles {
             }
         }
     }
-    // rows o and o + 1 of A x (3-D), in the order of apply_row
+    // rows o and o + 1 of A x (3-D): the diagonal, then each offset and its mirror
     template <bool SKIP>
     __device__ __forceinline__ void apply_pair(const double* __restrict__ A, long long pl, const double* x,
                                                int i, long long o, double& s0, double& s1) const {
@@ -416,54 +370,6 @@ __global__ void k_row_sums32_t(RowGrid<DIM> g, const double* __restrict__ A, lon
         double v = 0.0;
         if (g.row_inner(r_) && i_ >= 1 && i_ <= g.n - 2) v = row_sum<DIM>(A, pl, g.ld, g.n, k);
         rs[k] = (float)v;
-    }
-}
-
-// p = z + beta p_old, then q = A p (difference form), alpha = rz / p.q, in one
-// pass: each row forms p at its nine (27) neighbours on the fly from z and
-// p_old, so p is written to a second buffer (p_old is still being read).
-template <int DIM>
-__global__ void k_pspmv32_t(RowGrid<DIM> g, const float* __restrict__ A, const float* __restrict__ rs, long long pl,
-                            const float* z, const float* pold, float* __restrict__ p,
-                            float* __restrict__ q, double* partials, KState* st, int parity) {
-    pdl_wait();
-    pdl_trigger();
-    const float beta = (float)st->beta;
-    Acc32 acc;
-    FOR_ROWS(g) {
-        const long long k = (long long)r_ * g.ld + i_;
-        float pv = 0.0f, v = 0.0f;
-        if (g.row_inner(r_) && i_ >= 1 && i_ <= g.n - 2) {
-            auto P = [&](long long o) { return z[o] + beta * pold[o]; };
-            pv = P(k);
-            float s = rs[k] * pv;
-            if (DIM == 2) {
-                const int ld = g.ld;
-                s += A[W2 * pl + k] * (P(k - 1) - pv);
-                s += A[W2 * pl + k + 1] * (P(k + 1) - pv);
-                s += A[S2 * pl + k] * (P(k - ld) - pv);
-                s += A[S2 * pl + k + ld] * (P(k + ld) - pv);
-                s += A[SW2 * pl + k] * (P(k - ld - 1) - pv);
-                s += A[SW2 * pl + k + ld + 1] * (P(k + ld + 1) - pv);
-                s += A[NW2 * pl + k] * (P(k + ld - 1) - pv);
-                s += A[NW2 * pl + k - ld + 1] * (P(k - ld + 1) - pv);
-            } else {
-#pragma unroll
-                for (int t = 0; t < 13; t++) {
-                    const long long d = d3(t, g.ld, g.n);
-                    s += A[(long long)t * pl + k] * (P(k + d) - pv);
-                    s += A[(long long)t * pl + k - d] * (P(k - d) - pv);
-                }
-            }
-            v = s;
-        }
-        p[k] = pv;
-        q[k] = v;
-        acc.add(pv * v);
-    }
-    double t;
-    if (grid_sum(acc.value(), partials, &st->counter[2], &t)) {
-        set_alpha32(st, t, parity);
     }
 }
 
@@ -715,7 +621,14 @@ bmg_status k_residual_to32(Ctx& c) {
     return BMG_OK;
 }
 
-// 2-D form of k_pspmv32_t: a warp owns a strip of 64 columns and a band of H
+// p = z + beta p_old, q = A p and alpha = r.z / p.q in one pass; p goes to a
+// second buffer, since p_old is still being read.  The product is in difference
+// form, s_i p_i + sum_{j != i} a_ij (p_j - p_i), with the row sums s_i formed in
+// FP64: the operator's rows nearly sum to zero, so the plain FP32 product loses
+// the smooth part of A p to cancellation, and the differences keep FP32
+// relative accuracy on every mode.
+//
+// 2-D: a warp owns a strip of 64 columns and a band of H
 // rows and marches up the rows on its own, without barriers.  A lane holds the
 // column pair (i, i + 1), i even, of the three rows in play in registers (p and
 // the planes' values, loaded two wide); its neighbours' columns come by
@@ -725,7 +638,7 @@ bmg_status k_residual_to32(Ctx& c) {
 // on small ones.  4097^2: 103 us, 65^2: 7 us, against 129 and 8.1 us for a
 // thread per column, a block barrier per row and the planes in shared memory;
 // with two CTAs an SM instead of three (92 registers a thread for 80) 120 us.
-// Same arithmetic, in the same order, as k_pspmv32_t<2>.
+// A node's terms are summed in the order W, E, S, N, SW, NE, NW, SE.
 __global__ void __launch_bounds__(kThreads, 3) k_pspmv2d_strips(int n, int ld, long long pl, int H, int strips, int bands,
                                                              const float* __restrict__ A,
                                                              const float* __restrict__ rs, const float* z,
@@ -871,7 +784,7 @@ bmg_status k_rz_beta32(Ctx& c, const float* z, const float* zo) {
     return BMG_OK;
 }
 
-// 3-D form of k_pspmv32_t: one CTA per tile of 64 columns x 8 rows and a band
+// The same in 3-D: one CTA per tile of 64 columns x 8 rows and a band
 // of k-planes, marching up k; p of the next plane, with a halo of one row and
 // one column pair, goes from registers (loaded a step ahead) into a shared
 // ring of 4 slots, so one barrier per plane suffices.
@@ -881,8 +794,8 @@ bmg_status k_rz_beta32(Ctx& c, const float* z, const float* zo) {
 // straight from global memory, issued before the step's barrier so that they
 // overlap the wait; the mirrors are other threads' own values, served by L1
 // and L2.  HBM bounds the kernel (72 bytes a node).  257^3: 214 us, against
-// 252 us with a thread per node and one-wide loads.  Same products in the same
-// order as k_pspmv32_t<3>.
+// 252 us with a thread per node and one-wide loads.  A node's terms are
+// summed by offset, each followed by its mirror.
 constexpr int kP3I = 64, kP3J = 8;
 constexpr int kP3Pairs = kP3I / 2 + 2, kP3W = 2 * kP3Pairs, kP3H = kP3J + 2;   // halo tile: pairs a row, columns, rows
 constexpr int kP3A = kP3W * kP3H;
@@ -1043,22 +956,19 @@ bmg_status pspmv_prepare(Ctx& c) {
 
 bmg_status k_pspmv32(Ctx& c, const float* z, int parity) {
     const Level& L = c.lev[0];
+    if (c.spmv_h < 1) return BMG_ERR_STATE;   // pspmv_prepare has not run
     prof_begin(c, BMG_PROF_SPMV, 0);
-    if (c.dim == 2 && c.spmv_h > 0) {
+    if (c.dim == 2) {
         BMG_CUDA(launch_pdl(k_pspmv2d_strips, dim3(c.spmv_tiles), dim3(kThreads), 0, c.stream, L.n, L.ld, L.plane,
                             c.spmv_h, c.spmv_tiles_x, cdiv(L.n - 2, c.spmv_h), L.A32, c.rs32, z, c.p32s[parity ^ 1],
                             c.p32s[parity], c.q32, c.partials, c.st, parity));
-        c.launches++;
-    } else if (c.dim == 3 && c.spmv_h > 0) {
+    } else {
         const int tj = cdiv(L.n - 2, kP3J);
         BMG_CUDA(launch_pdl(k_pspmv3d_direct, dim3(c.spmv_tiles), dim3(kThreads), 0, c.stream, L.n, L.ld, L.plane,
                             c.spmv_h, c.spmv_tiles_x, tj, L.A32, c.rs32, z, c.p32s[parity ^ 1], c.p32s[parity], c.q32,
                             c.partials, c.st, parity));
-        c.launches++;
-    } else {
-        DISPATCH_DIM(c, k_pspmv32_t, L.A32, c.rs32, L.plane, z, c.p32s[parity ^ 1], c.p32s[parity], c.q32,
-                     c.partials, c.st, parity);
     }
+    c.launches++;
     prof_end(c, BMG_PROF_SPMV, 0, (c.ns + 4) * 4.0 * dofs0(c));
     BMG_CUDA(cudaGetLastError());
     return BMG_OK;

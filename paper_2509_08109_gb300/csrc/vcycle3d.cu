@@ -203,12 +203,10 @@ __global__ void __launch_bounds__(64) k_residual3d_sweep(L3<T> L, const T* x, T*
 // direction where d = -1), in the plane of f's parity mask m and of the
 // corner K - owner.  All of that is fixed by d, so the loop unrolls to plain
 // loads.
-// ldv: row length of the coarse vector bc (ldc, that of the weight planes,
-// unless the coarse level lives in another layout).
 template <typename T>
 __device__ __forceinline__ void restrict_node3d(int nf, int ldf, const T* r, const T* __restrict__ P,
-                                                int nc, int ldc, long long plc, T* __restrict__ bc, int ldv, int I,
-                                                int J, int K) {
+                                                int nc, int ldc, long long plc, T* __restrict__ bc, int I, int J,
+                                                int K) {
     const long long oc = (long long)I + (long long)ldc * (J + (long long)nc * K);
     const long long of = 2LL * I + (long long)ldf * (2 * J + (long long)nf * 2 * K);
     T s = 0;
@@ -224,7 +222,7 @@ __device__ __forceinline__ void restrict_node3d(int nf, int ldf, const T* r, con
         }
         s += w * r[of + dx + (long long)ldf * (dy + (long long)nf * dz)];
     }
-    bc[(long long)I + (long long)ldv * (J + (long long)nc * K)] = s;
+    bc[oc] = s;
 }
 
 template <typename T>
@@ -235,7 +233,7 @@ __global__ void k_restrict3d(int nf, int ldf, const T* r, const T* __restrict__ 
     const int I = blockIdx.x * blockDim.x + threadIdx.x;
     const int J = blockIdx.y, K = blockIdx.z;
     if (I < 1 || J < 1 || K < 1 || I > nc - 2 || J > nc - 2 || K > nc - 2) return;
-    restrict_node3d<T>(nf, ldf, r, P, nc, ldc, plc, bc, ldc, I, J, K);
+    restrict_node3d<T>(nf, ldf, r, P, nc, ldc, plc, bc, I, J, K);
 }
 
 // x_f += sum over s subset of m of P(f, (I,J,K) + s) x_c((I,J,K) + s) for the
@@ -243,17 +241,15 @@ __global__ void k_restrict3d(int nf, int ldf, const T* r, const T* __restrict__ 
 // (I,J,K) owns: one thread per coarse node, the 26 weights of its cell read
 // once and contiguously across the warp.  Summation over s ascending, as the
 // weights' own numbering.
-// ldv: row length of the coarse vector xc (as in restrict_node3d).
 template <typename T>
 __device__ __forceinline__ void prolong_node3d(int nf, int ldf, T* __restrict__ x, const T* __restrict__ P, int nc,
-                                               int ldc, long long plc, const T* xc, int ldv, int I,
-                                               int J, int K) {
+                                               int ldc, long long plc, const T* xc, int I, int J,
+                                               int K) {
     const long long oc = (long long)I + (long long)ldc * (J + (long long)nc * K);
-    const long long ov = (long long)I + (long long)ldv * (J + (long long)nc * K);
-    const long long sy = ldv, sz = (long long)ldv * nc;
+    const long long sy = ldc, sz = (long long)ldc * nc;
     T c8[8];
 #pragma unroll
-    for (int q = 0; q < 8; q++) c8[q] = xc[ov + (q & 1) + sy * ((q >> 1) & 1) + sz * (q >> 2)];
+    for (int q = 0; q < 8; q++) c8[q] = xc[oc + (q & 1) + sy * ((q >> 1) & 1) + sz * (q >> 2)];
 #pragma unroll
     for (int b = 0; b < 8; b++) {
         const int fi = 2 * I + (b & 1), fj = 2 * J + ((b >> 1) & 1), fk = 2 * K + (b >> 2);
@@ -276,13 +272,7 @@ __global__ void k_prolong3d(int nf, int ldf, T* __restrict__ x, const T* __restr
     const int I = blockIdx.x * blockDim.x + threadIdx.x;
     const int J = blockIdx.y, K = blockIdx.z;
     if (I > nc - 2 || J > nc - 2 || K > nc - 2) return;
-    prolong_node3d<T>(nf, ldf, x, P, nc, ldc, plc, xc, ldc, I, J, K);
-}
-
-template <typename T>
-__global__ void k_coarsest3d(L3<T> L, const double* __restrict__ A64, const T* __restrict__ b, T* __restrict__ x) {
-    const long long o = L.idx(1, 1, 1);
-    x[o] = (T)((double)b[o] / A64[13 * L.pl + o]);
+    prolong_node3d<T>(nf, ldf, x, P, nc, ldc, plc, xc, I, J, K);
 }
 
 inline dim3 g3(int ni, int nj, int nk) { return dim3(cdiv(ni, 64), nj, nk); }
@@ -1030,7 +1020,7 @@ bmg_status hs3_up(Ctx& c, int l, const T* f, T* x, const T* xc) {
 }
 
 template <typename T>
-bmg_status vcycle3d_impl(Ctx& c, const T* b0, T* x0, T* xout) {
+bmg_status vcycle3d_impl(Ctx& c, const T* b0, T* x0) {
     cudaStream_t s = c.stream;
     const int L = c.nlev;
     const double sz = sizeof(T);
@@ -1095,7 +1085,6 @@ bmg_status vcycle3d_impl(Ctx& c, const T* b0, T* x0, T* xout) {
         for (int col = 7; col >= 0; col--) BMG_TRY(colour_sweep<T>(c, l, v, bl(l), xl(l), col, h));
         c.launches += 1;   // prolongation
     }
-    (void)xout;
     BMG_CUDA(cudaGetLastError());
     return BMG_OK;
 }
@@ -1128,7 +1117,7 @@ bmg_status tail3_pack(Ctx& c) {
     return c.opts.precision == BMG_PREC_FP32 ? tail3_pack_impl<float>(c) : tail3_pack_impl<double>(c);
 }
 
-template bmg_status vcycle3d_impl<double>(Ctx&, const double*, double*, double*);
-template bmg_status vcycle3d_impl<float>(Ctx&, const float*, float*, float*);
+template bmg_status vcycle3d_impl<double>(Ctx&, const double*, double*);
+template bmg_status vcycle3d_impl<float>(Ctx&, const float*, float*);
 
 }  // namespace bmg
