@@ -24,7 +24,8 @@
 // systems iterate in lockstep; between refinements the host reads every
 // system's FP64 residual, retires the converged ones, and gives every
 // active system its own number of inner iterations for the next run (the
-// single-problem rule); the run lasts as long as the largest, and a system
+// count that a single solve's run starts with; a first run does not go on
+// beyond it here); the run lasts as long as the largest, and a system
 // whose count is used up, or whose r.z has fallen by the run's goal, freezes
 // (no further updates) until the next refinement.  A problem whose systems
 // are all frozen is skipped by every batched kernel of the iteration.
@@ -1313,12 +1314,8 @@ bmg_status batch_solve(Batch& B, int nrhs, const double* const* b, double* const
                 status[s] = BMG_ERR_NOT_CONVERGED;
                 continue;
             }
-            double want = sqrt(lim / rr[s]);
-            if (want < 1e-6) want = 1e-6;
-            int m = (int)ceil(log(want) / log(rho[s])) + 1;
-            if (m < 2) m = 2;
-            if (m > kMaxInner) m = kMaxInner;
-            if (m > maxit - it[s]) m = maxit - it[s];
+            const double want = std::max(sqrt(lim / rr[s]), kRefineFloor);
+            const int m = refine_start(want, rho[s], maxit - it[s]);
             m_of[s] = m;
             want_of[s] = want;
             m_need = std::max(m_need, m);
@@ -1349,11 +1346,7 @@ bmg_status batch_solve(Batch& B, int nrhs, const double* const* b, double* const
             it[s] += m;
             refs[s]++;
             const double nr = B.sys_h[s].rr;
-            const double red = sqrt(nr / rr[s]);
-            if (m > 0 && red > 0 && red < 1) {
-                const double r1 = pow(red, 1.0 / m);
-                if (r1 > 0.02 && r1 < 0.999) rho[s] = r1;
-            }
+            if (m > 0) rho[s] = refine_rho(rho[s], sqrt(nr / rr[s]), m);
             rr[s] = nr;
             lastm[s] = m;
         }

@@ -73,7 +73,7 @@ struct SysState {
     int first;        // 1: the next inner iteration takes p = z
     int active;       // 0: converged, zero right-hand side or out of iterations: no updates
     int left;         // inner iterations this system still takes in the current run (its own
-                      // count, as the single-problem refinement sizes it); at 0 it freezes
+                      // count, refine_start's); at 0 it freezes
     int taken;        // inner iterations it took in the current run
 };
 
@@ -469,7 +469,7 @@ bmg_status k_row_sums32(Ctx& c);                // rs32 = row sums of A (compute
 bmg_status k_residual_to32(Ctx& c);             // r32 = (float)(b - A x); rr; resets the inner CG state
 bmg_status k_rz_beta32(Ctx& c, const float* z, const float* zo);
 bmg_status k_update_dr32(Ctx& c, int parity);    // r32 -= alpha q; odd parity: x (FP64) += both iterations' alpha p
-// run lengths of the refinement mode (api.cu)
+// run lengths of the refinement mode, single, concurrent and batched (api.cu)
 constexpr double kRefineFloor = 1e-6;   // reduction one FP32 inner solve can deliver
 int refine_start(double want, double rho, int left);
 int refine_next(const KState& h, double want, double rho, int done, int left);
