@@ -444,7 +444,7 @@ bmg_status bmg_create(const bmg_opts* opts, bmg_ctx** out) {
     c.mrhs_bytes = c.opts.max_rhs > 1 ? batch_single_bytes(c) : 0;
     c.ws_need = carve(c, nullptr);
     const long long rows = ipow(c.lev[0].n, c.dim - 1);
-    c.red_blocks = (int)(rows > 152 * 8 ? 152 * 8 : rows);
+    c.red_blocks = (int)(rows > kChipSms * 8 ? kChipSms * 8 : rows);
     *out = ctx;
     return BMG_OK;
 }

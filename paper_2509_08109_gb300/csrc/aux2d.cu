@@ -41,7 +41,7 @@ using namespace bmg;
 namespace {
 
 constexpr int kAuxThreads = kThreads;     // 256, as block_sum expects
-constexpr int kRedBlocks = 4 * 152;       // fixed grid of the reducing kernels
+constexpr int kRedBlocks = 4 * kChipSms;  // fixed grid of the reducing kernels
 
 struct AuxState {
     double rr;          // ||f - A u||^2 (interior)

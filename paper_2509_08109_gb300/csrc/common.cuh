@@ -34,6 +34,7 @@ namespace bmg {
 
 constexpr int kMaxLevels = 20;
 constexpr int kThreads = 256;
+constexpr int kChipSms = 152;          // SMs of a GB300: grids whose size workspaces and results depend on
 constexpr int kMaxBlocks = 4096;       // partials buffer size for reductions (two sums per block)
 // refinement mode: most FP32 inner iterations between two FP64 residuals
 // (slowly converging problems, e.g. the 3-D shell, need hundreds per solve)
@@ -213,7 +214,7 @@ inline void prof_end(Ctx& c, int kind, int level, double bytes) {
 // where this grid leaves SMs idle: a large one's CTAs lose their places to
 // CTAs that wait (4097^2 solve 14.62 ms without triggers, 14.76 with; 65^2 1.00
 // and 0.96 ms; without the attribute 14.61 and 1.03 ms).
-constexpr unsigned kPdlGrid = 152;
+constexpr unsigned kPdlGrid = kChipSms;
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void pdl_trigger() {
     if (gridDim.x * gridDim.y * gridDim.z <= kPdlGrid) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");

@@ -437,7 +437,7 @@ __global__ void __launch_bounds__(kThreads) k_flush_x32(long long quads, double2
 }
 
 // r.z and r.z_old in one pass; the last block forms the flexible-CG beta.
-// Four values a load, two CTAs per SM (as the FP64 vector kernels).
+// Four values a load, four CTAs per SM (as the FP64 vector kernels).
 __global__ void __launch_bounds__(kThreads) k_rz_beta32_t(long long quads, const float4* r,
                                                           const float4* z,
                                                           const float4* zo, double* partials,

@@ -649,7 +649,7 @@ __global__ void k_tail3_pack(const T* __restrict__ A, int n, int ld, long long p
 // CTA does: 257 us against 196 for the 58-column tiles (169 since their
 // accesses are pairs and the first rows' stencils are fetched while the
 // iterates are staged).  The levels up to 65 take the slots that leave the
-// fewest row slots on the fullest of the 152 SMs (CTAs an SM, rounded up, times
+// fewest row slots on the fullest of the chip's 152 SMs (CTAs an SM, rounded up, times
 // S): at 65 five (eight tiles in 32 planes, two CTAs an SM), at 33 and below
 // three.  FP64, a reverse half sweep: 65^3 22.0 -> 16.3 us with five slots for
 // eight, 33^3 13.2 -> 11.1 and 17^3 12.9 -> 10.6 with three; 129^3 CG solve 6.48
