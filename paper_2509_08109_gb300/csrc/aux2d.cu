@@ -230,38 +230,56 @@ __global__ void k_inv(int nr, double* __restrict__ v) {
 // order, so the sum is the CSR row's, plus zero terms.
 //
 // s += term(value, x[column]) over the entries b, b + step, ... < e, in that
-// order.  Eight entries' values and columns are loaded before their gathers
-// (the bound is uniform over the warp), so a row waits for two memory
-// latencies per eight entries instead of two per entry.  Mesh of 423 x 632
-// vertices, flexible CG with the FP32 cycle: 4.04 -> 3.47 ms a solve together
-// with the fused conversions and the dependent launches below.
-template <typename V, typename X, typename F>
+// order.  D entries' values and columns are loaded before their gathers (the
+// bound is uniform over the warp), so a row waits for two memory latencies per
+// D entries instead of two per entry.
+//
+// Which D: eight take 56 to 64 registers in the kernels with a thread per row,
+// so an SM holds four blocks.  While that holds every row at once (kDeepRows),
+// a row's latency is the time.  Beyond it the other blocks hide the latency, and
+// the places that the registers cost count for more: four entries (32 registers
+// in FP32, 40 in the FP64 kernels of a fixed grid), one in the FP64 kernels with
+// a thread per row (32 registers; four take 48, or spill).  The order of the
+// sums, and so the result, is the same.  One solve, ms, on meshes of 60 x 80,
+// 250 x 350, 423 x 632 and 845 x 1262 vertices, all at eight and by the rule:
+//   stationary   5.8, 10.1, 13.5, 33.3   and 5.8, 10.1, 11.3, 29.7
+//   flexible CG  1.65, 2.38, 3.21, 6.94  and 1.66, 2.38, 3.10, 6.42
+// (one entry at a time everywhere, without the fused conversions and dependent
+// launches below: 6.7, 11.3, 13.4, 29.9 and 2.19, 2.92, 3.88, 7.01).
+constexpr int kDeep = 8, kFlat = 4;
+constexpr int kDeepRows = 4 * kChipSms * kAuxThreads;
+constexpr int row_depth(int D) { return D == kDeep ? kDeep : 1; }    // FP64, a thread per row
+#define BY_ROWS(kern, n) ((n) > kDeepRows ? kern<kFlat> : kern<kDeep>)
+constexpr int row_blocks(int D) { return D == kDeep ? 4 : 8; }       // their blocks an SM
+
+template <int D, typename V, typename X, typename F>
 __device__ __forceinline__ V sell_sum(int b, int e, int step, const int* __restrict__ ci, const V* __restrict__ va,
                                       const X* x, F&& term, V s = 0) {
-    for (int k = b; k < e; k += 8 * step) {
-        int c[8];
-        V v[8];
-        X g[8];
+    for (int k = b; k < e; k += D * step) {
+        int c[D];
+        V v[D];
+        X g[D];
 #pragma unroll
-        for (int u = 0; u < 8; u++)
+        for (int u = 0; u < D; u++)
             if (k + u * step < e) {
                 c[u] = ci[k + u * step];
                 v[u] = va[k + u * step];
             }
 #pragma unroll
-        for (int u = 0; u < 8; u++)
+        for (int u = 0; u < D; u++)
             if (k + u * step < e) g[u] = x[c[u]];
 #pragma unroll
-        for (int u = 0; u < 8; u++)
+        for (int u = 0; u < D; u++)
             if (k + u * step < e) s += term(v[u], g[u]);
     }
     return s;
 }
 
+template <int D>
 __device__ __forceinline__ double csr_row(const int* __restrict__ so, const int* __restrict__ ci,
                                           const double* __restrict__ va, const double* x, int i) {
     const int sl = i >> 5;
-    return sell_sum(so[sl] + (i & 31), so[sl + 1], 32, ci, va, x, [](double v, double g) { return v * g; });
+    return sell_sum<D>(so[sl] + (i & 31), so[sl + 1], 32, ci, va, x, [](double v, double g) { return v * g; });
 }
 
 // SELL values from CSR values: out[k] = src[map[k]], 0 for padding (map < 0)
@@ -284,16 +302,18 @@ __global__ void k_expand(int nv, const int* __restrict__ vid, const double* __re
 }
 
 // damped Jacobi: uo = u + omega D^-1 (f - A u)
-__global__ void k_jacobi(int nr, const int* __restrict__ rp, const int* __restrict__ ci, const double* __restrict__ va,
-                         const double* __restrict__ dinv, const double* f, const double* u,
-                         double* __restrict__ uo, double omega) {
+template <int D>
+__global__ void __launch_bounds__(kAuxThreads, row_blocks(D))
+    k_jacobi(int nr, const int* __restrict__ rp, const int* __restrict__ ci, const double* __restrict__ va,
+             const double* __restrict__ dinv, const double* f, const double* u, double* __restrict__ uo, double omega) {
     pdl_wait();
     pdl_trigger();
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < nr) uo[i] = u[i] + omega * dinv[i] * (f[i] - csr_row(rp, ci, va, u, i));
+    if (i < nr) uo[i] = u[i] + omega * dinv[i] * (f[i] - csr_row<row_depth(D)>(rp, ci, va, u, i));
 }
 
 // r = f - A u; with slot: *slot = ||r||^2 (deterministic grid reduction)
+template <int D>
 __global__ void k_residual_csr(int nr, const int* __restrict__ rp, const int* __restrict__ ci,
                                const double* __restrict__ va, const double* f,
                                const double* u, double* __restrict__ r, double* partials,
@@ -302,7 +322,7 @@ __global__ void k_residual_csr(int nr, const int* __restrict__ rp, const int* __
     pdl_trigger();
     double acc = 0.0;
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < nr; i += gridDim.x * blockDim.x) {
-        const double v = f[i] - csr_row(rp, ci, va, u, i);
+        const double v = f[i] - csr_row<D>(rp, ci, va, u, i);
         if (r) r[i] = v;
         acc += v * v;
     }
@@ -332,20 +352,21 @@ __global__ void k_restrict_ct(int nq, const int* __restrict__ rp, const int* __r
     if (w)
         for (int k = b; k < e; k += 32) s += va[k] * (y[ci[k]] * w[ci[k]]);
     else
-        s = sell_sum(b, e, 32, ci, va, y, [](double v, double g) { return v * g; });
+        s = sell_sum<kDeep>(b, e, 32, ci, va, y, [](double v, double g) { return v * g; });
     rc[map[q]] = s;
 }
 
 // prolongation: out[i] = (C z)_i * (w ? w[i] : 1), z in the padded coarse layout;
 // with u: u[i] += gamma * out[i] instead
-__global__ void k_prolong_c(int nr, const int* __restrict__ rp, const int* __restrict__ ci,
-                            const double* __restrict__ va, const double* z, const double* __restrict__ w,
-                            double* out, double* u, double gamma) {
+template <int D>
+__global__ void __launch_bounds__(kAuxThreads, row_blocks(D))
+    k_prolong_c(int nr, const int* __restrict__ rp, const int* __restrict__ ci, const double* __restrict__ va,
+                const double* z, const double* __restrict__ w, double* out, double* u, double gamma) {
     pdl_wait();
     pdl_trigger();
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= nr) return;
-    double s = csr_row(rp, ci, va, z, i);
+    double s = csr_row<row_depth(D)>(rp, ci, va, z, i);
     if (w) s *= w[i];
     if (u) u[i] += gamma * s;
     else out[i] = s;
@@ -367,11 +388,12 @@ __global__ void k_cg_init(int nr, const double* __restrict__ r, double* __restri
 }
 
 // q = M p; alpha = cg_rr / p.q (0 when p.q is not positive: r was zero)
+template <int D>
 __global__ void k_cg_mp(int nr, const int* __restrict__ rp, const int* __restrict__ ci, const double* __restrict__ va,
                         const double* __restrict__ p, double* __restrict__ q, double* partials, AuxState* st) {
     double acc = 0.0;
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < nr; i += gridDim.x * blockDim.x) {
-        const double v = csr_row(rp, ci, va, p, i);
+        const double v = csr_row<D>(rp, ci, va, p, i);
         q[i] = v;
         acc += p[i] * v;
     }
@@ -407,13 +429,14 @@ __global__ void k_cg_p(int nr, const double* __restrict__ res, double* __restric
 }
 
 // q = A p; alpha = rz / p.q (device-side, with a breakdown check)
+template <int D>
 __global__ void k_spmv_dot(int nr, const int* __restrict__ rp, const int* __restrict__ ci, const double* __restrict__ va,
                            const double* p, double* __restrict__ q, double* partials, AuxState* st) {
     pdl_wait();
     pdl_trigger();
     double acc = 0.0;
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < nr; i += gridDim.x * blockDim.x) {
-        const double v = csr_row(rp, ci, va, p, i);
+        const double v = csr_row<D>(rp, ci, va, p, i);
         q[i] = v;
         acc += p[i] * v;
     }
@@ -475,13 +498,14 @@ __global__ void k_p_update_aux(int nr, double* p, const double* z, const AuxStat
 // A_p products in difference form, rs_i u_i + sum_j a_ij (u_j - u_i) with
 // the row sums rs_i formed in FP64: a smooth u makes the plain FP32 product
 // lose A u to cancellation (the diagonal entry contributes a_ii * 0).
+template <int D>
 __device__ __forceinline__ float sell_diff32(const int* __restrict__ so, const int* __restrict__ ci,
                                             const float* __restrict__ va, const float* __restrict__ rs,
                                             const float* x, int i) {
     const int sl = i >> 5;
     const float xi = x[i];
-    return sell_sum(so[sl] + (i & 31), so[sl + 1], 32, ci, va, x, [xi](float v, float g) { return v * (g - xi); },
-                    rs[i] * xi);
+    return sell_sum<D>(so[sl] + (i & 31), so[sl + 1], 32, ci, va, x,
+                       [xi](float v, float g) { return v * (g - xi); }, rs[i] * xi);
 }
 
 // first sweep from the zero guess: f32 = (float)r, u = omega D^-1 f32
@@ -497,6 +521,7 @@ __global__ void k_jacobi32_first(int nr, const double* r, const float* __restric
 }
 
 // last sweep: z = u + omega D^-1 (f - A u), stored in FP64
+template <int D>
 __global__ void k_jacobi32_last(int nr, const int* __restrict__ so, const int* __restrict__ ci,
                                 const float* __restrict__ va, const float* __restrict__ rs,
                                 const float* __restrict__ dinv, const float* f,
@@ -505,17 +530,18 @@ __global__ void k_jacobi32_last(int nr, const int* __restrict__ so, const int* _
     pdl_trigger();
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= nr) return;
-    z[i] = (double)(u[i] + omega * dinv[i] * (f[i] - sell_diff32(so, ci, va, rs, u, i)));
+    z[i] = (double)(u[i] + omega * dinv[i] * (f[i] - sell_diff32<D>(so, ci, va, rs, u, i)));
 }
 
 // y = w (f - A u) (FP32, difference form): the residual with the lumped mass applied
+template <int D>
 __global__ void k_residual32(int nr, const int* __restrict__ so, const int* __restrict__ ci,
                              const float* __restrict__ va, const float* __restrict__ rs, const float* f,
                              const float* u, const float* __restrict__ w, float* __restrict__ y) {
     pdl_wait();
     pdl_trigger();
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < nr) y[i] = (f[i] - sell_diff32(so, ci, va, rs, u, i)) * w[i];
+    if (i < nr) y[i] = (f[i] - sell_diff32<D>(so, ci, va, rs, u, i)) * w[i];
 }
 
 // rc[map[q]] = sum_k C^T[q,k] y[col] (FP32 products, FP64 out for the coarse
@@ -533,7 +559,7 @@ __global__ void __launch_bounds__(32 * kCtWarps) k_restrict_ct32(int nq, const i
     pdl_wait();
     pdl_trigger();
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, q = 32 * blockIdx.x + lane;
-    part[w][lane] = sell_sum(so[blockIdx.x] + lane + 32 * w, so[blockIdx.x + 1], 32 * kCtWarps, ci, va, y,
+    part[w][lane] = sell_sum<kDeep>(so[blockIdx.x] + lane + 32 * w, so[blockIdx.x + 1], 32 * kCtWarps, ci, va, y,
                              [](float v, float g) { return v * g; });
     __syncthreads();
     if (w == 0 && q < nq) {
@@ -545,6 +571,7 @@ __global__ void __launch_bounds__(32 * kCtWarps) k_restrict_ct32(int nq, const i
 }
 
 // u += gamma w (C z), z the coarse correction (FP64, padded layout)
+template <int D>
 __global__ void k_prolong_c32(int nr, const int* __restrict__ so, const int* __restrict__ ci,
                               const float* __restrict__ va, const double* z, const float* __restrict__ w,
                               float* u, float gamma) {
@@ -553,7 +580,7 @@ __global__ void k_prolong_c32(int nr, const int* __restrict__ so, const int* __r
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= nr) return;
     const int sl = i >> 5;
-    const float s = sell_sum(so[sl] + (i & 31), so[sl + 1], 32, ci, va, z,
+    const float s = sell_sum<D>(so[sl] + (i & 31), so[sl + 1], 32, ci, va, z,
                              [](float v, double g) { return v * (float)g; });
     u[i] += gamma * (s * w[i]);
 }
@@ -581,7 +608,7 @@ __global__ void k_axpy(int nr, double* __restrict__ u, const double* __restrict_
 __global__ void k_spmv_csr(int nr, const int* __restrict__ rp, const int* __restrict__ ci,
                            const double* __restrict__ va, const double* __restrict__ x, double* __restrict__ y) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < nr) y[i] = csr_row(rp, ci, va, x, i);
+    if (i < nr) y[i] = csr_row<kDeep>(rp, ci, va, x, i);
 }
 
 // natural n x n grid vector <-> the coarse context's padded layout (interior only)
@@ -1136,9 +1163,10 @@ bmg_status mass_cg(bmg_aux& x, const double* r, double* y) {
     cudaStream_t s = x.coarse->c.stream;
     const int nr = x.nvi;
     k_cg_init<<<kRedBlocks, kAuxThreads, 0, s>>>(nr, r, y, x.d_cres, x.d_cp, x.d_partials, x.d_st_aux);
+    auto product = BY_ROWS(k_cg_mp, nr);
     for (int k = 0; k < x.opts.mass_steps; k++) {
         if (k > 0) k_cg_p<<<kRedBlocks, kAuxThreads, 0, s>>>(nr, x.d_cres, x.d_cp, x.d_st_aux);
-        k_cg_mp<<<kRedBlocks, kAuxThreads, 0, s>>>(nr, x.d_sam_off, x.d_sam_col, x.d_svm, x.d_cp, x.d_cq, x.d_partials,
+        product<<<kRedBlocks, kAuxThreads, 0, s>>>(nr, x.d_sam_off, x.d_sam_col, x.d_svm, x.d_cp, x.d_cq, x.d_partials,
                                                    x.d_st_aux);
         k_cg_update<<<kRedBlocks, kAuxThreads, 0, s>>>(nr, y, x.d_cres, x.d_cp, x.d_cq, x.d_partials, x.d_st_aux);
     }
@@ -1154,12 +1182,12 @@ bmg_status aux_cycle(bmg_aux& x, const double* f, double* u, double* u2) {
     const int nr = x.nvi, nq = (int)x.ct_map.size();
     const bool lumped = x.opts.mass_steps == 0;
     // 1. pre-relaxation
-    BMG_TRY(aux_launch(s, k_jacobi, blocks(nr), nr, x.d_sam_off, x.d_sam_col, x.d_sva, x.d_dinv, f, u, u2,
+    BMG_TRY(aux_launch(s, BY_ROWS(k_jacobi, nr), blocks(nr), nr, x.d_sam_off, x.d_sam_col, x.d_sva, x.d_dinv, f, u, u2,
                        x.opts.omega));
     std::swap(u, u2);
     // 2. restriction r_c = C^T M^-1 (f - A u)
-    BMG_TRY(aux_launch(s, k_residual_csr, red_blocks(nr), nr, x.d_sam_off, x.d_sam_col, x.d_sva, f, u, x.d_r,
-                       x.d_partials, &x.d_st_aux->counter[0], (double*)nullptr));
+    BMG_TRY(aux_launch(s, BY_ROWS(k_residual_csr, nr), red_blocks(nr), nr, x.d_sam_off, x.d_sam_col, x.d_sva, f, u,
+                       x.d_r, x.d_partials, &x.d_st_aux->counter[0], (double*)nullptr));
     const double* y = x.d_r;
     if (!lumped) {
         BMG_TRY(mass_cg(x, x.d_r, x.d_y));
@@ -1172,16 +1200,16 @@ bmg_status aux_cycle(bmg_aux& x, const double* f, double* u, double* u2) {
     BMG_TRY(vcycle(c, c.r, c.z[0]));
     // 4. prolongation u += gamma M^-1 C e_c
     if (lumped) {
-        BMG_TRY(aux_launch(s, k_prolong_c, blocks(nr), nr, x.d_sc_off, x.d_sc_col, x.d_svc, c.z[0], x.d_mlinv,
-                           (double*)nullptr, u, x.opts.gamma));
+        BMG_TRY(aux_launch(s, BY_ROWS(k_prolong_c, nr), blocks(nr), nr, x.d_sc_off, x.d_sc_col, x.d_svc, c.z[0],
+                           x.d_mlinv, (double*)nullptr, u, x.opts.gamma));
     } else {
-        k_prolong_c<<<blocks(nr), kAuxThreads, 0, s>>>(nr, x.d_sc_off, x.d_sc_col, x.d_svc, c.z[0], nullptr, x.d_w,
-                                                       nullptr, 0.0);
+        auto prolong = BY_ROWS(k_prolong_c, nr);
+        prolong<<<blocks(nr), kAuxThreads, 0, s>>>(nr, x.d_sc_off, x.d_sc_col, x.d_svc, c.z[0], nullptr, x.d_w, nullptr, 0.0);
         BMG_TRY(mass_cg(x, x.d_w, x.d_y));
         k_axpy<<<blocks(nr), kAuxThreads, 0, s>>>(nr, u, x.d_y, x.opts.gamma);
     }
     // 5. post-relaxation
-    BMG_TRY(aux_launch(s, k_jacobi, blocks(nr), nr, x.d_sam_off, x.d_sam_col, x.d_sva, x.d_dinv, f, u, u2,
+    BMG_TRY(aux_launch(s, BY_ROWS(k_jacobi, nr), blocks(nr), nr, x.d_sam_off, x.d_sam_col, x.d_sva, x.d_dinv, f, u, u2,
                        x.opts.omega));
     std::swap(u, u2);
     BMG_CUDA(cudaGetLastError());
@@ -1197,15 +1225,15 @@ bmg_status aux_precond32(bmg_aux& x, const double* r, double* z) {
     const int nr = x.nvi, nq = (int)x.ct_map.size();
     const float om = (float)x.opts.omega;
     BMG_TRY(aux_launch(s, k_jacobi32_first, blocks(nr), nr, r, x.d_dinv32, x.d_f32, x.d_u32, om));
-    BMG_TRY(aux_launch(s, k_residual32, blocks(nr), nr, x.d_sam_off, x.d_sam_col, x.d_sva32, x.d_rs32, x.d_f32, x.d_u32,
+    BMG_TRY(aux_launch(s, BY_ROWS(k_residual32, nr), blocks(nr), nr, x.d_sam_off, x.d_sam_col, x.d_sva32, x.d_rs32, x.d_f32, x.d_u32,
                        x.d_mlinv32, x.d_r32));
     // every interior node of c.r is written; its boundary is zero
     BMG_CUDA(launch_pdl(k_restrict_ct32, dim3(cdiv(nq, 32)), dim3(32 * kCtWarps), 0, s, nq, x.d_sct_off, x.d_sct_col,
                         x.d_svct32, x.d_ct_map, x.d_r32, c.r));
     BMG_TRY(vcycle(c, c.r, c.z[0]));
-    BMG_TRY(aux_launch(s, k_prolong_c32, blocks(nr), nr, x.d_sc_off, x.d_sc_col, x.d_svc32, c.z[0], x.d_mlinv32, x.d_u32,
+    BMG_TRY(aux_launch(s, BY_ROWS(k_prolong_c32, nr), blocks(nr), nr, x.d_sc_off, x.d_sc_col, x.d_svc32, c.z[0], x.d_mlinv32, x.d_u32,
                        (float)x.opts.gamma));
-    BMG_TRY(aux_launch(s, k_jacobi32_last, blocks(nr), nr, x.d_sam_off, x.d_sam_col, x.d_sva32, x.d_rs32, x.d_dinv32,
+    BMG_TRY(aux_launch(s, BY_ROWS(k_jacobi32_last, nr), blocks(nr), nr, x.d_sam_off, x.d_sam_col, x.d_sva32, x.d_rs32, x.d_dinv32,
                        x.d_f32, x.d_u32, z, om));
     BMG_CUDA(cudaGetLastError());
     return BMG_OK;
@@ -1229,7 +1257,7 @@ bmg_status fcg_body(bmg_aux& x, int par) {
     BMG_TRY(aux_precond(x, x.d_kr, zb[par]));
     BMG_TRY(aux_launch(s, k_dot2_aux, red_blocks(nr), nr, x.d_kr, zb[par], zb[par ^ 1], x.d_partials, dst, 0));
     BMG_TRY(aux_launch(s, k_p_update_aux, blocks(nr), nr, x.d_kp, zb[par], dst));
-    BMG_TRY(aux_launch(s, k_spmv_dot, red_blocks(nr), nr, x.d_sam_off, x.d_sam_col, x.d_sva, x.d_kp, x.d_kq, x.d_partials,
+    BMG_TRY(aux_launch(s, BY_ROWS(k_spmv_dot, nr), red_blocks(nr), nr, x.d_sam_off, x.d_sam_col, x.d_sva, x.d_kp, x.d_kq, x.d_partials,
                        dst));
     BMG_TRY(aux_launch(s, k_update_ur, red_blocks(nr), nr, x.d_u, x.d_kr, x.d_kp, x.d_kq, dst, x.d_partials,
                        &dst->counter[0], &dst->rr));
@@ -1240,9 +1268,10 @@ bmg_status fcg_body(bmg_aux& x, int par) {
 // one stationary iteration: a cycle, then ||f - A u||^2
 bmg_status stat_body(bmg_aux& x) {
     BMG_TRY(aux_cycle(x, x.d_f, x.d_u, x.d_u2));
-    k_residual_csr<<<kRedBlocks, kAuxThreads, 0, x.coarse->c.stream>>>(x.nvi, x.d_sam_off, x.d_sam_col, x.d_sva,
-                                                                       x.d_f, x.d_u, nullptr, x.d_partials,
-                                                                       &x.d_st_aux->counter[0], &x.d_st_aux->rr);
+    auto residual = BY_ROWS(k_residual_csr, x.nvi);
+    residual<<<kRedBlocks, kAuxThreads, 0, x.coarse->c.stream>>>(x.nvi, x.d_sam_off, x.d_sam_col, x.d_sva, x.d_f, x.d_u,
+                                                                 nullptr, x.d_partials, &x.d_st_aux->counter[0],
+                                                                 &x.d_st_aux->rr);
     BMG_CUDA(cudaGetLastError());
     return BMG_OK;
 }
@@ -1659,13 +1688,14 @@ extern "C" bmg_status bmg_aux_solve(bmg_aux* x, const double* f, double* u, doub
     Ctx& c = x->coarse->c;
     cudaStream_t s = c.stream;
     const int nr = x->nvi;
+    auto residual = BY_ROWS(k_residual_csr, nr);
     BMG_CUDA(cudaMemsetAsync(&x->d_st_aux->err, 0, sizeof(int), s));
     k_compress<<<blocks(nr), kAuxThreads, 0, s>>>(nr, x->d_vtx, f, x->d_f);
     k_compress<<<blocks(nr), kAuxThreads, 0, s>>>(nr, x->d_vtx, u, x->d_u);
     k_dot_aux<<<kRedBlocks, kAuxThreads, 0, s>>>(nr, x->d_f, x->d_f, x->d_partials, &x->d_st_aux->counter[0],
                                                  &x->d_st_aux->ff);
-    k_residual_csr<<<kRedBlocks, kAuxThreads, 0, s>>>(nr, x->d_sam_off, x->d_sam_col, x->d_sva, x->d_f, x->d_u, nullptr,
-                                                      x->d_partials, &x->d_st_aux->counter[0], &x->d_st_aux->rr);
+    residual<<<kRedBlocks, kAuxThreads, 0, s>>>(nr, x->d_sam_off, x->d_sam_col, x->d_sva, x->d_f, x->d_u, nullptr,
+                                                x->d_partials, &x->d_st_aux->counter[0], &x->d_st_aux->rr);
     BMG_CUDA(cudaGetLastError());
     AuxState h;
     BMG_TRY(aux_read(*x, h));
@@ -1689,14 +1719,15 @@ extern "C" bmg_status bmg_aux_solve(bmg_aux* x, const double* f, double* u, doub
         // iteration.  Iterations after the first replay a captured graph.
         const size_t vb = sizeof(double) * nr;
         AuxState* dst = x->d_st_aux;
-        k_residual_csr<<<kRedBlocks, kAuxThreads, 0, s>>>(nr, x->d_sam_off, x->d_sam_col, x->d_sva, x->d_f, x->d_u,
-                                                          x->d_kr, x->d_partials, cnt, &dst->rr);
+        residual<<<kRedBlocks, kAuxThreads, 0, s>>>(nr, x->d_sam_off, x->d_sam_col, x->d_sva, x->d_f, x->d_u,
+                                                    x->d_kr, x->d_partials, cnt, &dst->rr);
         BMG_TRY(aux_precond(*x, x->d_kr, x->d_kz));
         BMG_CUDA(cudaMemsetAsync(x->d_kzo, 0, vb, s));
         k_dot2_aux<<<kRedBlocks, kAuxThreads, 0, s>>>(nr, x->d_kr, x->d_kz, x->d_kzo, x->d_partials, dst, 1);
         BMG_CUDA(cudaMemcpyAsync(x->d_kp, x->d_kz, vb, cudaMemcpyDeviceToDevice, s));
-        k_spmv_dot<<<kRedBlocks, kAuxThreads, 0, s>>>(nr, x->d_sam_off, x->d_sam_col, x->d_sva, x->d_kp, x->d_kq,
-                                                      x->d_partials, dst);
+        auto product = BY_ROWS(k_spmv_dot, nr);
+        product<<<kRedBlocks, kAuxThreads, 0, s>>>(nr, x->d_sam_off, x->d_sam_col, x->d_sva, x->d_kp, x->d_kq,
+                                                   x->d_partials, dst);
         k_update_ur<<<kRedBlocks, kAuxThreads, 0, s>>>(nr, x->d_u, x->d_kr, x->d_kp, x->d_kq, dst, x->d_partials, cnt,
                                                        &dst->rr);
         BMG_CUDA(cudaGetLastError());
@@ -1709,8 +1740,8 @@ extern "C" bmg_status bmg_aux_solve(bmg_aux* x, const double* f, double* u, doub
             BMG_TRY(run_body(*x, it & 1));
         }
         // the recursive residual drifts from f - A u: report the true one
-        k_residual_csr<<<kRedBlocks, kAuxThreads, 0, s>>>(nr, x->d_sam_off, x->d_sam_col, x->d_sva, x->d_f, x->d_u,
-                                                          nullptr, x->d_partials, cnt, &x->d_st_aux->rr);
+        residual<<<kRedBlocks, kAuxThreads, 0, s>>>(nr, x->d_sam_off, x->d_sam_col, x->d_sva, x->d_f, x->d_u,
+                                                    nullptr, x->d_partials, cnt, &x->d_st_aux->rr);
         BMG_CUDA(cudaGetLastError());
         BMG_TRY(aux_read(*x, h));
         rel = sqrt(h.rr) / nf;
@@ -1760,8 +1791,9 @@ bmg_status apply_ptap(bmg_aux& x, const double* q, double* v) {
     const bool lumped = x.opts.mass_steps == 0;
     const dim3 gp(blocks(x.ld), x.n);
     k_to_padded<<<gp, kAuxThreads, 0, s>>>(x.n, x.ld, q, x.d_cpad);
-    k_prolong_c<<<blocks(nr), kAuxThreads, 0, s>>>(nr, x.d_sc_off, x.d_sc_col, x.d_svc, x.d_cpad,
-                                                   lumped ? x.d_mlinv : nullptr, x.d_w, nullptr, 0.0);
+    auto prolong = BY_ROWS(k_prolong_c, nr);
+    prolong<<<blocks(nr), kAuxThreads, 0, s>>>(nr, x.d_sc_off, x.d_sc_col, x.d_svc, x.d_cpad,
+                                               lumped ? x.d_mlinv : nullptr, x.d_w, nullptr, 0.0);
     const double* y = x.d_w;
     if (!lumped) {
         BMG_TRY(mass_cg(x, x.d_w, x.d_y));
