@@ -251,9 +251,11 @@ __global__ void k_bunpack_all(const BProbDev* __restrict__ probs, const PackEnt*
 // share of an SM's FP64 units for as long as its rows take, and few long blocks
 // leave the last ones running alone (16 problems of 65..1025 x 4, a solve's full
 // calls: 0.76 ms with eight rows a block, 0.64 with four, 0.62 with two, 0.555
-// with one).  A grid of the largest problem's rows for every problem, with
-// partials to match, costs an uneven batch blocks that only leave: one of 4097^2
-// beside 511 of 65^2 took 46.3 ms a solve and 132 MB more instead of 43.0.
+// with one; 512 problems x 4, whose blocks are many either way, 12.0 ms a call
+// against 11.2 with 32 blocks a problem).  A grid of the largest problem's rows
+// for every problem, with partials to match, costs an uneven batch blocks that
+// only leave: one of 4097^2 beside 511 of 65^2 took 46.3 ms a solve instead of
+// 43.0, and 132 MB more.
 __global__ void __launch_bounds__(kBThreads) k_bresidual(const BProbDev* __restrict__ probs,
                                                          const SpItem* __restrict__ items, SysState* sys,
                                                          double* partials, unsigned* counters, int bb) {
